@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "digits.cuh"
 #include "oddeven.cuh"
 #include "solver.cuh"
 
@@ -83,6 +84,9 @@ void free_op(coarse_op* op) {
   if (op->red) cudaFree(op->red);
   if (op->apply_scratch) cudaFree(op->apply_scratch);
   if (op->apply_cnt) cudaFree(op->apply_cnt);
+  if (op->dig) cudaFree(op->dig);
+  if (op->digscale) cudaFree(op->digscale);
+  if (op->digx) cudaFree(op->digx);
   delete op;
 }
 
@@ -113,6 +117,7 @@ int ingest(coarse_op* op, const void* self_b, const void* hop_b, uint32_t flags,
   TRY(launch_ingest((const double2*)self_b, (const double2*)hop_b, gamma5_only, op->V, op->n, op->nb,
                     op->blk[0].ptr, op->blk[1].ptr, op->blk[2].ptr, s));
   TRY(launch_pack_mrhs(op, s));
+  if (op->dig) TRY(launch_dig_blocks((const double2*)op->blk[0].ptr, op->V, op->n, op->dig, op->digscale, s));
   COARSE_CUDA(cudaStreamSynchronize(s));
   return COARSE_OK;
 }
@@ -165,11 +170,14 @@ int apply_impl(const coarse_op* op, const void* x, void* y, int nrhs, int precis
   if (nrhs > 1 && precision == COARSE_PREC_BF16) return launch_apply_mrhs_bf16(op, x, y, nrhs, adjoint, s);
   const size_t esz = precision == COARSE_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t col = esz * (size_t)op->V * op->n;
-  for (int c = 0; c < nrhs; ++c) {
+  const int pass = precision == COARSE_PREC_FP64 && op->dig ? kDigCols : 1;
+  for (int c = 0; c < nrhs; c += pass) {
     ApplyArgs a = make_apply_args(op, precision, (const char*)x + c * col, (char*)y + c * col);
     a.mu = adjoint ? -op->mu : op->mu;
     a.adjoint = adjoint;
-    TRY(launch_apply(precision, op->n, a, s));
+    const int nc = nrhs - c < pass ? nrhs - c : pass;
+    if (nc > 1) TRY(launch_apply_digits(op->n, a, nc, (long long)op->V * op->n, s));
+    else TRY(launch_apply(precision, op->n, a, s));
   }
   return COARSE_OK;
 }
@@ -351,6 +359,23 @@ int coarse_op_create(const coarse_op_desc* d, const void* self_blocks, const voi
   op->norms = op->red + 2 * 304;
   op->coef = (double2*)(op->norms + 8);
   op->counter = (unsigned*)(op->coef + 2);
+  {
+    // digit copy of the FP64 blocks, where it leaves most of the free memory to the solvers
+    const size_t db = dig_block_bytes(op->n, op->V);
+    const size_t xb = dig_x_bytes(op->n, op->V, op->max_nrhs < kDigCols ? op->max_nrhs : kDigCols);
+    size_t mfree = 0, mtotal = 0;
+    cudaMemGetInfo(&mfree, &mtotal);
+    if (db + xb <= mfree / 3 &&
+        (cudaMalloc(&op->dig, db) != cudaSuccess || cudaMalloc((void**)&op->digscale, dig_scale_bytes(op->V)) != cudaSuccess ||
+         cudaMalloc(&op->digx, xb) != cudaSuccess)) {
+      cudaGetLastError();
+      cudaFree(op->dig);
+      cudaFree(op->digscale);
+      op->dig = nullptr;
+      op->digscale = nullptr;
+      op->digx = nullptr;
+    }
+  }
   const double2 cst[2] = {make_double2(-1.0, 0.0), make_double2(1.0, 0.0)};
   if ((op->eo_sites &&
        (cudaMemcpyAsync(op->eo_sites, eo_sites.data(), eo_sites.size() * sizeof(int), cudaMemcpyHostToDevice, s) !=

@@ -20,6 +20,7 @@
 #include "common.cuh"
 #include "apply_core.cuh"
 #include "batch.cuh"
+#include "digits.cuh"
 #include "pipe.cuh"
 #include "tune.cuh"
 
@@ -439,7 +440,9 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
 int launch_apply(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
   if (a.V <= 0) return COARSE_OK;
   switch (prec) {
-    case COARSE_PREC_FP64: return launch_t<double2, double2, double2>(n, a, s);
+    case COARSE_PREC_FP64:
+      if (a.dig) return launch_apply_digits(n, a, 1, 0, s);
+      return launch_t<double2, double2, double2>(n, a, s);
     case COARSE_PREC_FP32: return launch_tuned<float2>(prec, n, a, s);
     case COARSE_PREC_BF16: return launch_tuned<cbf16>(prec, n, a, s);
   }

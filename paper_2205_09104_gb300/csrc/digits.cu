@@ -1,0 +1,550 @@
+// FP64 stencil y = D_c x by exact products of 8-bit digits on the tensor cores.
+//
+// GB300 runs FP64 fused multiply-adds at about 1.25 TFLOP/s, a sixtieth of its FP32 rate, so the FP64
+// stencil on the FP64 pipe is bound by that rate whatever the layout (16^4 sites, n = 48: 10.3 ms against
+// 1.8 ms of block traffic).  Here each block and each site vector is written once as 64-bit fixed-point
+// numbers with a common power-of-two scale, cut into eight signed 8-bit digits (radix 256, digits
+// -128 .. 127), and the products of digits are summed by mma.sync m16n8k16 (FP16 operands, FP32 sums):
+//   a = 2^(E-6) sum_p a_p 256^-p,  x = 2^(F-6) sum_q x_q 256^-q,  |a| < 2^E, |x| < 2^F for the whole
+//   block / site vector,  sum_j a_ij x_j = 2^(E+F-12) sum_s 256^-s L_s,  L_s = sum_{p+q=s} sum_j a_p x_q.
+// Every L_s is an integer below 2^23, so the FP32 sums are exact, and only two roundings are left: the
+// fixed-point conversions (2^-62 of the largest entry) and the levels s >= 8 that are dropped (2^-62 of
+// the product of the largest entries); the FP64 pipe adds up one number per block, row and part.
+// The products of one block row are therefore far more exact than an FP64 sum of n terms, as long as
+// the entries that matter lie within a few binary orders of their block's or site's largest one.
+// Where they may not (a row or column of a block, or a chirality half of a site vector, more than 2^8
+// below the largest; scales near the FP64 range's ends; infinities and NaN) the scale is set to NaN and
+// the site is computed on the FP64 pipe instead.
+//
+// Digits in FP16: an unsigned byte b = digit + 128 zero-extended to 16 bits is the FP16 subnormal
+// b 2^-24, so a block digit becomes an MMA operand with one byte permutation.  The excess 128 is taken out
+// by starting the sums at -128 2^-24 sum_{p<=s} sum_j x_{s-p,j}, which the column pack computes.
+//
+// Operands: A = a digit plane of a 16 x 16 tile (real or imaginary part), B = the eight levels of the
+// site vector (n = 8): for block digit p, level s takes vector digit s - p, so B is the digit table
+// shifted by p rows (ldmatrix row addresses; rows of zeros before digit 0).  Real and imaginary block
+// planes keep separate sums and are combined per block.  A backward hop uses the transposed tiles: the
+// (re, im) bytes of one entry are one 16-bit element of movmatrix.
+//
+// Block layout: per block n/16 x n/16 tiles, per tile [digit p][lane] uint4, words a0..a3 of the
+// m16n8k16 A fragment, each the bytes {re, im of column 2t, re, im of column 2t + 1}: 8 bytes per real
+// number, one 4 KB stream per tile.
+//
+// One CTA of nine warps per site, one block product per warp (the nine sums are added in a fixed order).
+// A forward block is read again, transposed, by the site in front of it; with a whole site in flight at
+// once, and so as few sites as fill the chip, that second read still finds the block in L2.
+#include <cuda_fp16.h>
+
+#include "digits.cuh"
+
+namespace coarse {
+namespace {
+
+constexpr int kDW = 9;  // warps per site: one block product each
+constexpr unsigned long long kBias = 0x8080808080808080ull;
+constexpr int kMaxExp = 900;        // scales beyond 2^+-900 go to the FP64 pipe
+constexpr int kRange = 8;           // binary orders a block's row or column, or a site's half, may lie below the largest
+
+// The packs look at the doubles as integers (the FP64 pipe would bound them): magnitudes by their high
+// words, whose top bits are the biased exponent.
+__device__ __forceinline__ uint32_t high_abs(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
+__device__ __forceinline__ bool high_finite(uint32_t h) { return h < 0x7ff00000u; }
+
+// Scale of entries whose largest high word is m (finite): true and the biased exponent of the largest, or
+// false where it is too near the range's ends.  m = 0: no entry above the subnormals.
+__device__ __forceinline__ bool scale_of(uint32_t m, int& ex) {
+  ex = (int)(m >> 20);
+  return ex > 1023 - kMaxExp && ex < 1023 + kMaxExp;
+}
+// 2^(E - 6) with 2^E the next power of two above a number of biased exponent ex
+__device__ __forceinline__ double scale_value(int ex) { return __hiloint2double((ex + 1 - 6) << 20, 0); }
+__device__ __forceinline__ double scale_special() { return __hiloint2double(0x7ff80000, 0); }
+
+// fixed-point digits of v, |v| < 2^E, in units of 2^(E - 62): byte 7 - p = digit p + 128
+__device__ __forceinline__ unsigned long long digits_of(double v, int ex) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+  const int e = (int)((hi >> 20) & 0x7ffu), d = ex - e;
+  unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  m = (e == 0 || d > 63) ? 0ull : (m << 9) >> d;
+  return ((hi >> 31) ? 0ull - m : m) + kBias;
+}
+
+// ------------------------------------------------------------------------------- operand packing
+// One CTA per stored block; bound by the 32 n^2 bytes it reads and writes.
+__global__ void __launch_bounds__(256) k_dig_blocks(const double2* __restrict__ blocks, int n, uint4* __restrict__ dig,
+                                                    double* __restrict__ scale) {
+  __shared__ uint32_t rmax[48], cmax[48];
+  __shared__ int ex_sh;
+  const size_t blk = blockIdx.x;
+  const double2* B = blocks + blk * n * n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) rmax[i] = cmax[i] = 0u;
+  __syncthreads();
+  int bad = 0, any = 0;
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const double2 v = B[e];
+    const uint32_t m = max(high_abs(v.x), high_abs(v.y));
+    if (!high_finite(m)) bad = 1;
+    if (v.x != 0.0 || v.y != 0.0) any = 1;
+    atomicMax(rmax + e / n, m);
+    atomicMax(cmax + e % n, m);
+  }
+  bad = __syncthreads_or(bad);
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) {
+    uint32_t m = 0u;
+    for (int i = 0; i < n; ++i) m = max(m, rmax[i]);
+    int ex;
+    if (!scale_of(m, ex) && any) bad = 1;
+    for (int i = 0; i < n; ++i)
+      if ((rmax[i] && (int)(rmax[i] >> 20) + kRange < ex) || (cmax[i] && (int)(cmax[i] >> 20) + kRange < ex)) bad = 1;
+    ex_sh = bad ? 4096 : ex;  // 4096: every entry below the last digit
+    scale[blk] = bad ? scale_special() : (any ? scale_value(ex) : 0.0);
+  }
+  __syncthreads();
+  const int ex = ex_sh, NT = n / 16;
+  for (int w = threadIdx.x; w < NT * NT * 32; w += blockDim.x) {
+    const int lane = w & 31, tile = w >> 5, U = tile / NT, W = tile % NT;
+    const int r = 16 * U + (lane >> 2), c = 16 * W + 2 * (lane & 3);
+    unsigned long long d[4][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // fragment words: rows r, r + 8, then columns + 8
+      const double2* p = B + (size_t)(r + 8 * (k & 1)) * n + c + 8 * (k >> 1);
+      const double2 v0 = p[0], v1 = p[1];
+      d[k][0] = digits_of(v0.x, ex);
+      d[k][1] = digits_of(v0.y, ex);
+      d[k][2] = digits_of(v1.x, ex);
+      d[k][3] = digits_of(v1.y, ex);
+    }
+    uint4* out = dig + ((blk * NT * NT + tile) * 8) * 32 + lane;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      uint32_t o[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        o[k] = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[k] |= (uint32_t)((d[k][q] >> (56 - 8 * p)) & 255ull) << (8 * q);
+      }
+      out[p * 32] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+}
+
+// One warp per (column, site): digits, corrections and scale of the site vector.
+template <int N>
+__global__ void __launch_bounds__(128) k_dig_x(const double2* __restrict__ x, long long ldc, int V,
+                                               __half* __restrict__ xd, float* __restrict__ xc,
+                                               double* __restrict__ xs, const int* stop) {
+  if (stop != nullptr && *stop) return;
+  __shared__ short dg[4][16][N];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int site = blockIdx.x * 4 + warp, col = blockIdx.y;
+  if (site >= V) return;  // warp-uniform
+  const double2* p = x + col * ldc + (size_t)site * N;
+  constexpr int PER = (N + 31) / 32;
+  double2 v[PER];
+  uint32_t m[2] = {0u, 0u};  // largest high word of each chirality half
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int i = lane + 32 * k;
+    v[k] = i < N ? p[i] : make_double2(0.0, 0.0);
+    any = any || v[k].x != 0.0 || v[k].y != 0.0;
+    const uint32_t a = max(high_abs(v[k].x), high_abs(v[k].y));
+    if (i < N / 2) m[0] = max(m[0], a);
+    else m[1] = max(m[1], a);
+  }
+  m[0] = __reduce_max_sync(0xffffffffu, m[0]);
+  m[1] = __reduce_max_sync(0xffffffffu, m[1]);
+  any = __any_sync(0xffffffffu, any);
+  const uint32_t mx = max(m[0], m[1]), mn = min(m[0], m[1]);
+  int ex;
+  bool ok = (scale_of(mx, ex) || !any) && high_finite(mx);
+  if (mn != 0u && (int)(mn >> 20) + kRange < ex) ok = false;
+  if (!ok) ex = 4096;  // every entry below the last digit
+  const size_t rec = (size_t)col * V + site;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const int i = lane + 32 * k;
+    if (i < N) {
+      const unsigned long long dx = digits_of(v[k].x, ex), dy = digits_of(v[k].y, ex);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        dg[warp][q][i] = (short)((int)((dx >> (56 - 8 * q)) & 255ull) - 128);
+        dg[warp][8 + q][i] = (short)((int)((dy >> (56 - 8 * q)) & 255ull) - 128);
+      }
+    }
+  }
+  __syncwarp();
+  __half2* o = reinterpret_cast<__half2*>(xd + rec * dig_x_halves(N));
+  for (int w = lane; w < 8 * N; w += 32) {
+    const int row = w / (N / 2), c = 2 * (w % (N / 2));
+    o[w] = __floats2half2_rn((float)dg[warp][row][c], (float)dg[warp][row][c + 1]);
+  }
+  // lane = (half, part, digit): sums over the half, then the corrections of the two sigma3 variants
+  int sum = 0;
+  {
+    const int row = lane & 15, h = lane >> 4;
+    for (int i = 0; i < N / 2; ++i) sum += dg[warp][row][h * (N / 2) + i];
+  }
+  const int lo = __shfl_sync(0xffffffffu, sum, lane & 15), hi = __shfl_sync(0xffffffffu, sum, 16 + (lane & 15));
+  int t = lane < 16 ? lo + hi : lo - hi;  // lane = (variant, part, digit)
+#pragma unroll
+  for (int off = 1; off < 8; off <<= 1) {  // prefix sums over the digits: levels
+    const int u = __shfl_up_sync(0xffffffffu, t, off, 8);
+    if ((lane & 7) >= off) t += u;
+  }
+  xc[rec * kDigCorr + lane] = (float)t * -0x1p-17f;  // -128 * 2^-24
+  if (lane == 0) xs[rec] = ok ? (any ? scale_value(ex) : 0.0) : scale_special();
+}
+
+// -------------------------------------------------------------------------------------- the stencil
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t movmatrix(uint32_t v) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+  return r;
+}
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
+// Shared-memory digit table of one column: [part][7 zero rows + 8 digits][n], rows padded to an odd
+// number of 16-byte units (conflict-free ldmatrix).
+template <int N> constexpr int dig_row() { return 2 * N + 16; }
+template <int N> constexpr int dig_part() { return 15 * dig_row<N>(); }
+template <int N> constexpr int dig_slab() { return 2 * dig_part<N>(); }
+
+struct DigArgs {
+  const uint4* dig;
+  const double* bscale;
+  const __half* xd;
+  const float* xc;
+  const double* xs;
+};
+
+// One block product of the warp: the block's tiles times the columns' digit tables in `slab`, added to
+// acc[tile][column] (lane (g, t): row 16 tile + g + 8 (t & 1), part t >> 1).
+template <int N, int C, bool BWD>
+__device__ __forceinline__ void dig_block(const uint4* __restrict__ blk, uint4 (&w)[8], uint32_t slab,
+                                          const float* const (&cr)[C], const double (&sc)[C],
+                                          double (&acc)[N / 16][C], bool flip_out) {
+  constexpr int NT = N / 16, RS = dig_row<N>(), PS = dig_part<N>(), SL = dig_slab<N>();
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // ldmatrix row of this lane: matrix lane / 8 = (part, upper half of k), level lane % 8
+  const uint32_t lrow = slab + (uint32_t)((lane >> 4) * PS + (7 + (lane & 7)) * RS + ((lane >> 3) & 1) * 16);
+  float corr[C][4];
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const float2 r = __ldg(reinterpret_cast<const float2*>(cr[c] + 2 * t));
+    const float2 i = __ldg(reinterpret_cast<const float2*>(cr[c] + 8 + 2 * t));
+    corr[c][0] = r.x;
+    corr[c][1] = r.y;
+    corr[c][2] = i.x;
+    corr[c][3] = i.y;
+  }
+  // w: the tile being multiplied; each of its loads is replaced by the next tile's as soon as it is used,
+  // so that a tile's loads are in flight during the whole of the tile before it
+#pragma unroll
+  for (int O = 0; O < NT; ++O) {
+    // sums [column][plane of the block][part of the column]
+    float d[C][2][2][4];
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          d[c][pl][0][k] = corr[c][k & 1];
+          d[c][pl][1][k] = corr[c][2 + (k & 1)];
+        }
+#pragma unroll
+    for (int K = 0; K < NT; ++K) {
+      const int next = O * NT + K + 1;  // in the order (output tile, inner tile)
+      const uint4* tn = blk + (BWD ? (next % NT) * NT + next / NT : next) * 256 + lane;
+#pragma unroll
+      for (int p = 0; p < 8; ++p) {
+        uint32_t a[4];
+        if (BWD) {  // transposed tile: the row and column halves trade places
+          a[0] = movmatrix(w[p].x);
+          a[1] = movmatrix(w[p].z);
+          a[2] = movmatrix(w[p].y);
+          a[3] = movmatrix(w[p].w);
+        } else {
+          a[0] = w[p].x;
+          a[1] = w[p].y;
+          a[2] = w[p].z;
+          a[3] = w[p].w;
+        }
+        uint32_t re[4], im[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          re[k] = __byte_perm(a[k], 0u, 0x4240);
+          im[k] = __byte_perm(a[k], 0u, 0x4341);
+        }
+        if (next < NT * NT) w[p] = __ldg(tn + p * 32);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          uint32_t b[4];
+          ldsm4(lrow + (uint32_t)(c * SL + K * 32 - p * RS), b);
+          mma_f16(d[c][0][0], re, b[0], b[1]);
+          mma_f16(d[c][0][1], re, b[2], b[3]);
+          mma_f16(d[c][1][0], im, b[0], b[1]);
+          mma_f16(d[c][1][1], im, b[2], b[3]);
+        }
+      }
+    }
+    const bool neg = flip_out && (16 * O + g + 8 * (t & 1)) >= N / 2;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      // levels 2t, 2t + 1 of (row g, row g + 8) x (re, im) as integers; F x or F^H x from the planes
+      long long q[2][2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        int yr[2], yi[2];
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+          const int k = 2 * h + l;
+          const float fr = BWD ? d[c][0][0][k] + d[c][1][1][k] : d[c][0][0][k] - d[c][1][1][k];
+          const float fi = BWD ? d[c][0][1][k] - d[c][1][0][k] : d[c][0][1][k] + d[c][1][0][k];
+          yr[l] = __float2int_rn(fr * 0x1p24f);
+          yi[l] = __float2int_rn(fi * 0x1p24f);
+        }
+        q[h][0] = (long long)yr[0] * 256 + yr[1];
+        q[h][1] = (long long)yi[0] * 256 + yi[1];
+      }
+      // sum over the quad's levels: lanes t ^ 1 trade rows, lanes t ^ 2 trade parts
+      long long u[2];
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        const long long own = (t & 1) ? q[1][part] : q[0][part];
+        const long long got = __shfl_xor_sync(0xffffffffu, (t & 1) ? q[0][part] : q[1][part], 1);
+        u[part] = (t & 1) ? (got << 16) + own : (own << 16) + got;
+      }
+      const long long own = (t & 2) ? u[1] : u[0];
+      const long long got = __shfl_xor_sync(0xffffffffu, (t & 2) ? u[0] : u[1], 2);
+      const double hi = (double)((t & 2) ? got : own), lo = (double)((t & 2) ? own : got);
+      const double s = neg ? -sc[c] : sc[c];
+      acc[O][c] = fma(hi, s * 0x1p-24, fma(lo, s * 0x1p-56, acc[O][c]));
+    }
+  }
+}
+
+// The sums of the site's nine blocks on the FP64 pipe (scales marked NaN): eight lanes per row, by the
+// whole CTA; out[2 row + part].
+template <int N>
+__device__ __noinline__ void dig_plain(const ApplyArgs& a, const int* ublk, const int* usrc, const double2* x,
+                                       double* out) {
+  const double2* B = static_cast<const double2*>(a.blocks);
+  const int q = threadIdx.x & 7;
+#pragma unroll 1
+  for (int r0 = 0; r0 < N; r0 += 4 * kDW) {
+    const int r = r0 + (threadIdx.x >> 3), row = r < N ? r : N - 1;
+    double2 y = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int u = 0; u < 9; ++u) {
+      const bool flip = (u < 5) == (a.adjoint != 0);  // sigma3 on the operand and the result
+      const double2* blk = B + (size_t)ublk[u] * N * N;
+      const double2* v = x + (size_t)usrc[u] * N;
+      double2 p = make_double2(0.0, 0.0);
+#pragma unroll 1
+      for (int j = q; j < N; j += 8) {
+        double2 w = v[j];
+        if (flip && j >= N / 2) w = make_double2(-w.x, -w.y);
+        if (u < 5) cfma(p, blk[(size_t)row * N + j], w);
+        else cfma_conj(p, blk[(size_t)j * N + row], w);
+      }
+      if (flip && row >= N / 2) p = make_double2(-p.x, -p.y);
+      y = cadd(y, p);
+    }
+#pragma unroll
+    for (int off = 1; off < 8; off <<= 1) {
+      y.x += __shfl_xor_sync(0xffffffffu, y.x, off);
+      y.y += __shfl_xor_sync(0xffffffffu, y.y, off);
+    }
+    if (q == 0 && r < N) {
+      out[2 * r] = y.x;
+      out[2 * r + 1] = y.y;
+    }
+  }
+}
+
+template <int N, int C>
+__global__ void __launch_bounds__(32 * kDW, C > 1 ? 1 : (N == 16 ? 3 : 2)) k_apply_digits(const __grid_constant__ ApplyArgs a,
+                                                                           const __grid_constant__ DigArgs dgt, int ncol,
+                                                                           long long ldc) {
+  constexpr int NT = N / 16, RS = dig_row<N>(), PS = dig_part<N>(), SL = dig_slab<N>();
+  extern __shared__ __align__(16) unsigned char dsm[];  // [kDW][C] digit tables, then [kDW][C][2N] sums
+  static_assert(SL >= 2 * N * 8, "the sums take the place of the digit tables");
+  __shared__ int ublk[9], usrc[9];
+  if (a.stop != nullptr && *a.stop) return;
+  const int u = threadIdx.x >> 5, lane = threadIdx.x & 31;  // warp u: block product u
+  const int site = blockIdx.x, V = a.V;
+  const int nc = ncol < C ? ncol : C;
+  const int src = u == 0 ? site : __ldg(a.nb + site * 8 + (u - 1));
+  const int blk = u < 5 ? site * 5 + u : src * 5 + 1 + (u - 5);
+  const bool flip = (u < 5) == (a.adjoint != 0);  // sigma3 on the operand and the result
+  if (lane == 0) {
+    ublk[u] = blk;
+    usrc[u] = src;
+  }
+  const uint4* bp = dgt.dig + (size_t)blk * NT * NT * 256;
+  uint4 w[8];
+#pragma unroll
+  for (int p = 0; p < 8; ++p) w[p] = __ldg(bp + lane + p * 32);
+  unsigned char* slab = dsm + (size_t)u * C * SL;
+  const double bs = __ldg(dgt.bscale + blk);
+  const float* cr[C];
+  double sc[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    const size_t rec = (size_t)(c < nc ? c : 0) * V + src;
+    const uint4* xd = reinterpret_cast<const uint4*>(dgt.xd + rec * dig_x_halves(N));
+    constexpr int CH = N / 8;  // 16-byte chunks per row
+#pragma unroll
+    for (int i0 = 0; i0 < 16 * CH; i0 += 32) {
+      const int i = i0 + lane, row = i / CH, kc = i % CH;
+      uint4 v = __ldg(xd + i);
+      if (flip && kc * 8 >= N / 2) {
+        v.x ^= 0x80008000u;
+        v.y ^= 0x80008000u;
+        v.z ^= 0x80008000u;
+        v.w ^= 0x80008000u;
+      }
+      *reinterpret_cast<uint4*>(slab + c * SL + (row >> 3) * PS + (7 + (row & 7)) * RS + kc * 16) = v;
+    }
+    cr[c] = dgt.xc + rec * kDigCorr + (flip ? 16 : 0);
+    sc[c] = bs * __ldg(dgt.xs + rec);
+  }
+  for (int i = lane; i < C * 2 * 7 * (RS / 16); i += 32) {  // the zero rows
+    const int q = i / (RS / 16), tbl = q / 7;               // tbl = (column, part)
+    *reinterpret_cast<uint4*>(slab + (tbl >> 1) * SL + (tbl & 1) * PS + (q % 7) * RS + (i % (RS / 16)) * 16) =
+        make_uint4(0, 0, 0, 0);
+  }
+  int bad = 0;
+#pragma unroll
+  for (int c = 0; c < C; ++c) bad |= !isfinite(sc[c]);
+  __syncwarp();
+  double acc[NT][C];
+#pragma unroll
+  for (int O = 0; O < NT; ++O)
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[O][c] = 0.0;
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(slab);
+  if (u < 5) dig_block<N, C, false>(bp, w, sa, cr, sc, acc, flip);
+  else dig_block<N, C, true>(bp, w, sa, cr, sc, acc, flip);
+  bad = __syncthreads_or(bad);  // also: every warp is done with its tables
+  double* part = reinterpret_cast<double*>(dsm);  // [warp][column][2 row + part]
+  if (!bad) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int O = 0; O < NT; ++O)
+#pragma unroll
+      for (int c = 0; c < C; ++c) part[(u * C + c) * 2 * N + 2 * (16 * O + g + 8 * (t & 1)) + (t >> 1)] = acc[O][c];
+  } else {
+    for (int c = 0; c < nc; ++c)
+      dig_plain<N>(a, ublk, usrc, static_cast<const double2*>(a.x) + (size_t)c * ldc, part + c * 2 * N);
+  }
+  __syncthreads();
+  const double2 c0 = a.mode != APPLY_PLAIN ? a.coef[0] : make_double2(0.0, 0.0);
+  const double2 c1 = a.mode != APPLY_PLAIN ? a.coef[1] : make_double2(0.0, 0.0);
+  const double2 c2 = a.mode == APPLY_POLY_FIRST ? a.coef[2] : make_double2(0.0, 0.0);
+  for (int i = threadIdx.x; i < nc * N; i += blockDim.x) {
+    const int c = i / N, e = i % N;
+    const size_t idx = (size_t)c * ldc + (size_t)site * N + e;
+    const double2* X = static_cast<const double2*>(a.x);
+    const double* pc = part + c * 2 * N + 2 * e;
+    double2 r = make_double2(pc[0], pc[1]);
+    if (!bad)
+#pragma unroll
+      for (int w = 1; w < kDW; ++w) r = cadd(r, make_double2(pc[w * C * 2 * N], pc[w * C * 2 * N + 1]));
+    const double2 xs = X[idx];
+    const double m = e < N / 2 ? a.mu : -a.mu;  // + i mu sigma3 x
+    r.x -= m * xs.y;
+    r.y += m * xs.x;
+    double2* y = static_cast<double2*>(a.y) + idx;
+    if (a.mode == APPLY_PLAIN) {
+      *y = r;
+    } else if (a.mode == APPLY_AXPBY) {
+      *y = cadd(cmul(c0, r), cmul(c1, static_cast<const double2*>(a.z)[idx]));
+    } else {
+      // chain step: s' = s - c0 D s ; acc = acc + c1 s'  (first: acc = c2 s + c1 s')
+      double2* accp = static_cast<double2*>(a.acc) + idx;
+      const double2 ac = a.mode == APPLY_POLY_FIRST ? cmul(c2, xs) : *accp;
+      r = csub(xs, cmul(c0, r));
+      *y = r;
+      *accp = cadd(ac, cmul(c1, r));
+    }
+  }
+}
+
+template <int N, int C>
+int launch_dig_nc(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, cudaStream_t s) {
+  constexpr size_t smem = (size_t)kDW * C * dig_slab<N>();
+  if (smem > 32 * 1024) {  // with the static tables beyond the default 48 KB
+    static bool attr = false;
+    if (!attr) {
+      COARSE_CUDA(cudaFuncSetAttribute(k_apply_digits<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      attr = true;
+    }
+  }
+  k_apply_digits<N, C><<<a.V, 32 * kDW, smem, s>>>(a, d, ncol, ldc);
+  note_launch();
+  COARSE_CUDA(cudaGetLastError());
+  return COARSE_OK;
+}
+
+template <int N>
+int launch_dig_n(const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {
+  DigArgs d;
+  d.dig = static_cast<const uint4*>(a.dig);
+  d.bscale = a.digscale;
+  char* m = static_cast<char*>(a.digx);
+  __half* xd = reinterpret_cast<__half*>(m);
+  m += (size_t)ncol * a.V * dig_x_halves(N) * sizeof(__half);
+  float* xc = reinterpret_cast<float*>(m);
+  m += (size_t)ncol * a.V * kDigCorr * sizeof(float);
+  double* xs = reinterpret_cast<double*>(m);
+  d.xd = xd;
+  d.xc = xc;
+  d.xs = xs;
+  k_dig_x<N><<<dim3((a.V + 3) / 4, ncol), 128, 0, s>>>(static_cast<const double2*>(a.x), ldc, a.V, xd, xc, xs, a.stop);
+  note_launch();
+  COARSE_CUDA(cudaGetLastError());
+  // two columns share the block operand's loads and byte permutations (8^4, n = 48: 427 us for two
+  // columns against 2 x 240 us); four would need 168 registers and spill (1008 us)
+  if (ncol == 1) return launch_dig_nc<N, 1>(a, d, ncol, ldc, s);
+  return launch_dig_nc<N, 2>(a, d, ncol, ldc, s);
+}
+
+}  // namespace
+
+int launch_dig_blocks(const double2* blocks, int V, int n, void* dig, double* scale, cudaStream_t s) {
+  k_dig_blocks<<<V * 5, 256, 0, s>>>(blocks, n, static_cast<uint4*>(dig), scale);
+  note_launch();
+  COARSE_CUDA(cudaGetLastError());
+  return COARSE_OK;
+}
+
+int launch_apply_digits(int n, const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {
+  if (ncol < 1 || ncol > kDigCols) {
+    set_error("digit stencil: %d columns in one pass", ncol);
+    return COARSE_ERR_INVALID_ARG;
+  }
+  switch (n) {
+    case 16: return launch_dig_n<16>(a, ncol, ldc, s);
+    case 32: return launch_dig_n<32>(a, ncol, ldc, s);
+    case 48: return launch_dig_n<48>(a, ncol, ldc, s);
+  }
+  set_error("coarse_apply: unsupported n = %d (nv must be 8, 16 or 24)", n);
+  return COARSE_ERR_INVALID_ARG;
+}
+
+}  // namespace coarse

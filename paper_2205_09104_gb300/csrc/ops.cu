@@ -79,33 +79,50 @@ __global__ void k_gamma5_defect(const double2* self_b, const double2* hop_b, int
 // backward hop of y + mu depends on F_{y,mu} antilinearly, so its gradient folds onto the forward
 // block as sigma3 G^H sigma3:  G4[y][mu][i][j] = -lambda_y[i] conj(x_{y+mu}[j])
 //                                                 - s_i s_j x_y[i] conj(lambda_{y+mu}[j]).
-// One thread per output entry; writes are coalesced along j.
-__global__ void k_block_grad(const double2* lam, const double2* xv, const int* nb, int V, int n, int nhop,
-                             double2* g_self, double2* g_hop) {
-  const size_t nn = (size_t)n * n;
-  const size_t nb_out = 1 + (size_t)nhop;
-  const size_t total = (size_t)V * nb_out * nn;
-  const int half = n / 2;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t x = e / (nb_out * nn);
-    const size_t r = e % (nb_out * nn);
-    const int b = (int)(r / nn);
-    const int i = (int)((r % nn) / n), j = (int)(r % n);
-    const size_t src = (b == 0) ? x : (size_t)nb[x * 8 + (b - 1)];
-    const double2 l = lam[x * n + i];
-    const double2 v = xv[src * n + j];
-    double2 g = make_double2(-(l.x * v.x + l.y * v.y), -(l.y * v.x - l.x * v.y));
-    if (b > 0 && nhop == 4) {
-      // - s_i s_j x_y[i] conj(lambda_{y+mu}[j]), y = x, y + mu = src
-      const double2 xi = xv[x * n + i];
-      const double2 lj = lam[src * n + j];
-      const double sgn = ((i < half) == (j < half)) ? -1.0 : 1.0;
-      g.x += sgn * (xi.x * lj.x + xi.y * lj.y);
-      g.y += sgn * (xi.y * lj.x - xi.x * lj.y);
-    }
-    if (b == 0) g_self[x * nn + (size_t)i * n + j] = g;
-    else g_hop[(x * nhop + (b - 1)) * nn + (size_t)i * n + j] = g;
+//
+// Bound by the HBM writes: (1 + nhop) n^2 V complex128.  One CTA per site: the site's lambda (and, for
+// the folded form, x) and the source vectors of its blocks are read once into shared memory, then
+// the CTA writes the site's blocks in order, 16 bytes per thread and contiguous over the warp, with
+// every index a compile-time division.
+template <int N, int NHOP>
+__global__ void __launch_bounds__(256) k_block_grad(const double2* __restrict__ lam, const double2* __restrict__ xv,
+                                                    const int* __restrict__ nb, double2* __restrict__ g_self,
+                                                    double2* __restrict__ g_hop) {
+  constexpr int NN = N * N, NB = 1 + NHOP, NL = NHOP == 4 ? NB : 1;
+  __shared__ double2 xs[NB][N];  // x of the site and of its NHOP neighbours
+  __shared__ double2 ls[NL][N];  // lambda of the site (folded form: of its forward neighbours too)
+  const size_t x = blockIdx.x;
+  for (int e = threadIdx.x; e < NB * N; e += blockDim.x) {
+    const int b = e / N, j = e % N;
+    const size_t src = b == 0 ? x : (size_t)nb[x * 8 + (b - 1)];
+    xs[b][j] = xv[src * N + j];
+    if (b < NL) ls[b][j] = lam[src * N + j];
   }
+  __syncthreads();
+#pragma unroll 1
+  for (int b = 0; b < NB; ++b) {
+    double2* out = b == 0 ? g_self + x * NN : g_hop + (x * NHOP + (b - 1)) * NN;
+    for (int e = threadIdx.x; e < NN; e += 256) {
+      const int i = e / N, j = e % N;
+      const double2 l = ls[0][i], v = xs[b][j];
+      double2 g = make_double2(fma(-l.x, v.x, -l.y * v.y), fma(-l.y, v.x, l.x * v.y));
+      if (NHOP == 4 && b > 0) {
+        // - s_i s_j x_y[i] conj(lambda_{y+mu}[j]), y the site, y + mu its neighbour b - 1
+        const double2 xi = xs[0][i], lj = ls[b < NL ? b : 0][j];
+        const double sgn = ((i < N / 2) == (j < N / 2)) ? -1.0 : 1.0;
+        g.x += sgn * (xi.x * lj.x + xi.y * lj.y);
+        g.y += sgn * (xi.y * lj.x - xi.x * lj.y);
+      }
+      __stcs(out + e, g);
+    }
+  }
+}
+
+template <int N>
+void block_grad_n(const double2* lam, const double2* x, const int* nb, int V, int nhop, double2* g_self,
+                  double2* g_hop, cudaStream_t s) {
+  if (nhop == 4) k_block_grad<N, 4><<<V, 256, 0, s>>>(lam, x, nb, g_self, g_hop);
+  else k_block_grad<N, 8><<<V, 256, 0, s>>>(lam, x, nb, g_self, g_hop);
 }
 
 int grid_for(size_t total) {
@@ -139,8 +156,12 @@ int launch_gamma5_defect(const double2* self_b, const double2* hop_b, int V, int
 
 int launch_block_grad(const double2* lam, const double2* x, const int* nb, int V, int n, int nhop, double2* g_self,
                       double2* g_hop, cudaStream_t s) {
-  const size_t total = (size_t)V * (1 + nhop) * n * n;
-  k_block_grad<<<grid_for(total), 256, 0, s>>>(lam, x, nb, V, n, nhop, g_self, g_hop);
+  switch (n) {
+    case 16: block_grad_n<16>(lam, x, nb, V, nhop, g_self, g_hop, s); break;
+    case 32: block_grad_n<32>(lam, x, nb, V, nhop, g_self, g_hop, s); break;
+    case 48: block_grad_n<48>(lam, x, nb, V, nhop, g_self, g_hop, s); break;
+    default: set_error("coarse_block_grad: unsupported n = %d", n); return COARSE_ERR_INVALID_ARG;
+  }
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   return COARSE_OK;
