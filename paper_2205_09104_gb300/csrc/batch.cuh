@@ -206,7 +206,7 @@ enum BElem : int {
   BE_AXPY_E_PROJ,    // e += acc after the projection          (gate active, kc > 0)
   BE_TO_LOW,         // r = r64 / ||r64||, e = 0                (gate not done)
   BE_ADD_LOW,        // x64 += ||r64|| e                        (gate not done)
-  BE_ZERO_X,         // x64 = 0                                 (all)
+  BE_ZERO_X,         // x64 = 0, r64 = b64                      (all)
   // odd-even reduction (Sec. 2): the refinement's residual and correction through the halves
   BE_TO_LOW_F,       // f32 = r64 / ||r64||                     (gate not done, full length)
   BE_EO_SPLIT,       // re, ro = even / odd parts of f32, e = 0 (gate not done, half length)

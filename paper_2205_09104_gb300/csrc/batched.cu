@@ -17,6 +17,7 @@
 
 #include "batch.cuh"
 #include "common.cuh"
+#include "mcol.cuh"
 #include "mrhs_core.cuh"
 #include "oddeven.cuh"
 #include "solver.cuh"
@@ -39,6 +40,16 @@ struct Group {
   int count = 0;
   int total = 0;
   int* sidx = nullptr;
+  int* site_off = nullptr;
+};
+
+// n-group of the multi-column stencil phases: the columns of one operator in chunks of kMcCols
+struct CGroup {
+  int n = 0;
+  int count = 0;             // chunks
+  int total = 0;             // sites (or half sites) of all chunks
+  int rmax = 0;              // largest chunk
+  int2* chunks = nullptr;    // {first solve, columns}
   int* site_off = nullptr;
 };
 
@@ -75,11 +86,11 @@ struct Batch {
   int* flags = nullptr;
   int* chunk_off = nullptr;
   // odd-even reduction: the Krylov phases run on the even halves (chunk_off, total_chunks), the
-  // refinement's full-length phases on chunk_off_f / total_chunks_f; egroups: half-site groups
+  // refinement's full-length phases on chunk_off_f / total_chunks_f
   bool eo = false;
   int* chunk_off_f = nullptr;
   int total_chunks_f = 0;
-  std::vector<Group> egroups;
+  std::vector<CGroup> cgroups;  // stencil phases (half-site counts with the odd-even reduction)
   std::vector<Group> groups;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -94,10 +105,9 @@ struct Batch {
   // one half apply of the odd-even reduced operator over every n-group
   int eo_half(int out_par, int vsel, int zsel, int bsel, int ysel, int mode, int coef_off, int gate, bool chain,
               cudaStream_t s) {
-    for (const Group& g : egroups) {
+    for (const CGroup& g : cgroups) {
       BEoApply a;
       a.S = dS;
-      a.sidx = g.sidx;
       a.site_off = g.site_off;
       a.count = g.count;
       a.total = g.total;
@@ -111,7 +121,7 @@ struct Batch {
       a.gate = gate;
       a.step = step;
       a.poly_blocks = chain ? 1 : 0;
-      TRY(launch_beo_half(chain ? poly_prec : prec, g.n, a, s));
+      TRY(launch_beo_mc(chain ? poly_prec : prec, g.n, a, g.chunks, g.rmax, s));
     }
     return COARSE_OK;
   }
@@ -136,10 +146,10 @@ struct Batch {
       }
       return COARSE_OK;
     }
-    for (const Group& g : groups) {
+    for (const CGroup& g : cgroups) {
       BApply a;
       a.S = dS;
-      a.sidx = g.sidx;
+      a.sidx = nullptr;
       a.site_off = g.site_off;
       a.count = g.count;
       a.total = g.total;
@@ -150,7 +160,7 @@ struct Batch {
       a.gate = gate;
       a.step = step;
       a.poly_blocks = chain ? 1 : 0;
-      TRY(launch_bapply(chain ? poly_prec : prec, g.n, a, s));
+      TRY(launch_bapply_mc(chain ? poly_prec : prec, g.n, a, g.chunks, g.rmax, s));
     }
     return COARSE_OK;
   }
@@ -533,7 +543,7 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
   const size_t o_coff = take(sizeof(int) * (ns + 1));
   const size_t o_coff_f = take(sizeof(int) * (ns + 1));
   const size_t o_groups = take(sizeof(int) * (2 * ns + 8) * 3);
-  const size_t o_egroups = take(sizeof(int) * (2 * ns + 8) * 3);
+  const size_t o_cgroups = take((sizeof(int2) + sizeof(int)) * ((size_t)ns + 8) + 3 * 256);
   const size_t o_ctl = take(sizeof(BCtl));
   const size_t o_info = take(sizeof(BInfo) * ns);
   // multi-RHS stencil phases: BF16 inner solves, every operator carrying the fragment-layout
@@ -813,27 +823,34 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
       B.groups.push_back(g);
     }
   }
-  // odd-even: n-groups over the half-site counts (one output parity per half apply)
-  if (eo) {
-    int* g0 = reinterpret_cast<int*>(B.mem + o_egroups);
+  // n-groups of the multi-column phases: every operator's columns in chunks of nearly equal size
+  if (!B.mrhs) {
+    char* g0 = B.mem + o_cgroups;
     for (int n : {16, 32, 48}) {
-      std::vector<int> idx, off(1, 0);
-      for (int q = 0; q < ns; ++q)
-        if (hs[q].n == n) {
-          idx.push_back(q);
-          off.push_back(off.back() + hs[q].V / 2);
+      std::vector<int2> ch;
+      std::vector<int> off(1, 0);
+      CGroup g;
+      int s0 = 0;
+      for (int i = 0; i < nops; ++i) {
+        const int passes = (nrhs[i] + kMcCols - 1) / kMcCols;
+        for (int c = 0; ops[i]->n == n && c < passes; ++c) {
+          const int lo = (int)((long long)nrhs[i] * c / passes), hi = (int)((long long)nrhs[i] * (c + 1) / passes);
+          ch.push_back(make_int2(s0 + lo, hi - lo));
+          off.push_back(off.back() + (eo ? ops[i]->V / 2 : ops[i]->V));
+          g.rmax = std::max(g.rmax, hi - lo);
         }
-      if (idx.empty()) continue;
-      Group g;
+        s0 += nrhs[i];
+      }
+      if (ch.empty()) continue;
       g.n = n;
-      g.count = (int)idx.size();
+      g.count = (int)ch.size();
       g.total = off.back();
-      g.sidx = g0;
-      g.site_off = g0 + idx.size();
-      COARSE_CUDA(cudaMemcpyAsync(g.sidx, idx.data(), sizeof(int) * idx.size(), cudaMemcpyHostToDevice, s));
+      g.chunks = reinterpret_cast<int2*>(g0);
+      g.site_off = reinterpret_cast<int*>(g.chunks + ch.size());
+      COARSE_CUDA(cudaMemcpyAsync(g.chunks, ch.data(), sizeof(int2) * ch.size(), cudaMemcpyHostToDevice, s));
       COARSE_CUDA(cudaMemcpyAsync(g.site_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, s));
-      g0 += idx.size() + off.size();
-      B.egroups.push_back(g);
+      g0 += align256(sizeof(int2) * ch.size() + sizeof(int) * off.size());
+      B.cgroups.push_back(g);
     }
   }
   int kmin = m;
@@ -917,8 +934,12 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
     return COARSE_OK;
   };
   auto top = [&](cudaStream_t q) -> int {
-    if (zero_guess) TRY(B.elem(BE_ZERO_X, q));
-    TRY(B.residual64(q));
+    if (zero_guess) {  // x = 0: r = b exactly, no stencil
+      TRY(B.elem(BE_ZERO_X, q));
+      TRY(B.norms64(1, q));
+    } else {
+      TRY(B.residual64(q));
+    }
     TRY(B.norms64(2, q));
     kb_ctl_start<<<1, kCtlThreads, 0, q>>>(dctl, B.dS, dinfo, ns);
     note_launch();

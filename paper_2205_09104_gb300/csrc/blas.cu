@@ -596,7 +596,10 @@ __global__ void __launch_bounds__(32 * kW) kb_elem(int op, const BSolve* S, int 
         f[(size_t)s.eo_sites[k] * s.n + c] = ((const float2*)s.e)[idx];
         f[(size_t)s.eo_sites[s.V / 2 + k] * s.n + c] = ((const float2*)s.eoe)[idx];
       } break;
-      default: s.x64[idx] = make_double2(0.0, 0.0); break;
+      default:
+        s.x64[idx] = make_double2(0.0, 0.0);
+        s.r64[idx] = s.b64[idx];
+        break;
     }
   }
 }

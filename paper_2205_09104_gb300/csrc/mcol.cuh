@@ -1,0 +1,20 @@
+// Multi-column stencil and half apply on the FP32 pipe (mcol.cu).
+#pragma once
+
+#include "batch.cuh"
+#include "common.cuh"
+
+namespace coarse {
+
+constexpr int kMcCols = 12;  // columns of one pass (shared memory holds their vectors)
+
+// y = D x for R <= kMcCols complex64 columns (x + c * ldc -> y + c * ldc) on the FP32 blocks of `a`, plain
+// epilogue; x 16-byte aligned, ldc even.
+int launch_apply_mc(int n, const ApplyArgs& a, int R, long long ldc, cudaStream_t s);
+
+// The batched phases over column chunks: b.site_off are prefix sums over the chunks of one n-group, chunk k
+// covers the solves chunks[k].x .. + chunks[k].y - 1 of one operator; rmax: largest chunk of the group.
+int launch_beo_mc(int prec, int n, const BEoApply& b, const int2* chunks, int rmax, cudaStream_t s);
+int launch_bapply_mc(int prec, int n, const BApply& b, const int2* chunks, int rmax, cudaStream_t s);
+
+}  // namespace coarse
