@@ -325,40 +325,6 @@ int launch_tma(int n, const ApplyArgs& a, cudaStream_t s) {
   return COARSE_ERR_INVALID_ARG;
 }
 
-// ------------------------------------------------------------------------------------------
-// Batched stencil: one launch applies D_c for every solve of an n-group.  Warp g of the flat
-// grid takes global site g, finds its solve through the site prefix sums and runs the same
-// per-site push-pull body as k_apply with that solve's operator, vectors and scratch.
-template <int N, class BT>
-__global__ void __launch_bounds__(128) kb_apply(BApply b) {
-  __shared__ float2 ys[4][N];
-  const int warp = threadIdx.x >> 5;
-  const int g = blockIdx.x * 4 + warp;
-  if (g >= b.total) return;
-  const int k = find_solve(b.site_off, b.count, g);
-  const BSolve& s = b.S[b.sidx[k]];
-  if (!bgate(s, b.gate)) return;  // uniform for all sites of the solve
-  const int step = *b.step;
-  ApplyArgs a;
-  a.blocks = b.poly_blocks ? s.blk_poly : s.blk;
-  a.nb = s.nb;
-  a.V = s.V;
-  a.mu = s.mu;
-  a.x = bsel(s, b.xsel, step);
-  a.y = bsel(s, b.ysel, step);
-  a.z = nullptr;
-  a.acc = s.acc;
-  a.coef = s.polyc + b.coef_off;
-  a.mode = b.mode;
-  a.adjoint = 0;
-  a.stop = nullptr;
-  a.part = s.part;
-  a.push = s.push;
-  a.cnt = s.cnt;
-  a.err = s.cnt + s.V;
-  apply_site<N, BT, float2, float2>(a, g - b.site_off[k], ys[warp]);
-}
-
 // FP64 residual of every not-yet-converged solve: r64 = b64 - D x64.
 template <int N>
 __global__ void __launch_bounds__(128) kb_residual64(BApply b, const double2* coef) {
@@ -453,29 +419,6 @@ int launch_apply(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
 }  // namespace coarse
 
 namespace coarse {
-
-int launch_bapply(int prec, int n, const BApply& b, cudaStream_t s) {
-  if (b.total <= 0) return COARSE_OK;
-  const int grid = (b.total + 3) / 4;
-  if (prec == COARSE_PREC_FP32) {
-    switch (n) {
-      case 16: kb_apply<16, float2><<<grid, 128, 0, s>>>(b); break;
-      case 32: kb_apply<32, float2><<<grid, 128, 0, s>>>(b); break;
-      case 48: kb_apply<48, float2><<<grid, 128, 0, s>>>(b); break;
-      default: set_error("batched apply: unsupported n = %d", n); return COARSE_ERR_INVALID_ARG;
-    }
-  } else {
-    switch (n) {
-      case 16: kb_apply<16, cbf16><<<grid, 128, 0, s>>>(b); break;
-      case 32: kb_apply<32, cbf16><<<grid, 128, 0, s>>>(b); break;
-      case 48: kb_apply<48, cbf16><<<grid, 128, 0, s>>>(b); break;
-      default: set_error("batched apply: unsupported n = %d", n); return COARSE_ERR_INVALID_ARG;
-    }
-  }
-  note_launch();
-  COARSE_CUDA(cudaGetLastError());
-  return COARSE_OK;
-}
 
 int launch_bapply64_residual(int n, const BApply& b, cudaStream_t s) {
   if (b.total <= 0) return COARSE_OK;

@@ -72,6 +72,30 @@ struct BSolve {
 enum BSel : int { BS_NONE = -1, BS_VJ = 0, BS_VJ1, BS_SA, BS_SB, BS_ACC, BS_T, BS_R, BS_E, BS_TODD, BS_RE, BS_RO,
                   BS_TO, BS_EOE };
 
+// Byte offset of a solve's complex64 vector from the base of its vector memory (vb: bytes of a full-length
+// vector, m: restart length): the Krylov basis, the work vectors, then with the odd-even reduction the
+// full-length f32 and the halves.  The host fills BSolve's pointers by it, and the multi-column phases
+// compute their addresses from it, without a pointer chase.
+__host__ __device__ inline size_t batch_vec_offset(int sel, int step, int m, size_t vb) {
+  const size_t hb = vb / 2, w = (size_t)(m + 8) * vb;
+  switch (sel) {
+    case BS_VJ: return (size_t)step * vb;
+    case BS_VJ1: return (size_t)(step + 1) * vb;
+    case BS_R: return (size_t)(m + 1) * vb;
+    case BS_E: return (size_t)(m + 2) * vb;
+    case BS_T: return (size_t)(m + 3) * vb;
+    case BS_SA: return (size_t)(m + 4) * vb;
+    case BS_SB: return (size_t)(m + 5) * vb;
+    case BS_ACC: return (size_t)(m + 6) * vb;
+    case BS_RE: return w;
+    case BS_RO: return w + hb;
+    case BS_TO: return w + 2 * hb;
+    case BS_EOE: return w + 3 * hb;
+    case BS_TODD: return w + 4 * hb;
+  }
+  return 0;
+}
+
 // Gate of a batched phase: run the solve's part only if ...
 enum BGate : int {
   BG_STEP = 0,   // ... its Arnoldi cycle is running (st->stop == 0)
@@ -80,18 +104,15 @@ enum BGate : int {
   BG_NOTDONE = 3 // ... it has not met the tolerance (flags[1] == 0)
 };
 
+// FP64 residual phase: one site of one solve per warp
 struct BApply {
   const BSolve* S;
   const int* sidx;      // solves of this n-group
   const int* site_off;  // prefix sums of their site counts (count + 1 entries)
   int count;
   int total;            // total sites
-  int mode;             // ApplyMode
-  int xsel, ysel;       // BSel
-  int coef_off;         // offset (in double2) into polyc for POLY modes
   int gate;             // BGate
   const int* step;      // device step counter
-  int poly_blocks;      // 1: the solves' blk_poly (polynomial-chain phases), 0: blk
 };
 
 // work item -> solve, gates and vector selection shared by the batched kernels
@@ -133,25 +154,44 @@ __device__ inline void* bsel(const BSolve& s, int sel, int step) {
   return nullptr;
 }
 
-// One batched half apply of the odd-even reduced operator (Sec. 2, Sec. 3.2) over an n-group:
-// output sites of parity out_par, y = B^{-1} (z - sum hops v) or base - B^{-1} (...), chain epilogue.
-struct BEoApply {
+// One site of one column chunk of an operator: a CTA of the multi-column phases.
+struct __align__(16) McItem {
+  int s0, cols;      // first solve, columns (solves s0 .. s0 + cols - 1)
+  int q, nh;         // output site (of its parity), sites per parity; full stencil: the site, 0
+  const int4* rec;   // eo_rec of the operator
+  size_t vb;         // bytes of a full-length complex64 vector
+};
+
+// A multi-column stencil phase over the items of one n-group (Sec. 2, Sec. 3.2 for the half apply:
+// output sites of parity out_par, y = B^{-1} (z - sum hops v) or base - B^{-1} (...), chain epilogue).
+struct McPhase {
+  const McItem* items;
+  int count;            // items
+  int rmax;             // largest chunk
   const BSolve* S;
-  const int* sidx;      // solves of this n-group
-  const int* site_off;  // prefix sums of their half-site counts V / 2 (count + 1 entries)
-  int count;
-  int total;            // total output sites
+  const CycleState* states;  // of all solves
+  const int* flags;          // [solve][2]
+  char* const* vbase;        // vector memory of each solve
+  int m;
   int out_par;
-  int vsel, zsel, bsel, ysel;  // BSel (BS_NONE: absent)
+  int vsel, zsel, bsel, ysel;  // BSel (BS_NONE: absent); full stencil: vsel, ysel
   int mode;
   int coef_off;
   int gate;
   const int* step;
   int poly_blocks;      // 1: the chain's blocks and inverses
 };
-int launch_beo_half(int prec, int n, const BEoApply& b, cudaStream_t s);
 
-int launch_bapply(int prec, int n, const BApply& a, cudaStream_t s);
+// bgate() from the solves' arrays
+__device__ inline bool mc_gate(const McPhase& p, int q) {
+  switch (p.gate) {
+    case BG_STEP: return p.states[q].stop == 0;
+    case BG_ACTIVE: return p.flags[2 * q] != 0;
+    case BG_TAIL: return p.flags[2 * q] != 0 && p.states[q].j > 0;
+    case BG_NOTDONE: return p.flags[2 * q + 1] == 0;
+  }
+  return false;
+}
 
 // ---- multi-RHS (tensor-core) stencil phases: every column of one operator in one pass
 struct BMOp {

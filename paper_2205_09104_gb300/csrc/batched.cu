@@ -46,11 +46,7 @@ struct Group {
 // n-group of the multi-column stencil phases: the columns of one operator in chunks of kMcCols
 struct CGroup {
   int n = 0;
-  int count = 0;             // chunks
-  int total = 0;             // sites (or half sites) of all chunks
-  int rmax = 0;              // largest chunk
-  int2* chunks = nullptr;    // {first solve, columns}
-  int* site_off = nullptr;
+  McPhase p{};  // items and per-solve arrays; phase fields filled per launch
 };
 
 // n-group of the multi-RHS stencil phases
@@ -106,11 +102,7 @@ struct Batch {
   int eo_half(int out_par, int vsel, int zsel, int bsel, int ysel, int mode, int coef_off, int gate, bool chain,
               cudaStream_t s) {
     for (const CGroup& g : cgroups) {
-      BEoApply a;
-      a.S = dS;
-      a.site_off = g.site_off;
-      a.count = g.count;
-      a.total = g.total;
+      McPhase a = g.p;
       a.out_par = out_par;
       a.vsel = vsel;
       a.zsel = zsel;
@@ -119,9 +111,8 @@ struct Batch {
       a.mode = mode;
       a.coef_off = coef_off;
       a.gate = gate;
-      a.step = step;
       a.poly_blocks = chain ? 1 : 0;
-      TRY(launch_beo_mc(chain ? poly_prec : prec, g.n, a, g.chunks, g.rmax, s));
+      TRY(launch_beo_mc(chain ? poly_prec : prec, g.n, a, s));
     }
     return COARSE_OK;
   }
@@ -147,20 +138,15 @@ struct Batch {
       return COARSE_OK;
     }
     for (const CGroup& g : cgroups) {
-      BApply a;
-      a.S = dS;
-      a.sidx = nullptr;
-      a.site_off = g.site_off;
-      a.count = g.count;
-      a.total = g.total;
-      a.mode = mode;
-      a.xsel = xsel;
+      McPhase a = g.p;
+      a.vsel = xsel;
       a.ysel = ysel;
+      a.zsel = a.bsel = BS_NONE;
+      a.mode = mode;
       a.coef_off = coef_off;
       a.gate = gate;
-      a.step = step;
       a.poly_blocks = chain ? 1 : 0;
-      TRY(launch_bapply_mc(chain ? poly_prec : prec, g.n, a, g.chunks, g.rmax, s));
+      TRY(launch_bapply_mc(chain ? poly_prec : prec, g.n, a, s));
     }
     return COARSE_OK;
   }
@@ -224,12 +210,8 @@ struct Batch {
       a.site_off = g.site_off;
       a.count = g.count;
       a.total = g.total;
-      a.mode = APPLY_AXPBY;
-      a.xsel = a.ysel = 0;
-      a.coef_off = 0;
       a.gate = BG_NOTDONE;
       a.step = step;
-      a.poly_blocks = 0;
       TRY(launch_bapply64_residual(g.n, a, s));
     }
     return norms64(1, s);
@@ -543,7 +525,11 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
   const size_t o_coff = take(sizeof(int) * (ns + 1));
   const size_t o_coff_f = take(sizeof(int) * (ns + 1));
   const size_t o_groups = take(sizeof(int) * (2 * ns + 8) * 3);
-  const size_t o_cgroups = take((sizeof(int2) + sizeof(int)) * ((size_t)ns + 8) + 3 * 256);
+  const size_t o_vbase = take(sizeof(char*) * ns);
+  size_t n_items = 0;  // sites of all column chunks
+  for (int i = 0; i < nops; ++i)
+    n_items += (size_t)((nrhs[i] + kMcCols - 1) / kMcCols) * (eo ? ops[i]->V / 2 : ops[i]->V);
+  const size_t o_items = take(sizeof(McItem) * n_items);
   const size_t o_ctl = take(sizeof(BCtl));
   const size_t o_info = take(sizeof(BInfo) * ns);
   // multi-RHS stencil phases: BF16 inner solves, every operator carrying the fragment-layout
@@ -657,24 +643,20 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
         S.mu = op->mu;
         std::vector<void*>& T = tabs[sidx];
         for (int j = 0; j <= m; ++j) T.push_back(v + j * vb);
-        S.r = v + (m + 1) * vb;
-        S.e = v + (m + 2) * vb;
-        S.t = v + (m + 3) * vb;
-        S.sa = v + (m + 4) * vb;
-        S.sb = v + (m + 5) * vb;
-        S.acc = v + (m + 6) * vb;
-        S.part = v + (m + 7) * vb;
-        S.push = v + (m + 8) * vb;
+        auto vec = [&](int sel) { return v + batch_vec_offset(sel, 0, m, vb); };
+        S.r = vec(BS_R);
+        S.e = vec(BS_E);
+        S.t = vec(BS_T);
+        S.sa = vec(BS_SA);
+        S.sb = vec(BS_SB);
+        S.acc = vec(BS_ACC);
         if (eo) {
-          // the half apply keeps no stencil scratch: its 5 N-vector region holds the odd-even work
-          const size_t hb = vb / 2;
-          char* w = v + (m + 7) * vb;
-          S.f32 = w;
-          S.re = w + vb;
-          S.ro = w + vb + hb;
-          S.to = w + vb + 2 * hb;
-          S.eoe = w + vb + 3 * hb;
-          S.todd = w + vb + 4 * hb;
+          S.f32 = v + (m + 7) * vb;
+          S.re = vec(BS_RE);
+          S.ro = vec(BS_RO);
+          S.to = vec(BS_TO);
+          S.eoe = vec(BS_EOE);
+          S.todd = vec(BS_TODD);
           S.inv = op->inv[0][prec].ptr;
           S.inv_poly = op->inv[0][B.poly_prec].ptr;
           S.eo_rec = op->eo_rec;
@@ -823,33 +805,41 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
       B.groups.push_back(g);
     }
   }
-  // n-groups of the multi-column phases: every operator's columns in chunks of nearly equal size
+  // n-groups of the multi-column phases: every operator's columns in chunks of nearly equal size, one item
+  // (CTA) per chunk and site
+  std::vector<char*> vbase(ns);
+  std::vector<McItem> items[3];
   if (!B.mrhs) {
-    char* g0 = B.mem + o_cgroups;
+    for (int q = 0; q < ns; ++q) vbase[q] = B.mem + off_vec[q];
+    char** dbase = reinterpret_cast<char**>(B.mem + o_vbase);
+    COARSE_CUDA(cudaMemcpyAsync(dbase, vbase.data(), sizeof(char*) * ns, cudaMemcpyHostToDevice, s));
+    McItem* at = reinterpret_cast<McItem*>(B.mem + o_items);
     for (int n : {16, 32, 48}) {
-      std::vector<int2> ch;
-      std::vector<int> off(1, 0);
+      std::vector<McItem>& list = items[n / 16 - 1];
       CGroup g;
       int s0 = 0;
       for (int i = 0; i < nops; ++i) {
-        const int passes = (nrhs[i] + kMcCols - 1) / kMcCols;
+        const int passes = (nrhs[i] + kMcCols - 1) / kMcCols, sites = eo ? ops[i]->V / 2 : ops[i]->V;
         for (int c = 0; ops[i]->n == n && c < passes; ++c) {
           const int lo = (int)((long long)nrhs[i] * c / passes), hi = (int)((long long)nrhs[i] * (c + 1) / passes);
-          ch.push_back(make_int2(s0 + lo, hi - lo));
-          off.push_back(off.back() + (eo ? ops[i]->V / 2 : ops[i]->V));
-          g.rmax = std::max(g.rmax, hi - lo);
+          McItem t{s0 + lo, hi - lo, 0, eo ? sites : 0, ops[i]->eo_rec, sizeof(float2) * (size_t)ops[i]->V * n};
+          for (t.q = 0; t.q < sites; ++t.q) list.push_back(t);
+          g.p.rmax = std::max(g.p.rmax, hi - lo);
         }
         s0 += nrhs[i];
       }
-      if (ch.empty()) continue;
+      if (list.empty()) continue;
       g.n = n;
-      g.count = (int)ch.size();
-      g.total = off.back();
-      g.chunks = reinterpret_cast<int2*>(g0);
-      g.site_off = reinterpret_cast<int*>(g.chunks + ch.size());
-      COARSE_CUDA(cudaMemcpyAsync(g.chunks, ch.data(), sizeof(int2) * ch.size(), cudaMemcpyHostToDevice, s));
-      COARSE_CUDA(cudaMemcpyAsync(g.site_off, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice, s));
-      g0 += align256(sizeof(int2) * ch.size() + sizeof(int) * off.size());
+      g.p.items = at;
+      g.p.count = (int)list.size();
+      g.p.S = B.dS;
+      g.p.states = B.states;
+      g.p.flags = B.flags;
+      g.p.vbase = dbase;
+      g.p.m = m;
+      g.p.step = B.step;
+      COARSE_CUDA(cudaMemcpyAsync(at, list.data(), sizeof(McItem) * list.size(), cudaMemcpyHostToDevice, s));
+      at += list.size();
       B.cgroups.push_back(g);
     }
   }

@@ -265,51 +265,91 @@ __device__ __forceinline__ void mc_finish(int mode, float2 r, float2 xs, const d
   *acc = cadd(ac, cmul(c1, sp));
 }
 
-// Batched half apply: CTA -> (operator's column chunk, output site); columns whose gate is closed drop out.
-template <int N, class BT>
-__global__ void __launch_bounds__(32 * kMW) kb_eo_mc(BEoApply b, const int2* __restrict__ chunks) {
-  extern __shared__ __align__(16) unsigned char mc_sm[];
-  __shared__ const float2* vp[kMcCols];
-  __shared__ int act[kMcCols];
-  __shared__ int nact;
-  const int k = find_solve(b.site_off, b.count, blockIdx.x);
-  const int2 ch = chunks[k];  // first solve, columns
-  const int q = blockIdx.x - b.site_off[k];
-  const int step = *b.step;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0) {
-    const bool on = lane < ch.y && bgate(b.S[ch.x + (lane < ch.y ? lane : 0)], b.gate);
+// The vectors of a chunk's columns whose gate is open, gathered once per CTA in one round of loads (the
+// latency of a chain of descriptor loads would otherwise be most of a small site's time).
+struct McPtrs {
+  const float2* v[kMcCols];
+  const float2* z[kMcCols];
+  const float2* base[kMcCols];
+  float2* y[kMcCols];
+  float2* acc[kMcCols];
+  const double2* coef[kMcCols];
+  float mu[kMcCols];
+  int n;
+};
+
+// by the whole CTA; returns the number of columns
+__device__ __forceinline__ int mc_setup(McPtrs& P, const McPhase& p, const McItem& it) {
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x, q = it.s0 + lane;
+    const int step = *p.step;
+    const bool in = lane < it.cols;
+    char* base = in ? p.vbase[q] : nullptr;
+    const double2* coef = in ? p.S[q].polyc : nullptr;
+    const double mu = in ? p.S[q].mu : 0.0;
+    const bool on = in && mc_gate(p, q);
     const uint32_t m = __ballot_sync(0xffffffffu, on);
     if (on) {
       const int at = __popc(m & ((1u << lane) - 1u));
-      act[at] = ch.x + lane;
-      vp[at] = static_cast<const float2*>(bsel(b.S[ch.x + lane], b.vsel, step));
+      auto vec = [&](int sel) {
+        return sel == BS_NONE ? nullptr : reinterpret_cast<float2*>(base + batch_vec_offset(sel, step, p.m, it.vb));
+      };
+      P.v[at] = vec(p.vsel);
+      P.z[at] = vec(p.zsel);
+      P.base[at] = vec(p.bsel);
+      P.y[at] = vec(p.ysel);
+      P.acc[at] = vec(BS_ACC);
+      P.coef[at] = coef + p.coef_off;
+      P.mu[at] = (float)mu;
     }
-    if (lane == 0) nact = __popc(m);
+    if (lane == 0) P.n = __popc(m);
   }
-  const BSolve& s0 = b.S[ch.x];
-  const int nh = s0.V / 2;
-  const int4 rec = __ldg(s0.eo_rec + ((size_t)b.out_par * nh + q) * 4 + warp);
   __syncthreads();
-  const int R = nact;
+  return P.n;
+}
+
+__device__ __forceinline__ McItem load_item(const McItem* p) {
+  McItem it;
+  const int4 a = __ldg(reinterpret_cast<const int4*>(p));
+  const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(p) + 1);
+  it.s0 = a.x;
+  it.cols = a.y;
+  it.q = a.z;
+  it.nh = a.w;
+  it.rec = reinterpret_cast<const int4*>(b.x);
+  it.vb = b.y;
+  return it;
+}
+
+// Batched half apply: CTA -> (operator's column chunk, output site); columns whose gate is closed drop out.
+template <int N, class BT>
+__global__ void __launch_bounds__(32 * kMW) kb_eo_mc(const __grid_constant__ McPhase b) {
+  extern __shared__ __align__(16) unsigned char mc_sm[];
+  __shared__ McPtrs P;
+  const McItem it = load_item(b.items + blockIdx.x);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int4 rec = __ldg(it.rec + ((size_t)b.out_par * it.nh + it.q) * 4 + warp);
+  const BSolve& s0 = b.S[it.s0];
+  const BT* B = static_cast<const BT*>(b.poly_blocks ? s0.blk_poly : s0.blk);
+  const BT* inv = static_cast<const BT*>(b.poly_blocks ? s0.inv_poly : s0.inv) + (size_t)rec.w * N * N;
+  const int R = mc_setup(P, b, it);
   if (R == 0) return;
   float2* tabs = reinterpret_cast<float2*>(mc_sm);
   float* hp = reinterpret_cast<float*>(tabs + (size_t)2 * kMW * R * N);  // [warp][column][2 row + part]
   McSite s;
-  s.blocks = b.poly_blocks ? s0.blk_poly : s0.blk;
+  s.blocks = B;
   s.x = rec.w;
   s.R = R;
   s.adj = 0;
-  const BT* inv = static_cast<const BT*>(b.poly_blocks ? s0.inv_poly : s0.inv) + (size_t)s.x * N * N;
   Piece<N, BT> tail;
   if (b.vsel != BS_NONE) {
-    mc_hops<N, BT>(s, warp, rec, vp, tabs + (size_t)warp * R * N, hp + (size_t)warp * R * 2 * N, inv, tail, lane);
+    mc_hops<N, BT>(s, warp, rec, P.v, tabs + (size_t)warp * R * N, hp + (size_t)warp * R * 2 * N, inv, tail, lane);
     __syncthreads();
   } else {
     tail.load_rows(inv, 16 * (warp % (N / 16)), lane);
   }
   // g = z - h (or h): the operand of the inverse block
-  const size_t off = (size_t)q * N;
+  const size_t off = (size_t)it.q * N;
   for (int i = threadIdx.x; i < R * N; i += blockDim.x) {
     const int c = i / N, e = i % N;
     float2 g = make_float2(0.f, 0.f);
@@ -317,25 +357,21 @@ __global__ void __launch_bounds__(32 * kMW) kb_eo_mc(BEoApply b, const int2* __r
       const float2* h = reinterpret_cast<const float2*>(hp) + i;
       g = cadd(cadd(h[0], h[(size_t)R * N]), cadd(h[(size_t)2 * R * N], h[(size_t)3 * R * N]));
     }
-    if (b.zsel != BS_NONE) {
-      const float2 z = static_cast<const float2*>(bsel(b.S[act[c]], b.zsel, step))[off + e];
-      g = csub(z, g);
-    }
+    if (b.zsel != BS_NONE) g = csub(P.z[c][off + e], g);
     tabs[i] = g;
   }
   __syncthreads();
   mc_block<N, BT, false>(tail, tabs, hp, R, false, warp, lane);
   __syncthreads();
   for (int i = threadIdx.x; i < R * N; i += blockDim.x) {
-    const BSolve& S = b.S[act[i / N]];
+    const int c = i / N;
     const size_t idx = off + i % N;
     float2 r = reinterpret_cast<const float2*>(hp)[i], xs = make_float2(0.f, 0.f);
     if (b.bsel != BS_NONE) {
-      xs = static_cast<const float2*>(bsel(S, b.bsel, step))[idx];
+      xs = P.base[c][idx];
       r = csub(xs, r);
     }
-    mc_finish(b.mode, r, xs, S.polyc + b.coef_off, static_cast<float2*>(bsel(S, b.ysel, step)) + idx,
-              static_cast<float2*>(S.acc) + idx);
+    mc_finish(b.mode, r, xs, P.coef[c], P.y[c] + idx, P.acc[c] + idx);
   }
 }
 
@@ -407,172 +443,174 @@ __device__ __forceinline__ void fill_split(unsigned char* tab, const float2* con
   }
 }
 
-// One row of tiles of a block (or of its transpose) in registers as loaded.
+// Tile (rt, K) of a block, or of its transpose, in registers as loaded: words [4 h + e] of the A fragment's
+// rows 2g + h and entries 4t + e.
 template <int N, bool BWD>
-struct TileRow {
-  uint32_t u[N / 16][8];
-  __device__ __forceinline__ void load(const cbf16* blk, int rt, int lane) {
-    const int g = lane >> 2, t = lane & 3;
-    const uint32_t* b = reinterpret_cast<const uint32_t*>(blk);
+__device__ __forceinline__ void load_tile(uint32_t (&u)[8], const cbf16* blk, int rt, int K, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  const uint32_t* b = reinterpret_cast<const uint32_t*>(blk);
+  if (!BWD) {
 #pragma unroll
-    for (int K = 0; K < N / 16; ++K) {
-      if (!BWD) {
+    for (int h = 0; h < 2; ++h) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(b + (16 * rt + 2 * g + h) * N + 16 * K + 4 * t));
+      u[4 * h] = v.x;
+      u[4 * h + 1] = v.y;
+      u[4 * h + 2] = v.z;
+      u[4 * h + 3] = v.w;
+    }
+  } else {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint4 v = __ldg(reinterpret_cast<const uint4*>(b + (16 * rt + 2 * g + h) * N + 16 * K + 4 * t));
-          u[K][4 * h] = v.x;
-          u[K][4 * h + 1] = v.y;
-          u[K][4 * h + 2] = v.z;
-          u[K][4 * h + 3] = v.w;
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint2 v = __ldg(reinterpret_cast<const uint2*>(b + (16 * K + 4 * t + q) * N + 16 * rt + 2 * g));
-          u[K][q] = v.x;
-          u[K][4 + q] = v.y;
-        }
-      }
+    for (int q = 0; q < 4; ++q) {
+      const uint2 v = __ldg(reinterpret_cast<const uint2*>(b + (16 * K + 4 * t + q) * N + 16 * rt + 2 * g));
+      u[q] = v.x;
+      u[4 + q] = v.y;
     }
   }
-};
+}
 
-// y[ct][row 2g, 2g+1: re, im] (+)= tile row times the columns of `tab`
-template <int N, bool BWD, bool ADD>
-__device__ __forceinline__ void mul_tiles(const TileRow<N, BWD>& a, uint32_t tab, int T, float (&y)[kMmaTiles][4],
-                                          float sg, int lane) {
-  float d[kMmaTiles][2][4];
+__device__ __forceinline__ uint32_t lane_row(uint32_t tab, int rs, int lane) {
+  return tab + (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * rs + ((lane >> 3) & 1) * 16);
+}
+
+// d[ct][plane] += tile times the columns' splits; the six sums of a step are independent, and each takes
+// the smallest part of the columns first
+template <int N>
+__device__ __forceinline__ void mul_tile(const uint32_t (&u)[8], uint32_t lrow, int K, int T,
+                                         float (&d)[kMmaTiles][2][4]) {
+  uint32_t re[4], im[4], b[kMmaTiles][4], c[kMmaTiles][2];
+#pragma unroll
+  for (int ct = 0; ct < kMmaTiles; ++ct)
+    if (ct < T) {
+      const uint32_t addr = lrow + ct * split_tile<N>() + K * 32;
+      asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+                   : "=r"(c[ct][0]), "=r"(c[ct][1])
+                   : "r"(addr + 16 * split_row<N>()));
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(b[ct][0]), "=r"(b[ct][1]), "=r"(b[ct][2]), "=r"(b[ct][3])
+                   : "r"(addr));
+    }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {  // rows 2g, 2g + 1 x entries 4t, 4t + 1, then 4t + 2, 4t + 3
+    const int i = 4 * (k & 1) + 2 * (k >> 1);
+    re[k] = __byte_perm(u[i], u[i + 1], 0x5410);
+    im[k] = __byte_perm(u[i], u[i + 1], 0x7632);
+  }
+#pragma unroll
+  for (int ct = 0; ct < kMmaTiles; ++ct)
+    if (ct < T) {
+      mma_bf16(d[ct][0], re, c[ct][0], c[ct][1]);
+      mma_bf16(d[ct][1], im, c[ct][0], c[ct][1]);
+    }
+#pragma unroll
+  for (int ct = 0; ct < kMmaTiles; ++ct)
+    if (ct < T) {
+      mma_bf16(d[ct][0], re, b[ct][2], b[ct][3]);
+      mma_bf16(d[ct][1], im, b[ct][2], b[ct][3]);
+    }
+#pragma unroll
+  for (int ct = 0; ct < kMmaTiles; ++ct)
+    if (ct < T) {
+      mma_bf16(d[ct][0], re, b[ct][0], b[ct][1]);
+      mma_bf16(d[ct][1], im, b[ct][0], b[ct][1]);
+    }
+}
+
+__device__ __forceinline__ void zero_sums(float (&d)[kMmaTiles][2][4]) {
 #pragma unroll
   for (int ct = 0; ct < kMmaTiles; ++ct)
 #pragma unroll
     for (int pl = 0; pl < 2; ++pl)
 #pragma unroll
       for (int k = 0; k < 4; ++k) d[ct][pl][k] = 0.f;
-  const uint32_t lrow = tab + (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * split_row<N>() + ((lane >> 3) & 1) * 16);
-#pragma unroll
-  for (int K = 0; K < N / 16; ++K) {
-    uint32_t re[4], im[4];  // rows 2g, 2g+1 x entries 4t, 4t+1, then 4t+2, 4t+3
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int i = 4 * (k & 1) + 2 * (k >> 1);
-      re[k] = __byte_perm(a.u[K][i], a.u[K][i + 1], 0x5410);
-      im[k] = __byte_perm(a.u[K][i], a.u[K][i + 1], 0x7632);
-    }
-#pragma unroll
-    for (int ct = 0; ct < kMmaTiles; ++ct) {
-      if (ct < T) {
-        uint32_t b[4], c[2];
-        const uint32_t addr = lrow + ct * split_tile<N>() + K * 32;
-        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                     : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
-                     : "r"(addr));
-        asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
-                     : "=r"(c[0]), "=r"(c[1])
-                     : "r"(addr + 16 * split_row<N>()));
-        mma_bf16(d[ct][0], re, c[0], c[1]);  // smallest part first
-        mma_bf16(d[ct][1], im, c[0], c[1]);
-        mma_bf16(d[ct][0], re, b[2], b[3]);
-        mma_bf16(d[ct][1], im, b[2], b[3]);
-        mma_bf16(d[ct][0], re, b[0], b[1]);
-        mma_bf16(d[ct][1], im, b[0], b[1]);
-      }
-    }
-  }
-#pragma unroll
-  for (int ct = 0; ct < kMmaTiles; ++ct)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {  // columns (re, im) = fragment columns 2t, 2t + 1
-      const float* r = &d[ct][0][2 * h];
-      const float* i = &d[ct][1][2 * h];
-      const float yr = BWD ? r[0] + i[1] : r[0] - i[1], yi = BWD ? r[1] - i[0] : r[1] + i[0];
-      y[ct][2 * h] = ADD ? fmaf(sg, yr, y[ct][2 * h]) : yr;
-      y[ct][2 * h + 1] = ADD ? fmaf(sg, yi, y[ct][2 * h + 1]) : yi;
-    }
 }
 
-// y to out[column][row]
-template <int N>
-__device__ __forceinline__ void put_rows(float2* out, const float (&y)[kMmaTiles][4], int rt, int R, int lane) {
+// planes -> F x (or F^H x), rows 2g, 2g + 1 of column 4 ct + t, to out[column][row] (+= sg * ... if ADD)
+template <int N, bool BWD, bool ADD>
+__device__ __forceinline__ void put_sums(const float (&d)[kMmaTiles][2][4], float2* out, int rt, int R, float sg,
+                                         int lane) {
   const int g = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int ct = 0; ct < kMmaTiles; ++ct)
-    if (4 * ct + t < R)
-      *reinterpret_cast<float4*>(out + (size_t)(4 * ct + t) * N + 16 * rt + 2 * g) =
-          make_float4(y[ct][0], y[ct][1], y[ct][2], y[ct][3]);
+    if (4 * ct + t < R) {
+      float y[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {  // columns (re, im) = fragment columns 2t, 2t + 1
+        const float* r = &d[ct][0][2 * h];
+        const float* i = &d[ct][1][2 * h];
+        y[2 * h] = BWD ? r[0] + i[1] : r[0] - i[1];
+        y[2 * h + 1] = BWD ? r[1] - i[0] : r[1] + i[0];
+      }
+      float4* o = reinterpret_cast<float4*>(out + (size_t)(4 * ct + t) * N + 16 * rt + 2 * g);
+      if (ADD) {
+        const float4 p = *o;
+        *o = make_float4(fmaf(sg, y[0], p.x), fmaf(sg, y[1], p.y), fmaf(sg, y[2], p.z), fmaf(sg, y[3], p.w));
+      } else {
+        *o = make_float4(y[0], y[1], y[2], y[3]);
+      }
+    }
+}
+
+// The warp's block (all its tile rows) times the columns of `tab`, to out; u: the tiles in flight, tile 0 and 1
+// loaded by the caller.  Two tiles are always on their way.
+template <int N, bool BWD>
+__device__ __forceinline__ void mul_block(uint32_t (&u)[3][8], const cbf16* blk, uint32_t tab, int T, float2* out, int R,
+                                          int lane) {
+  constexpr int NT = N / 16;
+  const uint32_t lrow = lane_row(tab, split_row<N>(), lane);
+  float d[kMmaTiles][2][4];
+#pragma unroll
+  for (int i = 0; i < NT * NT; ++i) {
+    if (i % NT == 0) zero_sums(d);
+    if (i + 2 < NT * NT) load_tile<N, BWD>(u[(i + 2) % 3], blk, (i + 2) / NT, (i + 2) % NT, lane);
+    mul_tile<N>(u[i % 3], lrow, i % NT, T, d);
+    if (i % NT == NT - 1)
+      // sigma3 of a backward hop's rows (a chirality boundary falls between row pairs)
+      put_sums<N, BWD, BWD>(d, out, i / NT, R, 16 * (i / NT) + 2 * (lane >> 2) < N / 2 ? 1.f : -1.f, lane);
+  }
 }
 
 template <int N>
-__global__ void __launch_bounds__(32 * kMW, 4) kb_eo_mma(BEoApply b, const int2* __restrict__ chunks) {
+__global__ void __launch_bounds__(32 * kMW, 4) kb_eo_mma(const __grid_constant__ McPhase b) {
   constexpr int NT = N / 16;
   constexpr size_t BSZ = (size_t)N * N;
   extern __shared__ __align__(16) unsigned char mc_sm[];
-  __shared__ const float2* vp[kMcCols];
-  __shared__ int act[kMcCols];
-  __shared__ int nact;
-  const int k = find_solve(b.site_off, b.count, blockIdx.x);
-  const int2 ch = chunks[k];  // first solve, columns
-  const int q = blockIdx.x - b.site_off[k];
-  const int step = *b.step;
+  __shared__ McPtrs P;
+  const McItem it = load_item(b.items + blockIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0) {
-    const bool on = lane < ch.y && bgate(b.S[ch.x + (lane < ch.y ? lane : 0)], b.gate);
-    const uint32_t m = __ballot_sync(0xffffffffu, on);
-    if (on) {
-      const int at = __popc(m & ((1u << lane) - 1u));
-      act[at] = ch.x + lane;
-      vp[at] = static_cast<const float2*>(bsel(b.S[ch.x + lane], b.vsel, step));
-    }
-    if (lane == 0) nact = __popc(m);
+  const int4 rec = __ldg(it.rec + ((size_t)b.out_par * it.nh + it.q) * 4 + warp);
+  const BSolve& s0 = b.S[it.s0];
+  const cbf16* B = static_cast<const cbf16*>(b.poly_blocks ? s0.blk_poly : s0.blk);
+  const cbf16* inv = static_cast<const cbf16*>(b.poly_blocks ? s0.inv_poly : s0.inv) + (size_t)rec.w * BSZ;
+  const cbf16* fb = B + ((size_t)rec.w * 5 + 1 + warp) * BSZ;
+  const cbf16* bb = B + ((size_t)rec.y * 5 + 1 + warp) * BSZ;
+  uint32_t u[3][8];
+  if (b.vsel != BS_NONE) {  // on their way while the columns are looked up
+    load_tile<N, false>(u[0], fb, 0, 0, lane);
+    if (NT > 1) load_tile<N, false>(u[1], fb, 0, 1, lane);
   }
-  const BSolve& s0 = b.S[ch.x];
-  const int nh = s0.V / 2;
-  const int4 rec = __ldg(s0.eo_rec + ((size_t)b.out_par * nh + q) * 4 + warp);
-  __syncthreads();
-  const int R = nact, T = (R + 3) / 4;
+  const int R = mc_setup(P, b, it), T = (R + 3) / 4;
   if (R == 0) return;
   unsigned char* tab = mc_sm + (size_t)warp * T * split_tile<N>();
   float2* hp = reinterpret_cast<float2*>(mc_sm + (size_t)kMW * T * split_tile<N>());  // [warp][column][row]
   float2* hw = hp + (size_t)warp * R * N;
   const uint32_t ta = (uint32_t)__cvta_generic_to_shared(tab);
-  const cbf16* B = static_cast<const cbf16*>(b.poly_blocks ? s0.blk_poly : s0.blk);
-  const cbf16* inv = static_cast<const cbf16*>(b.poly_blocks ? s0.inv_poly : s0.inv) + (size_t)rec.w * BSZ;
-  TileRow<N, false> fi;  // this warp's tile row of the inverse block
   if (b.vsel != BS_NONE) {
-    const cbf16* fb = B + ((size_t)rec.w * 5 + 1 + warp) * BSZ;
-    const cbf16* bb = B + ((size_t)rec.y * 5 + 1 + warp) * BSZ;
-    float y[NT][kMmaTiles][4];
-    {
-      TileRow<N, false> a, nx;
-      a.load(fb, 0, lane);
-      fill_split<N>(tab, vp, (size_t)rec.x * N, R, false, lane);
-      __syncwarp();
-#pragma unroll
-      for (int rt = 0; rt < NT; ++rt) {
-        if (rt + 1 < NT) nx.load(fb, rt + 1, lane);
-        mul_tiles<N, false, false>(a, ta, T, y[rt], 1.f, lane);
-        a = nx;
-      }
-    }
-    TileRow<N, true> a, nx;
-    a.load(bb, 0, lane);
+    fill_split<N>(tab, P.v, (size_t)rec.x * N, R, false, lane);
     __syncwarp();
-    fill_split<N>(tab, vp, (size_t)rec.z * N, R, true, lane);
+    mul_block<N, false>(u, fb, ta, T, hw, R, lane);
+    load_tile<N, true>(u[0], bb, 0, 0, lane);
+    if (NT > 1) load_tile<N, true>(u[1], bb, 0, 1, lane);
     __syncwarp();
-#pragma unroll
-    for (int rt = 0; rt < NT; ++rt) {
-      if (rt + 1 < NT) nx.load(bb, rt + 1, lane);
-      else if (warp < NT) fi.load(inv, warp, lane);
-      // sigma3 of the result's rows (a chirality boundary falls between row pairs)
-      mul_tiles<N, true, true>(a, ta, T, y[rt], 16 * rt + 2 * (lane >> 2) < N / 2 ? 1.f : -1.f, lane);
-      put_rows<N>(hw, y[rt], rt, R, lane);
-      a = nx;
-    }
-    __syncthreads();
-  } else if (warp < NT) {
-    fi.load(inv, warp, lane);
+    fill_split<N>(tab, P.v, (size_t)rec.z * N, R, true, lane);
+    __syncwarp();
+    mul_block<N, true>(u, bb, ta, T, hw, R, lane);
   }
+  if (warp < NT)  // this warp's tile row of the inverse block
+#pragma unroll
+    for (int K = 0; K < NT; ++K) load_tile<N, false>(u[K], inv, warp, K, lane);
+  __syncthreads();
   // g = z - h (or h): the operand of the inverse block, shared by the warps
-  const size_t off = (size_t)q * N;
+  const size_t off = (size_t)it.q * N;
   for (int i = threadIdx.x; i < R * (N / 4); i += blockDim.x) {
     const int c = i / (N / 4), j = 4 * (i % (N / 4));
     float2 v[4];
@@ -589,8 +627,7 @@ __global__ void __launch_bounds__(32 * kMW, 4) kb_eo_mma(BEoApply b, const int2*
         v[3] = cadd(v[3], make_float2(h1.z, h1.w));
       }
     if (b.zsel != BS_NONE) {
-      const float4* z = reinterpret_cast<const float4*>(
-          static_cast<const float2*>(bsel(b.S[act[c]], b.zsel, step)) + off + j);
+      const float4* z = reinterpret_cast<const float4*>(P.z[c] + off + j);
       const float4 z0 = z[0], z1 = z[1];
       v[0] = csub(make_float2(z0.x, z0.y), v[0]);
       v[1] = csub(make_float2(z0.z, z0.w), v[1]);
@@ -601,21 +638,23 @@ __global__ void __launch_bounds__(32 * kMW, 4) kb_eo_mma(BEoApply b, const int2*
   }
   __syncthreads();
   if (warp < NT) {
-    float y[kMmaTiles][4];
-    mul_tiles<N, false, false>(fi, (uint32_t)__cvta_generic_to_shared(mc_sm), T, y, 1.f, lane);
-    put_rows<N>(hp, y, warp, R, lane);
+    const uint32_t lrow = lane_row((uint32_t)__cvta_generic_to_shared(mc_sm), split_row<N>(), lane);
+    float d[kMmaTiles][2][4];
+    zero_sums(d);
+#pragma unroll
+    for (int K = 0; K < NT; ++K) mul_tile<N>(u[K], lrow, K, T, d);
+    put_sums<N, false, false>(d, hp, warp, R, 1.f, lane);
   }
   __syncthreads();
   for (int i = threadIdx.x; i < R * N; i += blockDim.x) {
-    const BSolve& S = b.S[act[i / N]];
+    const int c = i / N;
     const size_t idx = off + i % N;
     float2 r = hp[i], xs = make_float2(0.f, 0.f);
     if (b.bsel != BS_NONE) {
-      xs = static_cast<const float2*>(bsel(S, b.bsel, step))[idx];
+      xs = P.base[c][idx];
       r = csub(xs, r);
     }
-    mc_finish(b.mode, r, xs, S.polyc + b.coef_off, static_cast<float2*>(bsel(S, b.ysel, step)) + idx,
-              static_cast<float2*>(S.acc) + idx);
+    mc_finish(b.mode, r, xs, P.coef[c], P.y[c] + idx, P.acc[c] + idx);
   }
 }
 
@@ -647,44 +686,28 @@ __device__ __forceinline__ float2 mc_full_sum(const float* hp, int i, int R, flo
 
 // Batched full stencil over (operator's column chunk, site).
 template <int N, class BT>
-__global__ void __launch_bounds__(32 * kMW) kb_apply_mc(BApply b, const int2* __restrict__ chunks) {
+__global__ void __launch_bounds__(32 * kMW) kb_apply_mc(const __grid_constant__ McPhase b) {
   extern __shared__ __align__(16) unsigned char mc_sm[];
-  __shared__ const float2* vp[kMcCols];
-  __shared__ int act[kMcCols];
-  __shared__ int nact;
-  const int k = find_solve(b.site_off, b.count, blockIdx.x);
-  const int2 ch = chunks[k];
-  const int step = *b.step;
+  __shared__ McPtrs P;
+  const McItem it = load_item(b.items + blockIdx.x);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0) {
-    const bool on = lane < ch.y && bgate(b.S[ch.x + (lane < ch.y ? lane : 0)], b.gate);
-    const uint32_t m = __ballot_sync(0xffffffffu, on);
-    if (on) {
-      const int at = __popc(m & ((1u << lane) - 1u));
-      act[at] = ch.x + lane;
-      vp[at] = static_cast<const float2*>(bsel(b.S[ch.x + lane], b.xsel, step));
-    }
-    if (lane == 0) nact = __popc(m);
-  }
-  __syncthreads();
-  const int R = nact;
+  const BSolve& s0 = b.S[it.s0];
+  const int R = mc_setup(P, b, it);
   if (R == 0) return;
-  const BSolve& s0 = b.S[ch.x];
   McSite s;
   s.blocks = b.poly_blocks ? s0.blk_poly : s0.blk;
-  s.x = blockIdx.x - b.site_off[k];
+  s.x = it.q;
   s.R = R;
   s.adj = 0;
   float2* tabs = reinterpret_cast<float2*>(mc_sm);
   float* hp = reinterpret_cast<float*>(tabs + (size_t)2 * kMW * R * N);
-  mc_full_site<N, BT>(s, s0.nb, vp, tabs, hp, warp, lane);
+  mc_full_site<N, BT>(s, s0.nb, P.v, tabs, hp, warp, lane);
   for (int i = threadIdx.x; i < R * N; i += blockDim.x) {
-    const BSolve& S = b.S[act[i / N]];
+    const int c = i / N;
     const size_t idx = (size_t)s.x * N + i % N;
-    const float2 xs = vp[i / N][idx];
-    const float2 r = mc_full_sum<N>(hp, i, R, (float)S.mu, xs, i % N);
-    mc_finish(b.mode, r, xs, S.polyc + b.coef_off, static_cast<float2*>(bsel(S, b.ysel, step)) + idx,
-              static_cast<float2*>(S.acc) + idx);
+    const float2 xs = P.v[c][idx];
+    const float2 r = mc_full_sum<N>(hp, i, R, P.mu[c], xs, i % N);
+    mc_finish(b.mode, r, xs, P.coef[c], P.y[c] + idx, P.acc[c] + idx);
   }
 }
 
@@ -718,7 +741,7 @@ int mc_attr(K kernel, size_t bytes) {
 }
 
 template <int N>
-int launch_beo_mc_n(bool bf, const BEoApply& b, const int2* chunks, int rmax, cudaStream_t s) {
+int launch_beo_mc_n(bool bf, const McPhase& b, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
     int rc = mc_attr(kb_eo_mc<N, float2>, mc_smem<N>(kMcCols));
@@ -726,22 +749,22 @@ int launch_beo_mc_n(bool bf, const BEoApply& b, const int2* chunks, int rmax, cu
     if (rc != COARSE_OK) return rc;
     attr = true;
   }
-  if (bf) kb_eo_mma<N><<<b.total, 32 * kMW, mma_smem<N>(rmax), s>>>(b, chunks);
-  else kb_eo_mc<N, float2><<<b.total, 32 * kMW, mc_smem<N>(rmax), s>>>(b, chunks);
+  if (bf) kb_eo_mma<N><<<b.count, 32 * kMW, mma_smem<N>(b.rmax), s>>>(b);
+  else kb_eo_mc<N, float2><<<b.count, 32 * kMW, mc_smem<N>(b.rmax), s>>>(b);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   return COARSE_OK;
 }
 
 template <int N, class BT>
-int launch_bapply_mc_n(const BApply& b, const int2* chunks, int rmax, cudaStream_t s) {
+int launch_bapply_mc_n(const McPhase& b, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
     const int rc = mc_attr(kb_apply_mc<N, BT>, mc_smem<N>(kMcCols));
     if (rc != COARSE_OK) return rc;
     attr = true;
   }
-  kb_apply_mc<N, BT><<<b.total, 32 * kMW, mc_smem<N>(rmax), s>>>(b, chunks);
+  kb_apply_mc<N, BT><<<b.count, 32 * kMW, mc_smem<N>(b.rmax), s>>>(b);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   return COARSE_OK;
@@ -763,25 +786,25 @@ int launch_apply_mc_n(const ApplyArgs& a, int R, long long ldc, cudaStream_t s) 
 
 }  // namespace
 
-int launch_beo_mc(int prec, int n, const BEoApply& b, const int2* chunks, int rmax, cudaStream_t s) {
-  if (b.total <= 0) return COARSE_OK;
+int launch_beo_mc(int prec, int n, const McPhase& b, cudaStream_t s) {
+  if (b.count <= 0) return COARSE_OK;
   const bool bf = prec == COARSE_PREC_BF16;
   switch (n) {
-    case 16: return launch_beo_mc_n<16>(bf, b, chunks, rmax, s);
-    case 32: return launch_beo_mc_n<32>(bf, b, chunks, rmax, s);
-    case 48: return launch_beo_mc_n<48>(bf, b, chunks, rmax, s);
+    case 16: return launch_beo_mc_n<16>(bf, b, s);
+    case 32: return launch_beo_mc_n<32>(bf, b, s);
+    case 48: return launch_beo_mc_n<48>(bf, b, s);
   }
   set_error("batched half apply: unsupported n = %d", n);
   return COARSE_ERR_INVALID_ARG;
 }
 
-int launch_bapply_mc(int prec, int n, const BApply& b, const int2* chunks, int rmax, cudaStream_t s) {
-  if (b.total <= 0) return COARSE_OK;
+int launch_bapply_mc(int prec, int n, const McPhase& b, cudaStream_t s) {
+  if (b.count <= 0) return COARSE_OK;
   const bool bf = prec == COARSE_PREC_BF16;
   switch (n) {
-    case 16: return bf ? launch_bapply_mc_n<16, cbf16>(b, chunks, rmax, s) : launch_bapply_mc_n<16, float2>(b, chunks, rmax, s);
-    case 32: return bf ? launch_bapply_mc_n<32, cbf16>(b, chunks, rmax, s) : launch_bapply_mc_n<32, float2>(b, chunks, rmax, s);
-    case 48: return bf ? launch_bapply_mc_n<48, cbf16>(b, chunks, rmax, s) : launch_bapply_mc_n<48, float2>(b, chunks, rmax, s);
+    case 16: return bf ? launch_bapply_mc_n<16, cbf16>(b, s) : launch_bapply_mc_n<16, float2>(b, s);
+    case 32: return bf ? launch_bapply_mc_n<32, cbf16>(b, s) : launch_bapply_mc_n<32, float2>(b, s);
+    case 48: return bf ? launch_bapply_mc_n<48, cbf16>(b, s) : launch_bapply_mc_n<48, float2>(b, s);
   }
   set_error("batched apply: unsupported n = %d", n);
   return COARSE_ERR_INVALID_ARG;

@@ -12,9 +12,8 @@ constexpr int kMcCols = 12;  // columns of one pass (shared memory holds their v
 // epilogue; x 16-byte aligned, ldc even.
 int launch_apply_mc(int n, const ApplyArgs& a, int R, long long ldc, cudaStream_t s);
 
-// The batched phases over column chunks: b.site_off are prefix sums over the chunks of one n-group, chunk k
-// covers the solves chunks[k].x .. + chunks[k].y - 1 of one operator; rmax: largest chunk of the group.
-int launch_beo_mc(int prec, int n, const BEoApply& b, const int2* chunks, int rmax, cudaStream_t s);
-int launch_bapply_mc(int prec, int n, const BApply& b, const int2* chunks, int rmax, cudaStream_t s);
+// The batched phases (half apply, full stencil) over the items of one n-group.
+int launch_beo_mc(int prec, int n, const McPhase& p, cudaStream_t s);
+int launch_bapply_mc(int prec, int n, const McPhase& p, cudaStream_t s);
 
 }  // namespace coarse

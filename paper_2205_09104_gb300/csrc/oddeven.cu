@@ -362,34 +362,6 @@ __global__ void __launch_bounds__(32 * W, eo_min_blocks<N, AC, W, PF>()) k_eo_ha
   eo_half_site<N, BT, VT, AC, W, UNROLL, PF>(a, blockIdx.x);
 }
 
-// Batched half apply: CTA g of the flat grid takes output site g of the n-group (half-site prefix
-// sums give its solve), builds that solve's arguments and runs the two-warp unrolled layout.
-template <int N, class BT>
-__global__ void __launch_bounds__(64) kb_eo_half(BEoApply b) {
-  const int g = blockIdx.x;
-  if (g >= b.total) return;
-  const int k = find_solve(b.site_off, b.count, g);
-  const BSolve& s = b.S[b.sidx[k]];
-  if (!bgate(s, b.gate)) return;  // uniform for all sites of the solve
-  const int step = *b.step;
-  EoArgs a{};
-  a.blocks = b.poly_blocks ? s.blk_poly : s.blk;
-  a.inv = b.poly_blocks ? s.inv_poly : s.inv;
-  a.rec = s.eo_rec;
-  a.err = s.cnt + s.V;
-  a.V = s.V;
-  a.out_par = b.out_par;
-  a.v = bsel(s, b.vsel, step);
-  a.z = bsel(s, b.zsel, step);
-  a.base = bsel(s, b.bsel, step);
-  a.y = bsel(s, b.ysel, step);
-  a.mode = b.mode;
-  a.acc = s.acc;
-  a.coef = s.polyc + b.coef_off;
-  a.stop = nullptr;
-  eo_half_site<N, BT, float2, float2, 2, true, false>(a, g - b.site_off[k]);
-}
-
 // Warp-per-site variant (4 sites per CTA): one warp walks all 9 blocks of its site.
 template <int N, class BT, class VT, class AC>
 __global__ void __launch_bounds__(128) k_eo_half_w(EoArgs a) {
@@ -1120,23 +1092,6 @@ int launch_eo_merge(int v64, const void* ev, const void* od, const int* sites, i
 
 // y = S x on compressed even vectors (t: odd scratch of the vector type), with an optional
 // polynomial-chain epilogue (mode, acc, coef) as the full stencil's.
-int launch_beo_half(int prec, int n, const BEoApply& b, cudaStream_t s) {
-  if (b.total <= 0) return COARSE_OK;
-  const dim3 grid(b.total);
-#define BEO(NN)                                                                              \
-  if (prec == COARSE_PREC_BF16) kb_eo_half<NN, cbf16><<<grid, 64, 0, s>>>(b);                \
-  else kb_eo_half<NN, float2><<<grid, 64, 0, s>>>(b);
-  switch (n) {
-    case 16: BEO(16) break;
-    case 32: BEO(32) break;
-    case 48: BEO(48) break;
-    default: set_error("batched odd-even: unsupported n = %d", n); return COARSE_ERR_INVALID_ARG;
-  }
-#undef BEO
-  note_launch();
-  COARSE_CUDA(cudaGetLastError());
-  return COARSE_OK;
-}
 
 int launch_eo_schur(const coarse_op* op, int prec, double mu_eff, const void* x, void* y, void* t, int mode, void* acc,
                     const double2* coef, const int* stop, cudaStream_t s) {
