@@ -17,6 +17,7 @@
 
 #include "batch.cuh"
 #include "common.cuh"
+#include "digits.cuh"
 #include "mcol.cuh"
 #include "mrhs_core.cuh"
 #include "oddeven.cuh"
@@ -47,6 +48,13 @@ struct Group {
 struct CGroup {
   int n = 0;
   McPhase p{};  // items and per-solve arrays; phase fields filled per launch
+};
+
+// n-group of the FP64 residual through the digit operands (digits.cuh)
+struct DGroup {
+  int n = 0, sites = 0;
+  const DigPass* passes = nullptr;
+  const int* map = nullptr;
 };
 
 // n-group of the multi-RHS stencil phases
@@ -87,7 +95,8 @@ struct Batch {
   int* chunk_off_f = nullptr;
   int total_chunks_f = 0;
   std::vector<CGroup> cgroups;  // stencil phases (half-site counts with the odd-even reduction)
-  std::vector<Group> groups;
+  std::vector<Group> groups;    // FP64 residual on the FP64 pipe, n-groups with an operator without digits
+  std::vector<DGroup> dgroups;  // ... through the digit operands
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   long long launches = 0;
@@ -203,6 +212,9 @@ struct Batch {
   }
 
   int residual64(cudaStream_t s) {
+    // {-1, +1} for r = -D x + b lies right after the step counter
+    for (const DGroup& g : dgroups)
+      TRY(launch_bresidual_digits(g.n, g.passes, g.map, g.sites, flags, reinterpret_cast<const double2*>(step + 4), s));
     for (const Group& g : groups) {
       BApply a;
       a.S = dS;
@@ -219,6 +231,11 @@ struct Batch {
 };
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+
+// FP64 stencil scratch of one solve: pull partials and pushes, or the digit operands of one pass
+size_t part64_bytes(int n, int V) {
+  return align256(std::max(5 * sizeof(double2) * (size_t)V * n, dig_x_bytes(n, V, kDigCols)));
+}
 
 // ---- device-side control of the whole batched solve (refinement steps, cycles, Arnoldi steps)
 //
@@ -525,6 +542,14 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
   const size_t o_coff = take(sizeof(int) * (ns + 1));
   const size_t o_coff_f = take(sizeof(int) * (ns + 1));
   const size_t o_groups = take(sizeof(int) * (2 * ns + 8) * 3);
+  size_t n_dpass = 0, n_dmap = 0;
+  for (int i = 0; i < nops; ++i) {
+    const size_t passes = (nrhs[i] + kDigCols - 1) / kDigCols;
+    n_dpass += passes;
+    n_dmap += passes * ((ops[i]->V + kDigMapSites - 1) / kDigMapSites);
+  }
+  const size_t o_dpass = take(sizeof(DigPass) * n_dpass);
+  const size_t o_dmap = take(sizeof(int) * n_dmap);
   const size_t o_vbase = take(sizeof(char*) * ns);
   size_t n_items = 0;  // sites of all column chunks
   for (int i = 0; i < nops; ++i)
@@ -566,7 +591,7 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
         chunk_off[sidx + 1] = chunk_off[sidx] + nch[sidx];
         chunk_off_f[sidx + 1] = chunk_off_f[sidx] + nchf[sidx];
         off_vec[sidx] = take(sizeof(float2) * (size_t)N * (m + 7) + sizeof(float2) * 5 * (size_t)N +
-                             sizeof(double2) * 6 * (size_t)N + sizeof(int) * (V + 4) + 1024);
+                             sizeof(double2) * (size_t)N + part64_bytes(ops[i]->n, V) + sizeof(int) * (V + 4) + 1024);
         off_small[sidx] = take(sizeof(double2) * (2 * (size_t)ldh * kMaxDense + 3 * kMaxDense + (size_t)kMaxK * kMaxDense +
                                                   4 * maxq + 3 * kMaxPoly + 4) +
                                sizeof(double) * 2 * (size_t)kBatchMaxQ * nchf[sidx] + sizeof(void*) * (3 * (kc + m + 2)) +
@@ -665,7 +690,7 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
         char* v64 = v + (m + 12) * vb;
         S.r64 = reinterpret_cast<double2*>(v64);
         S.part64 = v64 + sizeof(double2) * (size_t)N;
-        S.cnt = reinterpret_cast<int*>(v64 + sizeof(double2) * 6 * (size_t)N);
+        S.cnt = reinterpret_cast<int*>(v64 + sizeof(double2) * (size_t)N + part64_bytes(S.n, S.V));
         S.b64 = static_cast<const double2*>(b[i]) + (size_t)c * N;
         S.x64 = static_cast<double2*>(x[i]) + (size_t)c * N;
         // small dense state
@@ -782,7 +807,10 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
     COARSE_CUDA(cudaMemcpyAsync(B.mem + o_mgrp, mgroup_tab.data(), sizeof(int) * mgroup_tab.size(),
                                 cudaMemcpyHostToDevice, s));
   }
-  // n-groups of the stencil phases
+  // n-groups of the FP64 residual
+  std::vector<DigPass> dpasses[3];
+  std::vector<int> dmaps[3];
+  size_t dpass_at = 0, dmap_at = 0;
   {
     int* g0 = reinterpret_cast<int*>(B.mem + o_groups);
     for (int n : {16, 32, 48}) {
@@ -793,6 +821,51 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
           off.push_back(off.back() + hs[q].V);
         }
       if (idx.empty()) continue;
+      bool digits = true;
+      for (int i = 0; i < nops; ++i) digits = digits && (ops[i]->n != n || ops[i]->dig);
+      if (digits) {
+        std::vector<DigPass>& dp = dpasses[n / 16 - 1];
+        std::vector<int>& map = dmaps[n / 16 - 1];
+        int s0 = 0;
+        for (int i = 0; i < nops; ++i) {
+          const size_t N = (size_t)ops[i]->V * n;
+          for (int c = 0; ops[i]->n == n && c < nrhs[i]; c += kDigCols) {
+            const BSolve& S = hs[s0 + c];
+            DigPass d{};
+            d.x = S.x64;
+            d.z = S.b64;
+            d.y = S.r64;
+            d.ldx = N;
+            d.cols = std::min(kDigCols, nrhs[i] - c);
+            d.ldy = d.cols > 1 ? (size_t)(hs[s0 + c + 1].r64 - S.r64) : 0;  // equal records of one operator's solves
+            d.dig = ops[i]->dig;
+            d.digscale = ops[i]->digscale;
+            d.digx = S.part64;
+            d.blocks = S.blk64;
+            d.nb = S.nb;
+            d.mu = S.mu;
+            d.V = S.V;
+            d.start = (int)map.size() * kDigMapSites;
+            d.q0 = s0 + c;
+            map.insert(map.end(), (S.V + kDigMapSites - 1) / kDigMapSites, (int)dp.size());
+            dp.push_back(d);
+          }
+          s0 += nrhs[i];
+        }
+        DGroup g;
+        g.n = n;
+        g.sites = (int)map.size() * kDigMapSites;
+        DigPass* pd = reinterpret_cast<DigPass*>(B.mem + o_dpass) + dpass_at;
+        int* pm = reinterpret_cast<int*>(B.mem + o_dmap) + dmap_at;
+        COARSE_CUDA(cudaMemcpyAsync(pd, dp.data(), sizeof(DigPass) * dp.size(), cudaMemcpyHostToDevice, s));
+        COARSE_CUDA(cudaMemcpyAsync(pm, map.data(), sizeof(int) * map.size(), cudaMemcpyHostToDevice, s));
+        g.passes = pd;
+        g.map = pm;
+        dpass_at += dp.size();
+        dmap_at += map.size();
+        B.dgroups.push_back(g);
+        continue;
+      }
       Group g;
       g.n = n;
       g.count = (int)idx.size();

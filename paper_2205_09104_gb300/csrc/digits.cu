@@ -130,17 +130,11 @@ __global__ void __launch_bounds__(256) k_dig_blocks(const double2* __restrict__ 
   }
 }
 
-// One warp per (column, site): digits, corrections and scale of the site vector.
+// Digits, corrections and scale of one site vector, by one warp (dg: 16 N shorts of its own).
 template <int N>
-__global__ void __launch_bounds__(128) k_dig_x(const double2* __restrict__ x, long long ldc, int V,
-                                               __half* __restrict__ xd, float* __restrict__ xc,
-                                               double* __restrict__ xs, const int* stop) {
-  if (stop != nullptr && *stop) return;
-  __shared__ short dg[4][16][N];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int site = blockIdx.x * 4 + warp, col = blockIdx.y;
-  if (site >= V) return;  // warp-uniform
-  const double2* p = x + col * ldc + (size_t)site * N;
+__device__ __forceinline__ void dig_x_site(const double2* __restrict__ p, size_t rec, short (*dg)[N],
+                                           __half* __restrict__ xd, float* __restrict__ xc, double* __restrict__ xs) {
+  const int lane = threadIdx.x & 31;
   constexpr int PER = (N + 31) / 32;
   double2 v[PER];
   uint32_t m[2] = {0u, 0u};  // largest high word of each chirality half
@@ -162,7 +156,6 @@ __global__ void __launch_bounds__(128) k_dig_x(const double2* __restrict__ x, lo
   bool ok = (scale_of(mx, ex) || !any) && high_finite(mx);
   if (mn != 0u && (int)(mn >> 20) + kRange < ex) ok = false;
   if (!ok) ex = 4096;  // every entry below the last digit
-  const size_t rec = (size_t)col * V + site;
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
     const int i = lane + 32 * k;
@@ -170,8 +163,8 @@ __global__ void __launch_bounds__(128) k_dig_x(const double2* __restrict__ x, lo
       const unsigned long long dx = digits_of(v[k].x, ex), dy = digits_of(v[k].y, ex);
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        dg[warp][q][i] = (short)((int)((dx >> (56 - 8 * q)) & 255ull) - 128);
-        dg[warp][8 + q][i] = (short)((int)((dy >> (56 - 8 * q)) & 255ull) - 128);
+        dg[q][i] = (short)((int)((dx >> (56 - 8 * q)) & 255ull) - 128);
+        dg[8 + q][i] = (short)((int)((dy >> (56 - 8 * q)) & 255ull) - 128);
       }
     }
   }
@@ -179,13 +172,13 @@ __global__ void __launch_bounds__(128) k_dig_x(const double2* __restrict__ x, lo
   __half2* o = reinterpret_cast<__half2*>(xd + rec * dig_x_halves(N));
   for (int w = lane; w < 8 * N; w += 32) {
     const int row = w / (N / 2), c = 2 * (w % (N / 2));
-    o[w] = __floats2half2_rn((float)dg[warp][row][c], (float)dg[warp][row][c + 1]);
+    o[w] = __floats2half2_rn((float)dg[row][c], (float)dg[row][c + 1]);
   }
   // lane = (half, part, digit): sums over the half, then the corrections of the two sigma3 variants
   int sum = 0;
   {
     const int row = lane & 15, h = lane >> 4;
-    for (int i = 0; i < N / 2; ++i) sum += dg[warp][row][h * (N / 2) + i];
+    for (int i = 0; i < N / 2; ++i) sum += dg[row][h * (N / 2) + i];
   }
   const int lo = __shfl_sync(0xffffffffu, sum, lane & 15), hi = __shfl_sync(0xffffffffu, sum, 16 + (lane & 15));
   int t = lane < 16 ? lo + hi : lo - hi;  // lane = (variant, part, digit)
@@ -196,6 +189,52 @@ __global__ void __launch_bounds__(128) k_dig_x(const double2* __restrict__ x, lo
   }
   xc[rec * kDigCorr + lane] = (float)t * -0x1p-17f;  // -128 * 2^-24
   if (lane == 0) xs[rec] = ok ? (any ? scale_value(ex) : 0.0) : scale_special();
+}
+
+template <int N>
+__global__ void __launch_bounds__(128) k_dig_x(const double2* __restrict__ x, long long ldc, int V,
+                                               __half* __restrict__ xd, float* __restrict__ xc,
+                                               double* __restrict__ xs, const int* stop) {
+  if (stop != nullptr && *stop) return;
+  __shared__ short dg[4][16][N];
+  const int warp = threadIdx.x >> 5, site = blockIdx.x * 4 + warp, col = blockIdx.y;
+  if (site >= V) return;  // warp-uniform
+  dig_x_site<N>(x + col * ldc + (size_t)site * N, (size_t)col * V + site, dg[warp], xd, xc, xs);
+}
+
+// The column operands of one pass in `mem` (dig_x_bytes).
+struct DigX {
+  __half* xd;
+  float* xc;
+  double* xs;
+};
+template <int N>
+__host__ __device__ __forceinline__ DigX dig_x_at(void* mem, int V, int cols) {
+  char* m = static_cast<char*>(mem);
+  DigX d;
+  d.xd = reinterpret_cast<__half*>(m);
+  m += (size_t)cols * V * dig_x_halves(N) * sizeof(__half);
+  d.xc = reinterpret_cast<float*>(m);
+  m += (size_t)cols * V * kDigCorr * sizeof(float);
+  d.xs = reinterpret_cast<double*>(m);
+  return d;
+}
+
+// Batched column pack: warp w of the launch takes site w - start of the pass found through the map.
+template <int N>
+__global__ void __launch_bounds__(128) kb_dig_x(const DigPass* __restrict__ passes, const int* __restrict__ map,
+                                                const int* __restrict__ flags) {
+  __shared__ short dg[4][16][N];
+  const int warp = threadIdx.x >> 5, w = blockIdx.x * 4 + warp;
+  const DigPass& p = passes[__ldg(map + w / kDigMapSites)];
+  const int site = w - p.start;
+  if (site >= p.V) return;  // warp-uniform
+  const DigX d = dig_x_at<N>(p.digx, p.V, p.cols);
+  if (flags[2 * p.q0 + 1] && flags[2 * (p.q0 + p.cols - 1) + 1]) return;  // every column of the pass is done
+  for (int c = 0; c < p.cols; ++c) {
+    dig_x_site<N>(p.x + (size_t)c * p.ldx + (size_t)site * N, (size_t)c * p.V + site, dg[warp], d.xd, d.xc, d.xs);
+    __syncwarp();
+  }
 }
 
 // -------------------------------------------------------------------------------------- the stencil
@@ -376,17 +415,16 @@ __device__ __noinline__ void dig_plain(const ApplyArgs& a, const int* ublk, cons
   }
 }
 
+// One site of the columns x + c ldx (c < ncol <= C), results y + c ldy, addend z + c ldz (AXPBY).
 template <int N, int C>
-__global__ void __launch_bounds__(32 * kDW, C > 1 ? 1 : (N == 16 ? 3 : 2)) k_apply_digits(const __grid_constant__ ApplyArgs a,
-                                                                           const __grid_constant__ DigArgs dgt, int ncol,
-                                                                           long long ldc) {
+__device__ __forceinline__ void dig_site(const ApplyArgs& a, const DigArgs& dgt, const int site, const int ncol,
+                                         const size_t ldx, const size_t ldy, const size_t ldz) {
   constexpr int NT = N / 16, RS = dig_row<N>(), PS = dig_part<N>(), SL = dig_slab<N>();
   extern __shared__ __align__(16) unsigned char dsm[];  // [kDW][C] digit tables, then [kDW][C][2N] sums
   static_assert(SL >= 2 * N * 8, "the sums take the place of the digit tables");
   __shared__ int ublk[9], usrc[9];
-  if (a.stop != nullptr && *a.stop) return;
   const int u = threadIdx.x >> 5, lane = threadIdx.x & 31;  // warp u: block product u
-  const int site = blockIdx.x, V = a.V;
+  const int V = a.V;
   const int nc = ncol < C ? ncol : C;
   const int src = u == 0 ? site : __ldg(a.nb + site * 8 + (u - 1));
   const int blk = u < 5 ? site * 5 + u : src * 5 + 1 + (u - 5);
@@ -450,7 +488,7 @@ __global__ void __launch_bounds__(32 * kDW, C > 1 ? 1 : (N == 16 ? 3 : 2)) k_app
       for (int c = 0; c < C; ++c) part[(u * C + c) * 2 * N + 2 * (16 * O + g + 8 * (t & 1)) + (t >> 1)] = acc[O][c];
   } else {
     for (int c = 0; c < nc; ++c)
-      dig_plain<N>(a, ublk, usrc, static_cast<const double2*>(a.x) + (size_t)c * ldc, part + c * 2 * N);
+      dig_plain<N>(a, ublk, usrc, static_cast<const double2*>(a.x) + (size_t)c * ldx, part + c * 2 * N);
   }
   __syncthreads();
   const double2 c0 = a.mode != APPLY_PLAIN ? a.coef[0] : make_double2(0.0, 0.0);
@@ -458,31 +496,67 @@ __global__ void __launch_bounds__(32 * kDW, C > 1 ? 1 : (N == 16 ? 3 : 2)) k_app
   const double2 c2 = a.mode == APPLY_POLY_FIRST ? a.coef[2] : make_double2(0.0, 0.0);
   for (int i = threadIdx.x; i < nc * N; i += blockDim.x) {
     const int c = i / N, e = i % N;
-    const size_t idx = (size_t)c * ldc + (size_t)site * N + e;
-    const double2* X = static_cast<const double2*>(a.x);
+    const size_t idx = (size_t)site * N + e;
     const double* pc = part + c * 2 * N + 2 * e;
     double2 r = make_double2(pc[0], pc[1]);
     if (!bad)
 #pragma unroll
       for (int w = 1; w < kDW; ++w) r = cadd(r, make_double2(pc[w * C * 2 * N], pc[w * C * 2 * N + 1]));
-    const double2 xs = X[idx];
+    const double2 xs = static_cast<const double2*>(a.x)[c * ldx + idx];
     const double m = e < N / 2 ? a.mu : -a.mu;  // + i mu sigma3 x
     r.x -= m * xs.y;
     r.y += m * xs.x;
-    double2* y = static_cast<double2*>(a.y) + idx;
+    double2* y = static_cast<double2*>(a.y) + c * ldy + idx;
     if (a.mode == APPLY_PLAIN) {
       *y = r;
     } else if (a.mode == APPLY_AXPBY) {
-      *y = cadd(cmul(c0, r), cmul(c1, static_cast<const double2*>(a.z)[idx]));
+      *y = cadd(cmul(c0, r), cmul(c1, static_cast<const double2*>(a.z)[c * ldz + idx]));
     } else {
       // chain step: s' = s - c0 D s ; acc = acc + c1 s'  (first: acc = c2 s + c1 s')
-      double2* accp = static_cast<double2*>(a.acc) + idx;
+      double2* accp = static_cast<double2*>(a.acc) + c * ldy + idx;
       const double2 ac = a.mode == APPLY_POLY_FIRST ? cmul(c2, xs) : *accp;
       r = csub(xs, cmul(c0, r));
       *y = r;
       *accp = cadd(ac, cmul(c1, r));
     }
   }
+}
+
+template <int N, int C>
+__global__ void __launch_bounds__(32 * kDW, C > 1 ? 1 : (N == 16 ? 3 : 2)) k_apply_digits(
+    const __grid_constant__ ApplyArgs a, const __grid_constant__ DigArgs dgt, int ncol, long long ldc) {
+  if (a.stop != nullptr && *a.stop) return;
+  dig_site<N, C>(a, dgt, blockIdx.x, ncol, ldc, ldc, ldc);
+}
+
+// Batched FP64 residual r = b - D x of every pass with an unfinished column (coef: {-1, +1}).
+template <int N>
+__global__ void __launch_bounds__(32 * kDW, 1) kb_residual_digits(const DigPass* __restrict__ passes,
+                                                                  const int* __restrict__ map,
+                                                                  const int* __restrict__ flags,
+                                                                  const double2* coef) {
+  const DigPass& p = passes[__ldg(map + blockIdx.x / kDigMapSites)];
+  const int site = blockIdx.x - p.start;
+  if (site >= p.V) return;
+  if (flags[2 * p.q0 + 1] && flags[2 * (p.q0 + p.cols - 1) + 1]) return;
+  const DigX dx = dig_x_at<N>(p.digx, p.V, p.cols);
+  DigArgs d;
+  d.dig = static_cast<const uint4*>(p.dig);
+  d.bscale = p.digscale;
+  d.xd = dx.xd;
+  d.xc = dx.xc;
+  d.xs = dx.xs;
+  ApplyArgs a{};
+  a.blocks = p.blocks;
+  a.nb = p.nb;
+  a.x = p.x;
+  a.y = p.y;
+  a.z = p.z;
+  a.coef = coef;
+  a.mu = p.mu;
+  a.V = p.V;
+  a.mode = APPLY_AXPBY;
+  dig_site<N, kDigCols>(a, d, site, p.cols, p.ldx, p.ldy, p.ldx);
 }
 
 template <int N, int C>
@@ -506,22 +580,35 @@ int launch_dig_n(const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {
   DigArgs d;
   d.dig = static_cast<const uint4*>(a.dig);
   d.bscale = a.digscale;
-  char* m = static_cast<char*>(a.digx);
-  __half* xd = reinterpret_cast<__half*>(m);
-  m += (size_t)ncol * a.V * dig_x_halves(N) * sizeof(__half);
-  float* xc = reinterpret_cast<float*>(m);
-  m += (size_t)ncol * a.V * kDigCorr * sizeof(float);
-  double* xs = reinterpret_cast<double*>(m);
-  d.xd = xd;
-  d.xc = xc;
-  d.xs = xs;
-  k_dig_x<N><<<dim3((a.V + 3) / 4, ncol), 128, 0, s>>>(static_cast<const double2*>(a.x), ldc, a.V, xd, xc, xs, a.stop);
+  const DigX x = dig_x_at<N>(a.digx, a.V, ncol);
+  d.xd = x.xd;
+  d.xc = x.xc;
+  d.xs = x.xs;
+  k_dig_x<N><<<dim3((a.V + 3) / 4, ncol), 128, 0, s>>>(static_cast<const double2*>(a.x), ldc, a.V, x.xd, x.xc, x.xs, a.stop);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   // two columns share the block operand's loads and byte permutations (8^4, n = 48: 427 us for two
   // columns against 2 x 240 us); four would need 168 registers and spill (1008 us)
   if (ncol == 1) return launch_dig_nc<N, 1>(a, d, ncol, ldc, s);
   return launch_dig_nc<N, 2>(a, d, ncol, ldc, s);
+}
+
+template <int N>
+int launch_bresidual_n(const DigPass* passes, const int* map, int sites, const int* flags, const double2* coef,
+                       cudaStream_t s) {
+  constexpr size_t smem = (size_t)kDW * kDigCols * dig_slab<N>();
+  static bool attr = false;
+  if (!attr) {
+    COARSE_CUDA(cudaFuncSetAttribute(kb_residual_digits<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    attr = true;
+  }
+  kb_dig_x<N><<<sites / 4, 128, 0, s>>>(passes, map, flags);
+  note_launch();
+  COARSE_CUDA(cudaGetLastError());
+  kb_residual_digits<N><<<sites, 32 * kDW, smem, s>>>(passes, map, flags, coef);
+  note_launch();
+  COARSE_CUDA(cudaGetLastError());
+  return COARSE_OK;
 }
 
 }  // namespace
@@ -531,6 +618,18 @@ int launch_dig_blocks(const double2* blocks, int V, int n, void* dig, double* sc
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   return COARSE_OK;
+}
+
+int launch_bresidual_digits(int n, const DigPass* passes, const int* map, int sites, const int* flags,
+                            const double2* coef, cudaStream_t s) {
+  if (sites <= 0) return COARSE_OK;
+  switch (n) {
+    case 16: return launch_bresidual_n<16>(passes, map, sites, flags, coef, s);
+    case 32: return launch_bresidual_n<32>(passes, map, sites, flags, coef, s);
+    case 48: return launch_bresidual_n<48>(passes, map, sites, flags, coef, s);
+  }
+  set_error("batched residual: unsupported n = %d", n);
+  return COARSE_ERR_INVALID_ARG;
 }
 
 int launch_apply_digits(int n, const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {

@@ -26,4 +26,26 @@ int launch_dig_blocks(const double2* blocks, int V, int n, void* dig, double* sc
 // operands a.dig (must be set); a.digx holds room for ncol columns.
 int launch_apply_digits(int n, const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s);
 
+// Batched FP64 residual: one pass = up to kDigCols columns of one operator.  Launches cover the passes' sites
+// padded to kDigMapSites each; map[i] is the pass of sites i * kDigMapSites ..
+constexpr int kDigMapSites = 64;
+struct DigPass {
+  const double2* x;  // columns at x + c ldx, addends z + c ldx, results y + c ldy
+  const double2* z;
+  double2* y;
+  size_t ldx, ldy;
+  const void* dig;
+  const double* digscale;
+  void* digx;        // room for `cols` columns
+  const void* blocks;
+  const int* nb;
+  double mu;
+  int V, cols;
+  int start;         // first site of the pass in the launch
+  int q0;            // first solve
+};
+// r = b - D x of the passes with a column that is not done (flags[2 q + 1]); sites: a multiple of kDigMapSites
+int launch_bresidual_digits(int n, const DigPass* passes, const int* map, int sites, const int* flags,
+                            const double2* coef, cudaStream_t s);
+
 }  // namespace coarse

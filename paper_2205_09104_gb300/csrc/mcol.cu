@@ -570,7 +570,7 @@ __device__ __forceinline__ void mul_block(uint32_t (&u)[3][8], const cbf16* blk,
 }
 
 template <int N>
-__global__ void __launch_bounds__(32 * kMW, 4) kb_eo_mma(const __grid_constant__ McPhase b) {
+__global__ void __launch_bounds__(32 * kMW, N == 48 ? 4 : 6) kb_eo_mma(const __grid_constant__ McPhase b) {
   constexpr int NT = N / 16;
   constexpr size_t BSZ = (size_t)N * N;
   extern __shared__ __align__(16) unsigned char mc_sm[];
