@@ -368,6 +368,8 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
     set_error("coarse_apply: unsupported n = %d (nv must be 8, 16 or 24)", n);
     return COARSE_ERR_INVALID_ARG;
   }
+  // the staged kernel copies site vectors in bulk: 16-byte aligned x only
+  if ((uintptr_t)a.x & 15) return launch_t<BT, float2, float2>(n, a, s);
   int choice = tune_fast_get(0, prec, ni, vb);
   if (choice < 0) {
     char key[64];
