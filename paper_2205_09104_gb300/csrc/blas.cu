@@ -104,28 +104,34 @@ __device__ __forceinline__ void warp_to_smem(float2 acc, double2* slot, int lane
   if (lane == 0) *slot = make_double2(double(acc.x), double(acc.y));
 }
 
+// Vectors read together by the chunk kernels: short chunks take more of them, so that a lane has as many
+// loads in flight either way (the vectors sit in L2 and the loop is bound by its latency).
+__host__ __device__ constexpr int chunk_group(int E) { return E >= 8 ? 2 : (E == 4 ? 4 : 8); }
+
 // dots of the chunk: wp[warp][i] = sum conj(q_i) w  (i < nq), wp[warp][nq] = ||w||^2
 template <class C, int E>
 __device__ __forceinline__ void chunk_dots(const C* const* q, int nq, const C (&wv)[E], long long base, int N,
                                            int lane, double2* wp) {
+  constexpr int G = chunk_group(E);
   int i = 0;
-  for (; i + 2 <= nq; i += 2) {
-    const C* q0 = q[i];
-    const C* q1 = q[i + 1];
-    C a0[E], a1[E];
+  for (; i + G <= nq; i += G) {
+    C a[G][E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const long long idx = base + lane + 32 * e;
-      if (idx < N) { a0[e] = q0[idx]; a1[e] = q1[idx]; } else { a0[e].x = a0[e].y = 0; a1[e].x = a1[e].y = 0; }
-    }
-    float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
+    for (int g = 0; g < G; ++g) {
+      const C* qg = q[i + g];
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      cfma_conj(s0, to_f2(a0[e]), to_f2(wv[e]));
-      cfma_conj(s1, to_f2(a1[e]), to_f2(wv[e]));
+      for (int e = 0; e < E; ++e) {
+        const long long idx = base + lane + 32 * e;
+        if (idx < N) a[g][e] = qg[idx]; else { a[g][e].x = a[g][e].y = 0; }
+      }
     }
-    warp_to_smem(s0, wp + i, lane);
-    warp_to_smem(s1, wp + i + 1, lane);
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int e = 0; e < E; ++e) cfma_conj(s, to_f2(a[g][e]), to_f2(wv[e]));
+      warp_to_smem(s, wp + i + g, lane);
+    }
   }
   for (; i < nq; ++i) {
     const C* q0 = q[i];
@@ -233,18 +239,23 @@ __global__ void __launch_bounds__(32 * kW) k_update(const C* const* q, int nq, c
     const long long idx = base + lane + 32 * e;
     if (idx < N) wv[e] = w[idx]; else { wv[e].x = 0; wv[e].y = 0; }
   }
+  constexpr int G = chunk_group(E) < 4 ? 4 : chunk_group(E);
   int i = 0;
-  for (; i + 4 <= nq; i += 4) {
-    const C *q0 = q[i], *q1 = q[i + 1], *q2 = q[i + 2], *q3 = q[i + 3];
-    const C h0 = hc[i], h1 = hc[i + 1], h2 = hc[i + 2], h3 = hc[i + 3];
+  for (; i + G <= nq; i += G) {
+    C a[G][E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const long long idx = base + lane + 32 * e;
-      if (idx < N) {
-        const C a0 = q0[idx], a1 = q1[idx], a2 = q2[idx], a3 = q3[idx];
-        cfma(wv[e], a0, h0); cfma(wv[e], a1, h1); cfma(wv[e], a2, h2); cfma(wv[e], a3, h3);
+    for (int g = 0; g < G; ++g) {
+      const C* qg = q[i + g];
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const long long idx = base + lane + 32 * e;
+        if (idx < N) a[g][e] = qg[idx]; else { a[g][e].x = a[g][e].y = 0; }
       }
     }
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int e = 0; e < E; ++e) cfma(wv[e], a[g][e], hc[i + g]);
   }
   for (; i < nq; ++i) {
     const C* q0 = q[i];
@@ -630,7 +641,11 @@ __global__ void __launch_bounds__(32 * kW) kb_norm64(const BSolve* S, int nsolve
 }  // namespace
 
 namespace {
-int chunk_elems(int N) { return N <= (1 << 18) ? 4 : (N <= (1 << 20) ? 8 : 16); }
+// Elements per lane: at least 128 CTAs from N = 32768 on (8^4, n = 32 halves: E = 2 instead of 4 took the
+// three Gram-Schmidt passes of a step from @@ to @@ us), few enough partials for the last CTA.
+int chunk_elems(int N) {
+  return N <= (1 << 15) ? 1 : (N <= (1 << 16) ? 2 : (N <= (1 << 18) ? 4 : (N <= (1 << 20) ? 8 : 16)));
+}
 int chunk_grid(int N, int E) { return (int)(((long long)N + 32LL * kW * E - 1) / (32LL * kW * E)); }
 
 template <class C>
@@ -640,7 +655,9 @@ int multidot_t(const void* const* q, int nq, const void* w, int N, double2* out,
   const int grid = chunk_grid(N, E);
   auto qq = (const C* const*)q;
   auto ww = (const C*)w;
-  if (E == 4) k_multidot<C, 4><<<grid, 32 * kW, 0, s>>>(qq, nq, ww, N, out, wnorm2, partial, counter, stop);
+  if (E == 1) k_multidot<C, 1><<<grid, 32 * kW, 0, s>>>(qq, nq, ww, N, out, wnorm2, partial, counter, stop);
+  else if (E == 2) k_multidot<C, 2><<<grid, 32 * kW, 0, s>>>(qq, nq, ww, N, out, wnorm2, partial, counter, stop);
+  else if (E == 4) k_multidot<C, 4><<<grid, 32 * kW, 0, s>>>(qq, nq, ww, N, out, wnorm2, partial, counter, stop);
   else if (E == 8) k_multidot<C, 8><<<grid, 32 * kW, 0, s>>>(qq, nq, ww, N, out, wnorm2, partial, counter, stop);
   else k_multidot<C, 16><<<grid, 32 * kW, 0, s>>>(qq, nq, ww, N, out, wnorm2, partial, counter, stop);
   return grid;
@@ -653,7 +670,11 @@ int update_t(const void* const* q, int nq, const double2* h, int negate, void* w
   const int grid = chunk_grid(N, E);
   auto qq = (const C* const*)q;
   auto ww = (C*)w;
-  if (E == 4)
+  if (E == 1)
+    k_update<C, 1><<<grid, 32 * kW, 0, s>>>(qq, nq, h, negate, ww, N, mode, out, wnorm2, partial, counter, stop);
+  else if (E == 2)
+    k_update<C, 2><<<grid, 32 * kW, 0, s>>>(qq, nq, h, negate, ww, N, mode, out, wnorm2, partial, counter, stop);
+  else if (E == 4)
     k_update<C, 4><<<grid, 32 * kW, 0, s>>>(qq, nq, h, negate, ww, N, mode, out, wnorm2, partial, counter, stop);
   else if (E == 8)
     k_update<C, 8><<<grid, 32 * kW, 0, s>>>(qq, nq, h, negate, ww, N, mode, out, wnorm2, partial, counter, stop);
@@ -822,7 +843,7 @@ int launch_bnorms64(const BSolve* S, int nsolves, const int* chunk_off, int tota
   return COARSE_OK;
 }
 
-int batch_chunk_elems(int maxN) { return chunk_elems(maxN); }
+int batch_chunk_elems(int maxN) { return chunk_elems(maxN) < 4 ? 4 : chunk_elems(maxN); }
 int batch_chunks(int N, int E) { return chunk_grid(N, E); }
 
 }  // namespace coarse

@@ -116,8 +116,12 @@ __device__ void finalize_warp(CycleState* st, const double2* h1, const double2* 
   if (lane == 0) st->j = j + 1;  // last: the normalisation kernel of this step keys on st->j == j + 1
 }
 
-__global__ void __launch_bounds__(32) k_step_finalize(CycleState* st, const double2* h1, const double2* h2, Dense d) {
+// host_stop (pinned host memory, or null): receives the stop flag, for the host to read after the step
+__global__ void __launch_bounds__(32) k_step_finalize(CycleState* st, const double2* h1, const double2* h2, Dense d,
+                                                      volatile int* host_stop) {
   finalize_warp(st, h1, h2, d);
+  __syncwarp();
+  if (host_stop != nullptr && threadIdx.x == 0) *host_stop = st->stop;
 }
 
 __global__ void __launch_bounds__(32) kb_finalize(const BSolve* S) {
@@ -430,8 +434,9 @@ int launch_p1_prep(CycleState* st, const double2* h, const double* nva, double t
   return COARSE_OK;
 }
 
-int launch_step_finalize(CycleState* st, const double2* h1, const double2* h2, const Dense& d, cudaStream_t s) {
-  k_step_finalize<<<1, 32, 0, s>>>(st, h1, h2, d);
+int launch_step_finalize(CycleState* st, const double2* h1, const double2* h2, const Dense& d, int* host_stop,
+                         cudaStream_t s) {
+  k_step_finalize<<<1, 32, 0, s>>>(st, h1, h2, d, host_stop);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   return COARSE_OK;

@@ -261,6 +261,10 @@ template <int N> constexpr int dig_row() { return 2 * N + 16; }
 template <int N> constexpr int dig_part() { return 15 * dig_row<N>(); }
 template <int N> constexpr int dig_slab() { return 2 * dig_part<N>(); }
 
+// CTAs per SM to keep registers for: as many as measured faster (two columns, 8^4: n = 16 89 us with three
+// against 135 us with one, n = 32 174 us with two against 226 us, n = 48 404 us with one against 437 us)
+__host__ __device__ constexpr int dig_min_blocks(int N, int C) { return N == 16 ? 3 : (N == 48 && C > 1 ? 1 : 2); }
+
 struct DigArgs {
   const uint4* dig;
   const double* bscale;
@@ -523,7 +527,7 @@ __device__ __forceinline__ void dig_site(const ApplyArgs& a, const DigArgs& dgt,
 }
 
 template <int N, int C>
-__global__ void __launch_bounds__(32 * kDW, C > 1 ? 1 : (N == 16 ? 3 : 2)) k_apply_digits(
+__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, C)) k_apply_digits(
     const __grid_constant__ ApplyArgs a, const __grid_constant__ DigArgs dgt, int ncol, long long ldc) {
   if (a.stop != nullptr && *a.stop) return;
   dig_site<N, C>(a, dgt, blockIdx.x, ncol, ldc, ldc, ldc);
@@ -531,7 +535,7 @@ __global__ void __launch_bounds__(32 * kDW, C > 1 ? 1 : (N == 16 ? 3 : 2)) k_app
 
 // Batched FP64 residual r = b - D x of every pass with an unfinished column (coef: {-1, +1}).
 template <int N>
-__global__ void __launch_bounds__(32 * kDW, 1) kb_residual_digits(const DigPass* __restrict__ passes,
+__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, kDigCols)) kb_residual_digits(const DigPass* __restrict__ passes,
                                                                   const int* __restrict__ map,
                                                                   const int* __restrict__ flags,
                                                                   const double2* coef) {

@@ -233,7 +233,7 @@ int Solver::ensure(int m, int k, int dmax) {
   tabs_base = tabs;
   tabs_used = host.size();
   tabs_cap = 16 * (size_t)(2 * maxq + 8) * sizeof(double2) / sizeof(void*);
-  COARSE_CUDA(cudaMallocHost((void**)&st_host, sizeof(CycleState) + 4 * sizeof(int)));
+  COARSE_CUDA(cudaMallocHost((void**)&st_host, sizeof(CycleState) + (kMaxDense + 1) * sizeof(int)));
   stop_host = (int*)(st_host + 1);
   for (int i = 0; i < 2; ++i)
     if (!chunk_ev[i]) COARSE_CUDA(cudaEventCreateWithFlags(&chunk_ev[i], cudaEventDisableTiming));
@@ -407,7 +407,7 @@ int Solver::p1_step(int j, int kc, void* const* tab) {
                     &st->p1_skip, stream));
   TRY(launch_update(v64, (const void* const*)at, nq, h1, 1, Va[j + 1], N, 0, nullptr, nullptr, partial, counter,
                     &st->p1_skip, stream));
-  TRY(launch_step_finalize(st, h1, nullptr, dn, stream));
+  TRY(launch_step_finalize(st, h1, nullptr, dn, stop_host + j, stream));
   TRY(launch_scale(v64, V[j + 1], &st->inv_h, make_double2(1.0, 0.0), V[j + 1], N, &st->j, j + 1, stream));
   return launch_scale(v64, Va[j + 1], &st->inv_h, make_double2(1.0, 0.0), Va[j + 1], N, &st->j, j + 1, stream);
 }
@@ -423,7 +423,7 @@ int Solver::arnoldi_step(int j, int kc, void* const* tab) {
   TRY(launch_update(v64, (const void* const*)tab, nq, h1, 1, wv, N, 2, h2, nullptr, partial, counter, stop, stream));
   TRY(launch_update(v64, (const void* const*)tab, nq, h2, 1, wv, N, 1, nullptr, &st->wnorm2, partial, counter, stop,
                     stream));
-  TRY(launch_step_finalize(st, h1, h2, dn, stream));
+  TRY(launch_step_finalize(st, h1, h2, dn, stop_host + j, stream));
   // normalise v_{j+1} whenever the finalize of this step ran (st->j == j + 1), also on the step that stops
   return launch_scale(v64, wv, &st->inv_h, make_double2(1.0, 0.0), wv, N, &st->j, j + 1, stream);
 }
@@ -501,23 +501,19 @@ int Solver::inner(double target_abs, int max_cycles, int m, int kdef, int ulimit
     TRY(launch_cycle_init(st, kc, steps, norm2, extract_full ? 0.0 : target_abs, dn.g, stream));
     TRY(launch_scale(v64, r, &st->inv_h, make_double2(1.0, 0.0), V[0], N, &st->stop, 0, stream));
     if (p1_active) TRY(opA(V[0], Va[0], &st->stop));  // v^a_0 = A v_0
-    // Steps go out in chunks; the stop flag of chunk c-1 is read back (async copy +
-    // event) while chunk c runs, so at most one chunk of gated launches follows a stop.
-    constexpr int kChunk = 4;
-    int pending = -1;  // chunk whose flag copy is in flight
+    // Step j + 1 goes out while step j runs, once step j - 1 is known not to have stopped the cycle (its
+    // finalize wrote the flag to pinned memory): at most one step of gated launches follows a stop.  (In
+    // chunks of four steps, on average five gated steps of about 27 us each followed at 8^4, n = 32.)
     int launched = 0;
-    for (int j0 = 0; j0 < steps; j0 += kChunk) {
-      const int cnt = steps - j0 < kChunk ? steps - j0 : kChunk;
-      launched += cnt;
-      TRY(run_chunk(j0, cnt, kc, tab));
-      const int slot = (j0 / kChunk) & 1;
-      COARSE_CUDA(cudaMemcpyAsync(stop_host + slot, &st->stop, sizeof(int), cudaMemcpyDeviceToHost, stream));
-      COARSE_CUDA(cudaEventRecord(chunk_ev[slot], stream));
-      if (pending >= 0) {
-        COARSE_CUDA(cudaEventSynchronize(chunk_ev[pending]));
-        if (stop_host[pending]) break;
+    for (int j = 0; j < steps; ++j) {
+      stop_host[j] = 0;
+      TRY(run_chunk(j, 1, kc, tab));
+      ++launched;
+      COARSE_CUDA(cudaEventRecord(chunk_ev[j & 1], stream));
+      if (j > 0) {
+        COARSE_CUDA(cudaEventSynchronize(chunk_ev[(j - 1) & 1]));
+        if (*(volatile int*)(stop_host + j - 1)) break;
       }
-      pending = slot;
     }
     cur_tag = -1;
     TRY(read_state());

@@ -52,7 +52,7 @@ struct Solver {
   double* norm2 = nullptr;
   CycleState* st = nullptr;
   CycleState* st_host = nullptr;
-  int* stop_host = nullptr;             // pinned: stop flags of the last two step chunks
+  int* stop_host = nullptr;             // pinned: stop flag after each step of the cycle, written by its finalize
   cudaEvent_t chunk_ev[2] = {nullptr, nullptr};
 
   int d = 0;             // polynomial degree in use

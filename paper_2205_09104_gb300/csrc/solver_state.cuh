@@ -52,7 +52,8 @@ struct Dense {
 
 int launch_cycle_init(CycleState* st, int k, int steps, const double* rnorm2, double target, double2* g,
                       cudaStream_t s);
-int launch_step_finalize(CycleState* st, const double2* h1, const double2* h2, const Dense& d, cudaStream_t s);
+int launch_step_finalize(CycleState* st, const double2* h1, const double2* h2, const Dense& d, int* host_stop,
+                         cudaStream_t s);
 // Latency-1 pipelined Arnoldi (Sec. 3.5): from the fused reduction of step i (h = [C, V]^H v^a_{i-1}
 // and ||v^a_{i-1}||^2) form t = ||v^a||^2 - sum |h|^2 into st->wnorm2 for the finalize; t below
 // minus its rounding (tol_u: unit roundoff of the vectors) is a breakdown that stops the cycle.
