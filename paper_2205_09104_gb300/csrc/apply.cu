@@ -22,6 +22,7 @@
 #include "batch.cuh"
 #include "digits.cuh"
 #include "pipe.cuh"
+#include "site8.cuh"
 #include "tune.cuh"
 
 namespace coarse {
@@ -297,6 +298,68 @@ int launch_t(int n, const ApplyArgs& a, cudaStream_t s) {
 }
 
 
+// Eight warps per site (site8.cuh): pull only, the self block's rows split over the warps.
+template <int N, class BT>
+__global__ void __launch_bounds__(32 * kS8, N == 48 ? 2 : 3) k_apply8(ApplyArgs a) {
+  constexpr int CPL = N / 8;
+  constexpr size_t BSZ = (size_t)N * N;
+  __shared__ float2 hp[kS8][N];
+  __shared__ float2 us[N];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 7, mu = warp & 3;
+  const int x = blockIdx.x;
+  const int src = __ldg(a.nb + x * 8 + warp);
+  if (a.stop != nullptr && *a.stop) return;
+  const BT* B = static_cast<const BT*>(a.blocks);
+  const float2* X = static_cast<const float2*>(a.x);
+  const bool adj = a.adjoint;
+  S8Diag<N, BT> self;
+  self.load(B + (size_t)x * 5 * BSZ, warp, lane);
+  float2 w[CPL], xs = make_float2(0.f, 0.f), aux = xs;
+  load_vec<float2, float2, CPL>(X + (size_t)x * N + t * CPL, w);
+  const size_t idx = (size_t)x * N + threadIdx.x;
+  if (threadIdx.x < N) {
+    xs = X[idx];
+    if (a.mode == APPLY_POLY) aux = static_cast<const float2*>(a.acc)[idx];
+    if (a.mode == APPLY_AXPBY) aux = static_cast<const float2*>(a.z)[idx];
+  }
+  if (warp < 4) s8_fwd<N, BT>(B + ((size_t)x * 5 + 1 + mu) * BSZ, X + (size_t)src * N, adj, hp[warp], lane);
+  else s8_bwd<N, BT>(B + ((size_t)src * 5 + 1 + mu) * BSZ, X + (size_t)src * N, !adj, hp[warp], lane);
+  if (adj && t * CPL >= N / 2)
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) w[c] = make_float2(-w[c].x, -w[c].y);
+  self.mul(w, us, warp, lane);
+  __syncthreads();
+  if (threadIdx.x < N) {
+    float2 r = us[threadIdx.x];
+    if (adj && threadIdx.x >= N / 2) r = make_float2(-r.x, -r.y);
+#pragma unroll
+    for (int q = 0; q < kS8; ++q) r = cadd(r, hp[q][threadIdx.x]);
+    const float m = threadIdx.x < N / 2 ? (float)a.mu : -(float)a.mu;  // + i mu sigma3 x
+    r.x -= m * xs.y;
+    r.y += m * xs.x;
+    float2* y = static_cast<float2*>(a.y) + idx;
+    if (a.mode == APPLY_AXPBY) {
+      const double2 c0 = a.coef[0], c1 = a.coef[1];
+      *y = cadd(cmul(make_float2((float)c0.x, (float)c0.y), r), cmul(make_float2((float)c1.x, (float)c1.y), aux));
+    } else {
+      s8_finish(a.mode, r, xs, aux, a.coef, y, static_cast<float2*>(a.acc) + idx);
+    }
+  }
+}
+
+template <class BT>
+int launch_8(int n, const ApplyArgs& a, cudaStream_t s) {
+  switch (n) {
+    case 16: k_apply8<16, BT><<<a.V, 32 * kS8, 0, s>>>(a); break;
+    case 32: k_apply8<32, BT><<<a.V, 32 * kS8, 0, s>>>(a); break;
+    case 48: k_apply8<48, BT><<<a.V, 32 * kS8, 0, s>>>(a); break;
+    default: set_error("coarse_apply: unsupported n = %d (nv must be 8, 16 or 24)", n); return COARSE_ERR_INVALID_ARG;
+  }
+  note_launch();
+  COARSE_CUDA(cudaGetLastError());
+  return COARSE_OK;
+}
+
 template <int N, class BT>
 int launch_tma_n(const ApplyArgs& a, cudaStream_t s) {
   using Cfg = TmaCfg<N, BT>;
@@ -358,8 +421,8 @@ __global__ void __launch_bounds__(128) kb_residual64(BApply b, const double2* co
 }  // namespace
 
 // FP32 / BF16: the autotuner picks, per (precision, n, lattice-size bucket), between the
-// TMA-staged persistent kernel (candidate 0, the default) and the register push-pull kernel
-// (candidate 1).  Candidates are timed in plain mode into a scratch output, so that an epilogue
+// TMA-staged persistent kernel (candidate 0, the default), the register push-pull kernel
+// (candidate 1) and the pull kernel of eight warps per site (candidate 2).  Candidates are timed in plain mode into a scratch output, so that an epilogue
 // that accumulates (the polynomial chain) never runs twice; decisions are cached per process.
 template <class BT>
 int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
@@ -388,12 +451,12 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
       t.acc = nullptr;
       t.coef = nullptr;
       t.stop = nullptr;
-      return c.a == 1 ? launch_t<BT, float2, float2>(n, t, s) : launch_tma<BT>(n, t, s);
+      return c.a == 2 ? launch_8<BT>(n, t, s) : c.a == 1 ? launch_t<BT, float2, float2>(n, t, s) : launch_tma<BT>(n, t, s);
     };
     TuneChoice c;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(s, &cap);
-    const int rc = tune_pick(key, {TuneChoice{0, 0, 0}, TuneChoice{1, 0, 0}}, run, s, &c);
+    const int rc = tune_pick(key, {TuneChoice{0, 0, 0}, TuneChoice{1, 0, 0}, TuneChoice{2, 0, 0}}, run, s, &c);
     if (scratch) {
       cudaStreamSynchronize(s);
       cudaFree(scratch);
@@ -402,7 +465,7 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
     if (cap == cudaStreamCaptureStatusNone) tune_fast_put(0, prec, ni, vb, c.a);
     choice = c.a;
   }
-  return choice == 1 ? launch_t<BT, float2, float2>(n, a, s) : launch_tma<BT>(n, a, s);
+  return choice == 2 ? launch_8<BT>(n, a, s) : choice == 1 ? launch_t<BT, float2, float2>(n, a, s) : launch_tma<BT>(n, a, s);
 }
 
 int launch_apply(int prec, int n, const ApplyArgs& a, cudaStream_t s) {

@@ -20,6 +20,7 @@
 #include "batch.cuh"
 #include "oddeven.cuh"
 #include "pipe.cuh"
+#include "site8.cuh"
 #include "tune.cuh"
 
 namespace coarse {
@@ -842,6 +843,57 @@ __global__ void __launch_bounds__(kEoRingThreads, 1) k_eo_ring(EoArgs a, int S) 
   }
 }
 
+// Eight warps per site (site8.cuh): the hops, then the inverse block on their sum.
+template <int N, class BT>
+__global__ void __launch_bounds__(32 * kS8, N == 48 ? 2 : 3) k_eo_half8(EoArgs a) {
+  constexpr int CPL = N / 8;
+  constexpr size_t BSZ = (size_t)N * N;
+  __shared__ float2 hp[kS8][N];
+  __shared__ float2 us[N];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 7;
+  const int nh = a.V / 2, k = blockIdx.x;
+  const int4 q = __ldg(a.rec + ((size_t)a.out_par * nh + k) * 4 + (warp & 3));
+  if (a.stop && *a.stop) return;
+  const float2* v = static_cast<const float2*>(a.v);
+  const float2* z = static_cast<const float2*>(a.z);
+  const float2* base = static_cast<const float2*>(a.base);
+  const size_t off = (size_t)k * N;
+  S8Diag<N, BT> inv;
+  inv.load(static_cast<const BT*>(a.inv) + (size_t)q.w * BSZ, warp, lane);
+  float2 zz[CPL], bs = make_float2(0.f, 0.f), ac = bs;
+  if (z) load_vec<float2, float2, CPL>(z + off + t * CPL, zz);
+  if (threadIdx.x < N) {
+    if (base) bs = base[off + threadIdx.x];
+    if (a.mode == APPLY_POLY) ac = static_cast<const float2*>(a.acc)[off + threadIdx.x];
+  }
+  if (v) {
+    const BT* B = static_cast<const BT*>(a.blocks);
+    const int mu = warp & 3;
+    if (warp < 4) s8_fwd<N, BT>(B + ((size_t)q.w * 5 + 1 + mu) * BSZ, v + (size_t)q.x * N, false, hp[warp], lane);
+    else s8_bwd<N, BT>(B + ((size_t)q.y * 5 + 1 + mu) * BSZ, v + (size_t)q.z * N, true, hp[warp], lane);
+  }
+  __syncthreads();
+  float2 gi[CPL];
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) {
+    float2 h = make_float2(0.f, 0.f);
+    if (v) {
+      h = hp[0][t * CPL + c];
+#pragma unroll
+      for (int w = 1; w < kS8; ++w) h = cadd(h, hp[w][t * CPL + c]);
+    }
+    gi[c] = z ? csub(zz[c], h) : h;
+  }
+  inv.mul(gi, us, warp, lane);
+  __syncthreads();
+  if (threadIdx.x < N) {
+    const size_t idx = off + threadIdx.x;
+    float2 r = us[threadIdx.x];
+    if (base) r = csub(bs, r);
+    s8_finish(a.mode, r, bs, ac, a.coef, static_cast<float2*>(a.y) + idx, static_cast<float2*>(a.acc) + idx);
+  }
+}
+
 // full vector <-> (even, odd) compressed halves
 template <class VT>
 __global__ void k_eo_split(const VT* __restrict__ full, const int* __restrict__ sites, int V, int n, VT* ev, VT* od) {
@@ -982,6 +1034,20 @@ int launch_eo_variant(int variant, int n, const EoArgs& a, cudaStream_t s) {
     variant = 4;  // FP64 blocks, no hop input (the right-hand side pass) or unaligned vectors
   }
   if (variant >= 4 && (al & 15)) variant -= 2;
+  if (variant == 7) {
+    if constexpr (sizeof(decltype(AC{}.x)) == 4) {
+      switch (n) {
+        case 16: k_eo_half8<16, BT><<<half, 32 * kS8, 0, s>>>(a); break;
+        case 32: k_eo_half8<32, BT><<<half, 32 * kS8, 0, s>>>(a); break;
+        case 48: k_eo_half8<48, BT><<<half, 32 * kS8, 0, s>>>(a); break;
+        default: set_error("odd-even: unsupported n = %d", n); return COARSE_ERR_INVALID_ARG;
+      }
+      note_launch();
+      COARSE_CUDA(cudaGetLastError());
+      return COARSE_OK;
+    }
+    variant = 0;  // FP64
+  }
 #define EO_LAUNCH(NN)                                                                           \
   case NN:                                                                                      \
     if (variant == 1) k_eo_half_w<NN, BT, VT, AC><<<(half + 3) / 4, 128, 0, s>>>(a);             \
@@ -1007,7 +1073,7 @@ int launch_eo_variant(int variant, int n, const EoArgs& a, cudaStream_t s) {
 // site (candidate 0), one warp per site (candidate 1) and one CTA of 2 warps per site with the
 // direction loop rolled (candidates 2, 4) or unrolled (3, 5), the last two with the inverse block
 // and the epilogue vectors prefetched into shared memory, and (FP32 / BF16 blocks) the streamed
-// persistent layout (6); candidates run in plain mode into a scratch output.
+// persistent layout (6) and the CTA of 8 warps (7); candidates run in plain mode into a scratch output.
 template <class BT, class VT, class AC>
 int launch_eo_tuned(int prec, int n, const EoArgs& a, cudaStream_t s) {
   const int ni = n / 16 - 1, vb = std::min(tune_bucket(a.V), 31);
@@ -1045,7 +1111,7 @@ int launch_eo_tuned(int prec, int n, const EoArgs& a, cudaStream_t s) {
     cudaStreamIsCapturing(s, &cap);
     TuneChoice c;
     std::vector<TuneChoice> cands;
-    for (int v = 0; v <= 6; ++v)
+    for (int v = 0; v <= 7; ++v)
       if (v < 6 || sizeof(decltype(AC{}.x)) == 4) cands.push_back(TuneChoice{v, 0, 0});
     const int rc = tune_pick(key, cands, run, s, &c);
     if (scratch) {
