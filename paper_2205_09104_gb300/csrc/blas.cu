@@ -49,24 +49,30 @@ __device__ void block_sum(double (&v)[KV], double* sh /* [kThreads/32][KV] */) {
   __syncthreads();
 }
 
-// Last block: out[o] = sum_c partial[o][c] for o < nout (partial as double pairs).
+// Last block: out[o] = sum_c partial[o][c] for o < nout (partial as double pairs).  Eight lanes per real
+// number, so that the block works on 32 of them at once, each lane with four chains.
 __device__ void finish(const double* partial, int nout, int nch, double2* out, double* wnorm2, int norm_slot) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int o = warp; o < nout; o += kThreads / 32) {
-    double re = 0.0, im = 0.0;
-    for (int c = lane; c < nch; c += 32) {
-      re += partial[(size_t)(2 * o) * nch + c];
-      im += partial[(size_t)(2 * o + 1) * nch + c];
+  const int sub = threadIdx.x & 7;
+  for (int v0 = 0; v0 < 2 * nout; v0 += kThreads / 8) {
+    const int v = v0 + (threadIdx.x >> 3);
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    if (v < 2 * nout) {
+      const double* p = partial + (size_t)v * nch;
+      int c = sub;
+      for (; c + 24 < nch; c += 32)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[k] += p[c + 8 * k];
+      for (; c < nch; c += 8) s[0] += p[c];
     }
-    for (int off = 16; off > 0; off >>= 1) {
-      re += __shfl_xor_sync(0xffffffffu, re, off);
-      im += __shfl_xor_sync(0xffffffffu, im, off);
-    }
-    if (lane == 0) {
+    double r = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+    if (sub == 0 && v < 2 * nout) {
+      const int o = v >> 1;
       if (o == norm_slot) {
-        if (wnorm2) *wnorm2 = re;
+        if (wnorm2 && !(v & 1)) *wnorm2 = r;
       } else if (out) {
-        out[o] = make_double2(re, im);
+        reinterpret_cast<double*>(out)[v] = r;
       }
     }
   }
@@ -113,35 +119,27 @@ template <class C, int E>
 __device__ __forceinline__ void chunk_dots(const C* const* q, int nq, const C (&wv)[E], long long base, int N,
                                            int lane, double2* wp) {
   constexpr int G = chunk_group(E);
-  int i = 0;
-  for (; i + G <= nq; i += G) {
+  for (int i = 0; i < nq; i += G) {  // the last group is padded with its last vector
     C a[G][E];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      const C* qg = q[i + g];
+      const C* qg = q[i + g < nq ? i + g : nq - 1];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const long long idx = base + lane + 32 * e;
         if (idx < N) a[g][e] = qg[idx]; else { a[g][e].x = a[g][e].y = 0; }
       }
     }
+    float2 s[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      float2 s = make_float2(0.f, 0.f);
+      s[g] = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int e = 0; e < E; ++e) cfma_conj(s, to_f2(a[g][e]), to_f2(wv[e]));
-      warp_to_smem(s, wp + i + g, lane);
+      for (int e = 0; e < E; ++e) cfma_conj(s[g], to_f2(a[g][e]), to_f2(wv[e]));
     }
-  }
-  for (; i < nq; ++i) {
-    const C* q0 = q[i];
-    float2 s0 = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const long long idx = base + lane + 32 * e;
-      if (idx < N) cfma_conj(s0, to_f2(q0[idx]), to_f2(wv[e]));
-    }
-    warp_to_smem(s0, wp + i, lane);
+    for (int g = 0; g < G; ++g)
+      if (i + g < nq) warp_to_smem(s[g], wp + i + g, lane);
   }
   float nn = 0.f;
 #pragma unroll
@@ -181,12 +179,13 @@ __device__ void cta_finish(const double2* wp /*[kW][kMaxQ]*/, int nout, double* 
                            double2* out, double* wnorm2, int norm_slot, int cta = -1, int nch = -1) {
   __syncthreads();
   if (cta < 0) { cta = blockIdx.x; nch = gridDim.x; }
-  for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-    double re = 0.0, im = 0.0;
+  const double* w = reinterpret_cast<const double*>(wp);
+  for (int v = threadIdx.x; v < 2 * nout; v += blockDim.x) {
+    double r[kW];
 #pragma unroll
-    for (int w = 0; w < kW; ++w) { re += wp[w * kMaxQ + o].x; im += wp[w * kMaxQ + o].y; }
-    partial[(size_t)(2 * o) * nch + cta] = re;
-    partial[(size_t)(2 * o + 1) * nch + cta] = im;
+    for (int i = 0; i < kW; ++i) r[i] = w[i * 2 * kMaxQ + v];
+    static_assert(kW == 8, "pairwise sum");
+    partial[(size_t)v * nch + cta] = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
   }
   if (last_block(counter, nch)) {
     finish(partial, nout, nch, out, wnorm2, norm_slot);
@@ -199,17 +198,21 @@ template <class C, int E>
 __global__ void __launch_bounds__(32 * kW) k_multidot(const C* const* q, int nq, const C* w, int N, double2* out,
                                                       double* wnorm2, double* partial, unsigned* counter,
                                                       const int* stop) {
-  if (stop != nullptr && *stop) return;
   __shared__ double2 wp[kW * kMaxQ];
+  __shared__ const C* qp[kMaxQ];  // read once: a pointer load in front of every vector would double its latency
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long base = ((long long)blockIdx.x * kW + warp) * 32 * E;
+  for (int i = threadIdx.x; i < nq; i += blockDim.x) qp[i] = q[i];
+  const int halt = stop != nullptr ? *stop : 0;
   C wv[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const long long idx = base + lane + 32 * e;
     if (idx < N) wv[e] = w[idx]; else { wv[e].x = 0; wv[e].y = 0; }
   }
-  chunk_dots(q, nq, wv, base, N, lane, wp + warp * kMaxQ);
+  if (halt) return;
+  __syncthreads();
+  chunk_dots(qp, nq, wv, base, N, lane, wp + warp * kMaxQ);
   cta_finish(wp, nq + 1, partial, counter, out, wnorm2, nq);
 }
 
@@ -220,17 +223,18 @@ __global__ void __launch_bounds__(32 * kW) k_update(const C* const* q, int nq, c
                                                     int N, int mode /*0: none, 1: norm, 2: dots+norm*/,
                                                     double2* out, double* wnorm2, double* partial,
                                                     unsigned* counter, const int* stop) {
-  if (stop != nullptr && *stop) return;
   using T = typename Acc<C>::T;
   __shared__ double2 wp[kW * kMaxQ];
   __shared__ C hc[kMaxQ];
+  __shared__ const C* qp[kMaxQ];
   for (int i = threadIdx.x; i < nq; i += blockDim.x) {
     const double2 v = h[i];
     const double sg = negate ? -1.0 : 1.0;
+    qp[i] = q[i];
     hc[i].x = T(sg * v.x);
     hc[i].y = T(sg * v.y);
   }
-  __syncthreads();
+  const int halt = stop != nullptr ? *stop : 0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long base = ((long long)blockIdx.x * kW + warp) * 32 * E;
   C wv[E];
@@ -239,31 +243,49 @@ __global__ void __launch_bounds__(32 * kW) k_update(const C* const* q, int nq, c
     const long long idx = base + lane + 32 * e;
     if (idx < N) wv[e] = w[idx]; else { wv[e].x = 0; wv[e].y = 0; }
   }
-  constexpr int G = chunk_group(E) < 4 ? 4 : chunk_group(E);
-  int i = 0;
-  for (; i + G <= nq; i += G) {
-    C a[G][E];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const C* qg = q[i + g];
+  if (halt) return;
+  __syncthreads();
+  if constexpr (E >= 8) {
+    int i = 0;
+    for (; i + 4 <= nq; i += 4) {
+      const C *q0 = qp[i], *q1 = qp[i + 1], *q2 = qp[i + 2], *q3 = qp[i + 3];
+      const C h0 = hc[i], h1 = hc[i + 1], h2 = hc[i + 2], h3 = hc[i + 3];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const long long idx = base + lane + 32 * e;
-        if (idx < N) a[g][e] = qg[idx]; else { a[g][e].x = a[g][e].y = 0; }
+        if (idx < N) {
+          const C a0 = q0[idx], a1 = q1[idx], a2 = q2[idx], a3 = q3[idx];
+          cfma(wv[e], a0, h0); cfma(wv[e], a1, h1); cfma(wv[e], a2, h2); cfma(wv[e], a3, h3);
+        }
       }
     }
+    for (; i < nq; ++i) {
+      const C* q0 = qp[i];
+      const C h0 = hc[i];
 #pragma unroll
-    for (int g = 0; g < G; ++g)
+      for (int e = 0; e < E; ++e) {
+        const long long idx = base + lane + 32 * e;
+        if (idx < N) cfma(wv[e], q0[idx], h0);
+      }
+    }
+  } else {  // short chunks: as many loads in flight from more vectors, the last group padded
+    constexpr int G = E == 4 ? 4 : 8;
+    for (int i = 0; i < nq; i += G) {
+      C a[G][E];
 #pragma unroll
-      for (int e = 0; e < E; ++e) cfma(wv[e], a[g][e], hc[i + g]);
-  }
-  for (; i < nq; ++i) {
-    const C* q0 = q[i];
-    const C h0 = hc[i];
+      for (int g = 0; g < G; ++g) {
+        const C* qg = qp[i + g < nq ? i + g : nq - 1];
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const long long idx = base + lane + 32 * e;
-      if (idx < N) cfma(wv[e], q0[idx], h0);
+        for (int e = 0; e < E; ++e) {
+          const long long idx = base + lane + 32 * e;
+          if (idx < N) a[g][e] = qg[idx]; else { a[g][e].x = a[g][e].y = 0; }
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+        if (i + g < nq)
+#pragma unroll
+          for (int e = 0; e < E; ++e) cfma(wv[e], a[g][e], hc[i + g]);
     }
   }
 #pragma unroll
@@ -273,10 +295,10 @@ __global__ void __launch_bounds__(32 * kW) k_update(const C* const* q, int nq, c
   }
   if (mode == 0) return;
   if (mode == 2) {
-    chunk_dots(q, nq, wv, base, N, lane, wp + warp * kMaxQ);
+    chunk_dots(qp, nq, wv, base, N, lane, wp + warp * kMaxQ);
     cta_finish(wp, nq + 1, partial, counter, out, wnorm2, nq);
   } else {
-    chunk_dots(q, 0, wv, base, N, lane, wp + warp * kMaxQ);
+    chunk_dots(qp, 0, wv, base, N, lane, wp + warp * kMaxQ);
     cta_finish(wp, 1, partial, counter, nullptr, wnorm2, 0);
   }
 }
@@ -289,6 +311,8 @@ __global__ void __launch_bounds__(kThreads) k_combine(const C* const* in, int ni
   using T = typename Acc<C>::T;
   extern __shared__ unsigned char smem_raw[];
   C* cf = reinterpret_cast<C*>(smem_raw);  // [nin][TILE]
+  __shared__ const C* ip[kMaxQ];
+  for (int j = threadIdx.x; j < nin; j += kThreads) ip[j] = in[j];
   const int o0 = blockIdx.y * TILE;
   for (int k = threadIdx.x; k < nin * TILE; k += kThreads) {
     const int j = k / TILE, i = k % TILE;
@@ -302,8 +326,9 @@ __global__ void __launch_bounds__(kThreads) k_combine(const C* const* in, int ni
     C acc[TILE];
 #pragma unroll
     for (int i = 0; i < TILE; ++i) { acc[i].x = 0; acc[i].y = 0; }
+#pragma unroll 4
     for (int j = 0; j < nin; ++j) {
-      const C a = in[j][e];
+      const C a = ip[j][e];
 #pragma unroll
       for (int i = 0; i < TILE; ++i) cfma(acc[i], a, cf[j * TILE + i]);
     }
