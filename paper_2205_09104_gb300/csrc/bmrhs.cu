@@ -30,7 +30,9 @@ struct BMrhsPolicy {
     return r;
   }
   __device__ int adjoint() const { return 0; }
-  __device__ void finish(const MrhsGroup& gr, int x, int rt, const MrhsAcc<kMrhsMaxT>& acc) const {
+  struct Pre {};
+  __device__ void prefetch(const MrhsGroup&, int, int, Pre&) const {}
+  __device__ void finish(const MrhsGroup& gr, int x, int rt, const MrhsAcc<kMrhsMaxT>& acc, const Pre&) const {
     const BMApply& a = *pa;
     const BMOp& op = a.ops[gr.tag];
     const int lane = threadIdx.x & 31, t = lane & 3, g = lane >> 2;
@@ -45,7 +47,9 @@ struct BMrhsPolicy {
       const float2* xv = static_cast<const float2*>(bsel(s, a.xsel, step)) + (size_t)x * N;
       float2* yv = static_cast<float2*>(bsel(s, a.ysel, step)) + (size_t)x * N;
       float2 y[2];
-      mrhs_rows_out<N, kMrhsMaxT>(acc, tl, rt, xv, op.mu, 0, y[0], y[1]);
+      const float2 none = make_float2(0.f, 0.f);
+      mrhs_rows_out<N, kMrhsMaxT>(acc, tl, rt, op.mu != 0.f ? xv[r0] : none, op.mu != 0.f ? xv[r0 + 8] : none, op.mu, 0,
+                                  y[0], y[1]);
       if (a.mode == APPLY_PLAIN) {
         yv[r0] = y[0];
         yv[r0 + 8] = y[1];

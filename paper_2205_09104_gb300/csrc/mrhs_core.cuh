@@ -115,18 +115,15 @@ __device__ __forceinline__ void mrhs_block(const uint4* blk, const uint2* vec, i
 //   y = o (P + s3 Q + i mu' v),  v = (adj ? x : s3 x),  o = (adj ? s3 : 1),
 // with mu' already signed (-mu for the adjoint).  Returns the two complex values.
 template <int N, int T>
-__device__ __forceinline__ void mrhs_rows_out(const MrhsAcc<T>& acc, int tl, int rt, const float2* xsite, float mu,
+__device__ __forceinline__ void mrhs_rows_out(const MrhsAcc<T>& acc, int tl, int rt, float2 v0, float2 v1, float mu,
                                               int adj, float2& y0, float2& y1) {
   constexpr int NV = N / 2;
-  const int g = (threadIdx.x & 31) >> 2;
   const float s0 = (16 * rt < NV) ? 1.f : -1.f, s1 = (16 * rt + 8 < NV) ? 1.f : -1.f;
   y0 = make_float2(acc.P1[tl][0] - acc.P2[tl][1] + s0 * (acc.Q1[tl][0] + acc.Q2[tl][1]),
                    acc.P1[tl][1] + acc.P2[tl][0] + s0 * (acc.Q1[tl][1] - acc.Q2[tl][0]));
   y1 = make_float2(acc.P1[tl][2] - acc.P2[tl][3] + s1 * (acc.Q1[tl][2] + acc.Q2[tl][3]),
                    acc.P1[tl][3] + acc.P2[tl][2] + s1 * (acc.Q1[tl][3] - acc.Q2[tl][2]));
   if (mu != 0.f) {
-    const int r0 = 16 * rt + g;
-    const float2 v0 = __ldg(xsite + r0), v1 = __ldg(xsite + r0 + 8);
     const float m0 = adj ? mu : mu * s0, m1 = adj ? mu : mu * s1;
     y0.x -= m0 * v0.y; y0.y += m0 * v0.x;
     y1.x -= m1 * v1.y; y1.y += m1 * v1.x;

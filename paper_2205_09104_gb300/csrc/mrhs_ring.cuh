@@ -6,7 +6,9 @@
 //     __device__ int ngroups(int P) const;                  // site groups of P sites
 //     __device__ MrhsGroup group(int g, int P) const;       // blocks / vectors / sites of group g
 //     __device__ int adjoint() const;
-//     __device__ void finish(const MrhsGroup&, int x, int rt, const MrhsAcc<TACC>&) const;  // epilogue
+//     struct Pre;                                           // registers of the epilogue's operands
+//     __device__ void prefetch(const MrhsGroup&, int x, int rt, Pre&) const;  // loads them, nine items early
+//     __device__ void finish(const MrhsGroup&, int x, int rt, const MrhsAcc<TACC>&, const Pre&) const;  // epilogue
 //   };
 //
 // A CTA walks its site groups g = blockIdx.x + k * gridDim.x and for each the 9 items of Eq. (6):
@@ -138,11 +140,13 @@ __device__ __forceinline__ void mrhs_ring(const Policy& pol, int S, uint32_t SB,
   MrhsAcc<TACC> acc;
   acc.zero();
   MrhsGroup gr{};
+  typename Policy::Pre pre;
   int ok = 1;
   for (int it = 0; it < items; ++it) {
     const int slot = it % S;
     const int b = it % 9;
     if (b == 0) gr = pol.group((int)blockIdx.x + (it / 9) * (int)gridDim.x, P);
+    if (b == 0 && p < gr.np) pol.prefetch(gr, gr.x0 + p, rt, pre);
     if (!mbar_wait_suspend(full + slot, (uint32_t)((it / S) & 1))) ok = 0;
     if (!__all_sync(0xffffffffu, ok)) break;
     const bool valid = p < gr.np;
@@ -163,7 +167,7 @@ __device__ __forceinline__ void mrhs_ring(const Policy& pol, int S, uint32_t SB,
     __syncwarp();
     if (lane == 0) mbar_arrive(empty + slot);
     if (b == 8) {
-      if (valid) pol.finish(gr, gr.x0 + p, rt, acc);
+      if (valid) pol.finish(gr, gr.x0 + p, rt, acc, pre);
       acc.zero();
     }
   }

@@ -53,7 +53,7 @@ void append_cache(const std::string& key, const Entry& e) {
 }
 
 constexpr int kFastDevices = 64;
-std::atomic<int> g_fast[kFastDevices][2][3][3][32];
+std::atomic<int> g_fast[kFastDevices][3][4][3][32];
 std::once_flag g_fast_once;
 std::string g_model[kFastDevices];
 
@@ -97,14 +97,14 @@ const std::string& model_suffix() {
 int tune_fast_get(int family, int prec, int ni, int vb) {
   std::call_once(g_fast_once, fast_clear);
   const int dev = current_device();
-  if (dev < 0 || family < 0 || family > 1 || prec < 0 || prec > 2 || ni < 0 || ni > 2 || vb < 0 || vb > 31) return -1;
+  if (dev < 0 || family < 0 || family > 2 || prec < 0 || prec > 3 || ni < 0 || ni > 2 || vb < 0 || vb > 31) return -1;
   return g_fast[dev][family][prec][ni][vb].load(std::memory_order_acquire);
 }
 
 void tune_fast_put(int family, int prec, int ni, int vb, int choice) {
   std::call_once(g_fast_once, fast_clear);
   const int dev = current_device();
-  if (dev < 0 || family < 0 || family > 1 || prec < 0 || prec > 2 || ni < 0 || ni > 2 || vb < 0 || vb > 31) return;
+  if (dev < 0 || family < 0 || family > 2 || prec < 0 || prec > 3 || ni < 0 || ni > 2 || vb < 0 || vb > 31) return;
   g_fast[dev][family][prec][ni][vb].store(choice, std::memory_order_release);
 }
 

@@ -31,8 +31,9 @@ int tune_pick(const std::string& key, const std::vector<TuneChoice>& cands,
 int tune_bucket(long long v);
 
 // Decisions of the hot launch paths, per device ordinal, for lock-free reads on every launch:
-// family (0 = single-RHS stencil, 1 = odd-even half apply), block precision, n / 16 - 1, size
-// bucket -> candidate, or -1 while undecided.  tune_pick remains the source of the decisions;
+// family (0 = single-RHS stencil, 1 = odd-even half apply, 2 = multi-RHS stencil), block precision
+// (family 2: column tiles - 1), n / 16 - 1, size bucket -> candidate (family 2: a + 256 b), or -1 while
+// undecided.  tune_pick remains the source of the decisions;
 // coarse_autotune_set clears these entries so that the next launch looks its key up again.
 int tune_fast_get(int family, int prec, int ni, int vb);
 void tune_fast_put(int family, int prec, int ni, int vb, int choice);
