@@ -30,9 +30,8 @@
 // m16n8k16 A fragment, each the bytes {re, im of column 2t, re, im of column 2t + 1}: 8 bytes per real
 // number, one 4 KB stream per tile.
 //
-// One CTA of nine warps per site, one block product per warp (the nine sums are added in a fixed order).
-// A forward block is read again, transposed, by the site in front of it; with a whole site in flight at
-// once, and so as few sites as fill the chip, that second read still finds the block in L2.
+// Two kernels: one CTA of nine warps per site, one block product per warp (small lattices, several columns), and
+// the push kernel, which reads every block once (one column).
 #include <cuda_fp16.h>
 
 #include "digits.cuh"
@@ -273,28 +272,53 @@ struct DigArgs {
   const double* xs;
 };
 
+// One output tile's level sums [plane of the block][part of the column] -> this lane's (row, part) of the
+// product with the block (or with its adjoint).
+template <bool BWD>
+__device__ __forceinline__ double dig_flush(const float (&d)[2][2][4], double sc, int lane) {
+  const int t = lane & 3;
+  // levels 2t, 2t + 1 of (row g, row g + 8) x (re, im) as integers; F x or F^H x from the planes
+  long long q[2][2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int yr[2], yi[2];
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const int k = 2 * h + l;
+      const float fr = BWD ? d[0][0][k] + d[1][1][k] : d[0][0][k] - d[1][1][k];
+      const float fi = BWD ? d[0][1][k] - d[1][0][k] : d[0][1][k] + d[1][0][k];
+      yr[l] = __float2int_rn(fr * 0x1p24f);
+      yi[l] = __float2int_rn(fi * 0x1p24f);
+    }
+    q[h][0] = (long long)yr[0] * 256 + yr[1];
+    q[h][1] = (long long)yi[0] * 256 + yi[1];
+  }
+  // sum over the quad's levels: lanes t ^ 1 trade rows, lanes t ^ 2 trade parts
+  long long u[2];
+#pragma unroll
+  for (int part = 0; part < 2; ++part) {
+    const long long own = (t & 1) ? q[1][part] : q[0][part];
+    const long long got = __shfl_xor_sync(0xffffffffu, (t & 1) ? q[0][part] : q[1][part], 1);
+    u[part] = (t & 1) ? (got << 16) + own : (own << 16) + got;
+  }
+  const long long own = (t & 2) ? u[1] : u[0];
+  const long long got = __shfl_xor_sync(0xffffffffu, (t & 2) ? u[0] : u[1], 2);
+  const double hi = (double)((t & 2) ? got : own), lo = (double)((t & 2) ? own : got);
+  return fma(hi, sc * 0x1p-24, lo * (sc * 0x1p-56));
+}
+
 // One block product of the warp: the block's tiles times the columns' digit tables in `slab`, added to
-// acc[tile][column] (lane (g, t): row 16 tile + g + 8 (t & 1), part t >> 1).
+// acc[tile][column] (lane (g, t): row 16 tile + g + 8 (t & 1), part t >> 1).  flip: sigma3 on the operand and
+// the result.  w: the tile being multiplied; each of its loads is replaced by the next tile's as soon as it
+// is used, so that a tile's loads are in flight during the whole of the tile before it.
 template <int N, int C, bool BWD>
-__device__ __forceinline__ void dig_block(const uint4* __restrict__ blk, uint4 (&w)[8], uint32_t slab,
-                                          const float* const (&cr)[C], const double (&sc)[C],
-                                          double (&acc)[N / 16][C], bool flip_out) {
+__device__ __forceinline__ void dig_block(const uint4* __restrict__ blk, uint4 (&w)[8], uint32_t slab, const float (&corr)[C][4],
+                                          const double (&sc)[C], double (&acc)[N / 16][C], bool flip) {
   constexpr int NT = N / 16, RS = dig_row<N>(), PS = dig_part<N>(), SL = dig_slab<N>();
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const uint32_t fmask = flip ? 0x80008000u : 0u;
   // ldmatrix row of this lane: matrix lane / 8 = (part, upper half of k), level lane % 8
   const uint32_t lrow = slab + (uint32_t)((lane >> 4) * PS + (7 + (lane & 7)) * RS + ((lane >> 3) & 1) * 16);
-  float corr[C][4];
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    const float2 r = __ldg(reinterpret_cast<const float2*>(cr[c] + 2 * t));
-    const float2 i = __ldg(reinterpret_cast<const float2*>(cr[c] + 8 + 2 * t));
-    corr[c][0] = r.x;
-    corr[c][1] = r.y;
-    corr[c][2] = i.x;
-    corr[c][3] = i.y;
-  }
-  // w: the tile being multiplied; each of its loads is replaced by the next tile's as soon as it is used,
-  // so that a tile's loads are in flight during the whole of the tile before it
 #pragma unroll
   for (int O = 0; O < NT; ++O) {
     // sums [column][plane of the block][part of the column]
@@ -337,6 +361,14 @@ __device__ __forceinline__ void dig_block(const uint4* __restrict__ blk, uint4 (
         for (int c = 0; c < C; ++c) {
           uint32_t b[4];
           ldsm4(lrow + (uint32_t)(c * SL + K * 32 - p * RS), b);
+          if (16 * K >= N / 2) {  // sigma3: the second chirality's entries negated (N / 2 is a multiple of 8)
+            b[0] ^= fmask;
+            b[2] ^= fmask;
+          }
+          if (16 * K + 8 >= N / 2) {
+            b[1] ^= fmask;
+            b[3] ^= fmask;
+          }
           mma_f16(d[c][0][0], re, b[0], b[1]);
           mma_f16(d[c][0][1], re, b[2], b[3]);
           mma_f16(d[c][1][0], im, b[0], b[1]);
@@ -344,40 +376,41 @@ __device__ __forceinline__ void dig_block(const uint4* __restrict__ blk, uint4 (
         }
       }
     }
-    const bool neg = flip_out && (16 * O + g + 8 * (t & 1)) >= N / 2;
+    const bool neg = flip && (16 * O + g + 8 * (t & 1)) >= N / 2;
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      // levels 2t, 2t + 1 of (row g, row g + 8) x (re, im) as integers; F x or F^H x from the planes
-      long long q[2][2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        int yr[2], yi[2];
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          const int k = 2 * h + l;
-          const float fr = BWD ? d[c][0][0][k] + d[c][1][1][k] : d[c][0][0][k] - d[c][1][1][k];
-          const float fi = BWD ? d[c][0][1][k] - d[c][1][0][k] : d[c][0][1][k] + d[c][1][0][k];
-          yr[l] = __float2int_rn(fr * 0x1p24f);
-          yi[l] = __float2int_rn(fi * 0x1p24f);
-        }
-        q[h][0] = (long long)yr[0] * 256 + yr[1];
-        q[h][1] = (long long)yi[0] * 256 + yi[1];
-      }
-      // sum over the quad's levels: lanes t ^ 1 trade rows, lanes t ^ 2 trade parts
-      long long u[2];
-#pragma unroll
-      for (int part = 0; part < 2; ++part) {
-        const long long own = (t & 1) ? q[1][part] : q[0][part];
-        const long long got = __shfl_xor_sync(0xffffffffu, (t & 1) ? q[0][part] : q[1][part], 1);
-        u[part] = (t & 1) ? (got << 16) + own : (own << 16) + got;
-      }
-      const long long own = (t & 2) ? u[1] : u[0];
-      const long long got = __shfl_xor_sync(0xffffffffu, (t & 2) ? u[0] : u[1], 2);
-      const double hi = (double)((t & 2) ? got : own), lo = (double)((t & 2) ? own : got);
-      const double s = neg ? -sc[c] : sc[c];
-      acc[O][c] = fma(hi, s * 0x1p-24, fma(lo, s * 0x1p-56, acc[O][c]));
-    }
+    for (int c = 0; c < C; ++c) acc[O][c] += dig_flush<BWD>(d[c], neg ? -sc[c] : sc[c], lane);
   }
+}
+
+// Digit table of one column from its packed digits (asynchronous copies), its zero rows, its corrections.
+template <int N>
+__device__ __forceinline__ void dig_table(unsigned char* tab, const __half* xd, int lane) {
+  constexpr int CH = N / 8;  // 16-byte chunks per row
+#pragma unroll
+  for (int i0 = 0; i0 < 16 * CH; i0 += 32) {
+    const int i = i0 + lane, row = i / CH, kc = i % CH;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(
+                     tab + (row >> 3) * dig_part<N>() + (7 + (row & 7)) * dig_row<N>() + kc * 16)),
+                 "l"(reinterpret_cast<const uint4*>(xd) + i)
+                 : "memory");
+  }
+}
+template <int N, int C>
+__device__ __forceinline__ void dig_zero_rows(unsigned char* slab, int lane) {
+  constexpr int U = dig_row<N>() / 16;
+  for (int i = lane; i < C * 2 * 7 * U; i += 32) {
+    const int q = i / U, tbl = q / 7;  // tbl = (column, part)
+    *reinterpret_cast<uint4*>(slab + (tbl >> 1) * dig_slab<N>() + (tbl & 1) * dig_part<N>() + (q % 7) * dig_row<N>() +
+                              (i % U) * 16) = make_uint4(0, 0, 0, 0);
+  }
+}
+__device__ __forceinline__ void dig_corr(const float* xc, bool flip, float (&corr)[4], int lane) {
+  const float* p = xc + (flip ? 16 : 0) + 2 * (lane & 3);
+  const float2 r = __ldg(reinterpret_cast<const float2*>(p)), i = __ldg(reinterpret_cast<const float2*>(p + 8));
+  corr[0] = r.x;
+  corr[1] = r.y;
+  corr[2] = i.x;
+  corr[3] = i.y;
 }
 
 // The sums of the site's nine blocks on the FP64 pipe (scales marked NaN): eight lanes per row, by the
@@ -419,11 +452,46 @@ __device__ __noinline__ void dig_plain(const ApplyArgs& a, const int* ublk, cons
   }
 }
 
+// Entry e of column c of the site from the warps' sums `part`.
+template <int N, int C>
+__device__ __forceinline__ double2 dig_sum(const double* part, int bad, int c, int e) {
+  const double* pc = part + c * 2 * N + 2 * e;
+  double2 r = make_double2(pc[0], pc[1]);
+  if (!bad)
+#pragma unroll
+    for (int w = 1; w < kDW; ++w) r = cadd(r, make_double2(pc[w * C * 2 * N], pc[w * C * 2 * N + 1]));
+  return r;
+}
+
+// Mass term and epilogue of that entry: r the sum of the blocks, idx its index in a column.
+template <int N>
+__device__ __forceinline__ void dig_finish(const ApplyArgs& a, double2 r, int c, int e, size_t idx, size_t ldy,
+                                           double2 xs, double2 z) {
+  const double2 c0 = a.mode != APPLY_PLAIN ? a.coef[0] : make_double2(0.0, 0.0);
+  const double2 c1 = a.mode != APPLY_PLAIN ? a.coef[1] : make_double2(0.0, 0.0);
+  const double m = e < N / 2 ? a.mu : -a.mu;  // + i mu sigma3 x
+  r.x -= m * xs.y;
+  r.y += m * xs.x;
+  double2* y = static_cast<double2*>(a.y) + c * ldy + idx;
+  if (a.mode == APPLY_PLAIN) {
+    *y = r;
+  } else if (a.mode == APPLY_AXPBY) {
+    *y = cadd(cmul(c0, r), cmul(c1, z));
+  } else {
+    // chain step: s' = s - c0 D s ; acc = acc + c1 s'  (first: acc = c2 s + c1 s')
+    double2* accp = static_cast<double2*>(a.acc) + c * ldy + idx;
+    const double2 ac = a.mode == APPLY_POLY_FIRST ? cmul(a.coef[2], xs) : *accp;
+    r = csub(xs, cmul(c0, r));
+    *y = r;
+    *accp = cadd(ac, cmul(c1, r));
+  }
+}
+
 // One site of the columns x + c ldx (c < ncol <= C), results y + c ldy, addend z + c ldz (AXPBY).
 template <int N, int C>
 __device__ __forceinline__ void dig_site(const ApplyArgs& a, const DigArgs& dgt, const int site, const int ncol,
                                          const size_t ldx, const size_t ldy, const size_t ldz) {
-  constexpr int NT = N / 16, RS = dig_row<N>(), PS = dig_part<N>(), SL = dig_slab<N>();
+  constexpr int NT = N / 16, SL = dig_slab<N>();
   extern __shared__ __align__(16) unsigned char dsm[];  // [kDW][C] digit tables, then [kDW][C][2N] sums
   static_assert(SL >= 2 * N * 8, "the sums take the place of the digit tables");
   __shared__ int ublk[9], usrc[9];
@@ -443,33 +511,17 @@ __device__ __forceinline__ void dig_site(const ApplyArgs& a, const DigArgs& dgt,
   for (int p = 0; p < 8; ++p) w[p] = __ldg(bp + lane + p * 32);
   unsigned char* slab = dsm + (size_t)u * C * SL;
   const double bs = __ldg(dgt.bscale + blk);
-  const float* cr[C];
+  float corr[C][4];
   double sc[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const size_t rec = (size_t)(c < nc ? c : 0) * V + src;
-    const uint4* xd = reinterpret_cast<const uint4*>(dgt.xd + rec * dig_x_halves(N));
-    constexpr int CH = N / 8;  // 16-byte chunks per row
-#pragma unroll
-    for (int i0 = 0; i0 < 16 * CH; i0 += 32) {
-      const int i = i0 + lane, row = i / CH, kc = i % CH;
-      uint4 v = __ldg(xd + i);
-      if (flip && kc * 8 >= N / 2) {
-        v.x ^= 0x80008000u;
-        v.y ^= 0x80008000u;
-        v.z ^= 0x80008000u;
-        v.w ^= 0x80008000u;
-      }
-      *reinterpret_cast<uint4*>(slab + c * SL + (row >> 3) * PS + (7 + (row & 7)) * RS + kc * 16) = v;
-    }
-    cr[c] = dgt.xc + rec * kDigCorr + (flip ? 16 : 0);
+    dig_table<N>(slab + c * SL, dgt.xd + rec * dig_x_halves(N), lane);
+    dig_corr(dgt.xc + rec * kDigCorr, flip, corr[c], lane);
     sc[c] = bs * __ldg(dgt.xs + rec);
   }
-  for (int i = lane; i < C * 2 * 7 * (RS / 16); i += 32) {  // the zero rows
-    const int q = i / (RS / 16), tbl = q / 7;               // tbl = (column, part)
-    *reinterpret_cast<uint4*>(slab + (tbl >> 1) * SL + (tbl & 1) * PS + (q % 7) * RS + (i % (RS / 16)) * 16) =
-        make_uint4(0, 0, 0, 0);
-  }
+  dig_zero_rows<N, C>(slab, lane);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   int bad = 0;
 #pragma unroll
   for (int c = 0; c < C; ++c) bad |= !isfinite(sc[c]);
@@ -480,8 +532,8 @@ __device__ __forceinline__ void dig_site(const ApplyArgs& a, const DigArgs& dgt,
 #pragma unroll
     for (int c = 0; c < C; ++c) acc[O][c] = 0.0;
   const uint32_t sa = (uint32_t)__cvta_generic_to_shared(slab);
-  if (u < 5) dig_block<N, C, false>(bp, w, sa, cr, sc, acc, flip);
-  else dig_block<N, C, true>(bp, w, sa, cr, sc, acc, flip);
+  if (u < 5) dig_block<N, C, false>(bp, w, sa, corr, sc, acc, flip);
+  else dig_block<N, C, true>(bp, w, sa, corr, sc, acc, flip);
   bad = __syncthreads_or(bad);  // also: every warp is done with its tables
   double* part = reinterpret_cast<double*>(dsm);  // [warp][column][2 row + part]
   if (!bad) {
@@ -495,42 +547,237 @@ __device__ __forceinline__ void dig_site(const ApplyArgs& a, const DigArgs& dgt,
       dig_plain<N>(a, ublk, usrc, static_cast<const double2*>(a.x) + (size_t)c * ldx, part + c * 2 * N);
   }
   __syncthreads();
-  const double2 c0 = a.mode != APPLY_PLAIN ? a.coef[0] : make_double2(0.0, 0.0);
-  const double2 c1 = a.mode != APPLY_PLAIN ? a.coef[1] : make_double2(0.0, 0.0);
-  const double2 c2 = a.mode == APPLY_POLY_FIRST ? a.coef[2] : make_double2(0.0, 0.0);
   for (int i = threadIdx.x; i < nc * N; i += blockDim.x) {
     const int c = i / N, e = i % N;
     const size_t idx = (size_t)site * N + e;
-    const double* pc = part + c * 2 * N + 2 * e;
-    double2 r = make_double2(pc[0], pc[1]);
-    if (!bad)
-#pragma unroll
-      for (int w = 1; w < kDW; ++w) r = cadd(r, make_double2(pc[w * C * 2 * N], pc[w * C * 2 * N + 1]));
     const double2 xs = static_cast<const double2*>(a.x)[c * ldx + idx];
-    const double m = e < N / 2 ? a.mu : -a.mu;  // + i mu sigma3 x
-    r.x -= m * xs.y;
-    r.y += m * xs.x;
-    double2* y = static_cast<double2*>(a.y) + c * ldy + idx;
-    if (a.mode == APPLY_PLAIN) {
-      *y = r;
-    } else if (a.mode == APPLY_AXPBY) {
-      *y = cadd(cmul(c0, r), cmul(c1, static_cast<const double2*>(a.z)[c * ldz + idx]));
-    } else {
-      // chain step: s' = s - c0 D s ; acc = acc + c1 s'  (first: acc = c2 s + c1 s')
-      double2* accp = static_cast<double2*>(a.acc) + c * ldy + idx;
-      const double2 ac = a.mode == APPLY_POLY_FIRST ? cmul(c2, xs) : *accp;
-      r = csub(xs, cmul(c0, r));
-      *y = r;
-      *accp = cadd(ac, cmul(c1, r));
+    const double2 z = a.mode == APPLY_AXPBY ? static_cast<const double2*>(a.z)[c * ldz + idx] : xs;
+    dig_finish<N>(a, dig_sum<N, C>(part, bad, c, e), c, e, idx, ldy, xs, z);
+  }
+}
+
+// One CTA per site: two columns, and small lattices.
+template <int N, int C>
+__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, C)) k_site_digits(
+    const __grid_constant__ ApplyArgs a, const __grid_constant__ DigArgs dgt, int ncol, long long ldc) {
+  if (a.stop != nullptr && *a.stop) return;
+  dig_site<N, C>(a, dgt, blockIdx.x, ncol, ldc, ldc, ldc);
+}
+
+// ------------------------------------------------------------------ one column: every block once
+// The pull kernel reads a hop block twice, as a forward hop and transposed for the site in front: nine blocks per
+// site through L2, of which about a quarter hit (16^4, n = 48: 3.3 ms at 4.9 TB/s of DRAM).  Here the four warps of site x multiply each tile of F_{x,mu} both ways while it is in registers: forward with
+// the digits of x + mu into the site's own sum, transposed with the site's digits into the push for x + mu,
+//   P_x = A_x v_x + sum_mu F_{x,mu} v_{x+mu},   T_mu[x] = sigma3 F_{x,mu}^H sigma3 v_x,
+// and k_push_finish adds y_z = P_z + sum_mu T_mu[z - mu], the mass term and the epilogue.  The self block's tile
+// rows are dealt to the warps.
+constexpr int kPW = 4;
+
+__device__ __forceinline__ void dig_start(float (&d)[2][2][4], const float (&corr)[4]) {
+#pragma unroll
+  for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      d[pl][0][k] = corr[k & 1];
+      d[pl][1][k] = corr[2 + (k & 1)];
+    }
+}
+
+// planes of the four A words times the level operand at `addr`
+__device__ __forceinline__ void dig_mul(const uint32_t (&a)[4], uint32_t addr, uint32_t flo, uint32_t fhi,
+                                        float (&d)[2][2][4]) {
+  uint32_t re[4], im[4], b[4];
+  ldsm4(addr, b);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    re[k] = __byte_perm(a[k], 0u, 0x4240);
+    im[k] = __byte_perm(a[k], 0u, 0x4341);
+  }
+  b[0] ^= flo;
+  b[2] ^= flo;
+  b[1] ^= fhi;
+  b[3] ^= fhi;
+  mma_f16(d[0][0], re, b[0], b[1]);
+  mma_f16(d[0][1], re, b[2], b[3]);
+  mma_f16(d[1][0], im, b[0], b[1]);
+  mma_f16(d[1][1], im, b[2], b[3]);
+}
+
+template <int N>
+__global__ void __launch_bounds__(32 * kPW, 4) k_push_digits(const __grid_constant__ ApplyArgs a,
+                                                             const __grid_constant__ DigArgs dgt) {
+  constexpr int NT = N / 16, RS = dig_row<N>(), PS = dig_part<N>(), SL = dig_slab<N>();
+  extern __shared__ __align__(16) unsigned char dsm[];  // digit tables (own site, x + mu per warp), tile rings
+  __shared__ double part[kPW][2 * N];
+  __shared__ int srcs[kPW];
+  if (a.stop != nullptr && *a.stop) return;
+  const int mu = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int site = blockIdx.x, V = a.V;
+  const bool adj = a.adjoint != 0;
+  const int src = __ldg(a.nb + site * 8 + mu);
+  const uint4* self = dgt.dig + (size_t)site * 5 * NT * NT * 256 + lane;
+  const uint4* hop = self + (size_t)(1 + mu) * NT * NT * 256;
+  // Tiles of the warp in order: the hop's, then its tile row of the self block; two are in flight in the
+  // warp's ring (registers would hold one, and leave room for three CTAs per SM instead of four).
+  uint4* ring = reinterpret_cast<uint4*>(dsm + (size_t)(1 + kPW) * SL) + (size_t)mu * 2 * 256 + lane;
+  const int tiles = NT * NT + (mu < NT ? NT : 0);
+  auto fetch = [&](int i) {
+    if (i < tiles) {
+      const uint4* from = i < NT * NT ? hop + i * 256 : self + (size_t)(mu * NT + i - NT * NT) * 256;
+      const uint32_t to = (uint32_t)__cvta_generic_to_shared(ring + (i & 1) * 256);
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + p * 512), "l"(from + p * 32) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (lane == 0) srcs[mu] = src;
+  unsigned char* own = dsm;
+  unsigned char* nbr = dsm + (size_t)(1 + mu) * SL;
+  if (mu == 0) dig_table<N>(own, dgt.xd + (size_t)site * dig_x_halves(N), lane);
+  dig_table<N>(nbr, dgt.xd + (size_t)src * dig_x_halves(N), lane);
+  if (mu == 0) dig_zero_rows<N, 1>(own, lane);
+  dig_zero_rows<N, 1>(nbr, lane);
+  const double bh = __ldg(dgt.bscale + (size_t)site * 5 + 1 + mu), b0 = __ldg(dgt.bscale + (size_t)site * 5);
+  const double x0 = __ldg(dgt.xs + site), xn = __ldg(dgt.xs + src);
+  const double sf = bh * xn, sb = bh * x0, ss = b0 * x0;
+  float cf[4], cb[4];
+  dig_corr(dgt.xc + (size_t)src * kDigCorr, adj, cf, lane);
+  dig_corr(dgt.xc + (size_t)site * kDigCorr, !adj, cb, lane);
+  asm volatile("cp.async.commit_group;" ::: "memory");  // the tables, then the first two tiles
+  fetch(0);
+  fetch(1);
+  asm volatile("cp.async.wait_group 2;" ::: "memory");
+  const int bad = __syncthreads_or(!isfinite(sf) || !isfinite(sb) || !isfinite(ss));
+  double2* P = static_cast<double2*>(a.part) + (size_t)site * N;
+  double2* T = static_cast<double2*>(a.push) + ((size_t)mu * V + site) * N;
+  if (!bad) {
+    const uint32_t off = (uint32_t)((lane >> 4) * PS + (7 + (lane & 7)) * RS + ((lane >> 3) & 1) * 16);
+    const uint32_t of = (uint32_t)__cvta_generic_to_shared(nbr) + off;
+    const uint32_t ob = (uint32_t)__cvta_generic_to_shared(own) + off;
+    const uint32_t mf = adj ? 0x80008000u : 0u, mb = adj ? 0u : 0x80008000u;
+    double pull[NT];
+    float db[NT][2][2][4];
+#pragma unroll
+    for (int W = 0; W < NT; ++W) dig_start(db[W], cb);
+#pragma unroll
+    for (int U = 0; U < NT; ++U) {
+      float df[2][2][4];
+      dig_start(df, cf);
+#pragma unroll
+      for (int W = 0; W < NT; ++W) {
+        const int i = U * NT + W;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          const uint4 w = ring[(i & 1) * 256 + p * 32];
+          const uint32_t af[4] = {w.x, w.y, w.z, w.w};
+          const uint32_t ab[4] = {movmatrix(w.x), movmatrix(w.z), movmatrix(w.y), movmatrix(w.w)};
+          dig_mul(af, of + (uint32_t)(W * 32 - p * RS), 16 * W >= N / 2 ? mf : 0u, 16 * W + 8 >= N / 2 ? mf : 0u, df);
+          dig_mul(ab, ob + (uint32_t)(U * 32 - p * RS), 16 * U >= N / 2 ? mb : 0u, 16 * U + 8 >= N / 2 ? mb : 0u, db[W]);
+        }
+        __syncwarp();  // the slot has been read
+        fetch(i + 2);
+      }
+      const bool neg = adj && 16 * U + g + 8 * (t & 1) >= N / 2;
+      pull[U] = dig_flush<false>(df, neg ? -sf : sf, lane);
+    }
+#pragma unroll
+    for (int W = 0; W < NT; ++W) {
+      const int row = 16 * W + g + 8 * (t & 1);
+      const bool neg = !adj && row >= N / 2;
+      reinterpret_cast<double*>(T + row)[t >> 1] = dig_flush<true>(db[W], neg ? -sb : sb, lane);
+    }
+    if (mu < NT) {  // tile row mu of the self block
+      float ds[2][2][4], cs[4];
+      dig_corr(dgt.xc + (size_t)site * kDigCorr, adj, cs, lane);
+      dig_start(ds, cs);
+#pragma unroll
+      for (int W = 0; W < NT; ++W) {
+        const int i = NT * NT + W;
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          const uint4 w = ring[(i & 1) * 256 + p * 32];
+          const uint32_t af[4] = {w.x, w.y, w.z, w.w};
+          dig_mul(af, ob + (uint32_t)(W * 32 - p * RS), 16 * W >= N / 2 ? mf : 0u, 16 * W + 8 >= N / 2 ? mf : 0u, ds);
+        }
+        __syncwarp();
+        fetch(i + 2);
+      }
+      const bool neg = adj && 16 * mu + g + 8 * (t & 1) >= N / 2;
+      const double v = dig_flush<false>(ds, neg ? -ss : ss, lane);
+#pragma unroll
+      for (int U = 0; U < NT; ++U)
+        if (U == mu) pull[U] += v;
+    }
+#pragma unroll
+    for (int U = 0; U < NT; ++U) part[mu][2 * (16 * U + g + 8 * (t & 1)) + (t >> 1)] = pull[U];
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * N; i += blockDim.x)
+      reinterpret_cast<double*>(P)[i] = (part[0][i] + part[1][i]) + (part[2][i] + part[3][i]);
+  } else {
+    // on the FP64 pipe: warp q of four lanes per row; P by rows, then the four pushes by columns
+    const double2* B = static_cast<const double2*>(a.blocks) + (size_t)site * 5 * N * N;
+    const double2* X = static_cast<const double2*>(a.x);
+    auto sgn = [&](double2 v, bool on, int j) { return on && j >= N / 2 ? make_double2(-v.x, -v.y) : v; };
+    const int l4 = threadIdx.x & 3;
+#pragma unroll 1
+    for (int r0 = 0; r0 < N; r0 += 8 * kPW) {
+      const int r = r0 + (threadIdx.x >> 2), row = r < N ? r : N - 1;
+      double2 y = make_double2(0.0, 0.0);
+#pragma unroll 1
+      for (int u = 0; u < 5; ++u) {
+        const double2* v = X + (size_t)(u == 0 ? site : srcs[u == 0 ? 0 : u - 1]) * N;
+        double2 p = make_double2(0.0, 0.0), q = p;
+#pragma unroll 1
+        for (int j = l4; j < N; j += 8) {
+          cfma(p, B[(size_t)u * N * N + row * N + j], sgn(v[j], adj, j));
+          if (j + 4 < N) cfma(q, B[(size_t)u * N * N + row * N + j + 4], sgn(v[j + 4], adj, j + 4));
+        }
+        y = cadd(y, cadd(p, q));
+      }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        y.x += __shfl_xor_sync(0xffffffffu, y.x, o);
+        y.y += __shfl_xor_sync(0xffffffffu, y.y, o);
+      }
+      if (l4 == 0 && r < N) P[r] = sgn(y, adj, r);
+#pragma unroll 1
+      for (int m = 0; m < 4; ++m) {
+        double2 p = make_double2(0.0, 0.0);
+#pragma unroll 1
+        for (int i = l4; i < N; i += 4)
+          cfma_conj(p, B[(size_t)(1 + m) * N * N + i * N + row], sgn(X[(size_t)site * N + i], !adj, i));
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+          p.x += __shfl_xor_sync(0xffffffffu, p.x, o);
+          p.y += __shfl_xor_sync(0xffffffffu, p.y, o);
+        }
+        if (l4 == 0 && r < N) static_cast<double2*>(a.push)[((size_t)m * V + site) * N + r] = sgn(p, !adj, r);
+      }
     }
   }
 }
 
-template <int N, int C>
-__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, C)) k_apply_digits(
-    const __grid_constant__ ApplyArgs a, const __grid_constant__ DigArgs dgt, int ncol, long long ldc) {
+// y_z = P_z + T_0[z-0] + .. + T_3[z-3] + i mu sigma3 x_z, then the epilogue; one thread per entry.
+template <int N>
+__global__ void __launch_bounds__(256) k_push_finish(const __grid_constant__ ApplyArgs a) {
   if (a.stop != nullptr && *a.stop) return;
-  dig_site<N, C>(a, dgt, blockIdx.x, ncol, ldc, ldc, ldc);
+  const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
+  if (i >= (size_t)a.V * N) return;
+  const int z = (int)(i / N), e = (int)(i % N);
+  const double2* T = static_cast<const double2*>(a.push);
+  double2 t[4];
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) t[mu] = T[((size_t)mu * a.V + __ldg(a.nb + z * 8 + 4 + mu)) * N + e];
+  double2 r = static_cast<const double2*>(a.part)[i];
+  const double2 xs = static_cast<const double2*>(a.x)[i];
+  const double2 zv = a.mode == APPLY_AXPBY ? static_cast<const double2*>(a.z)[i] : xs;
+  r = cadd(r, cadd(cadd(t[0], t[1]), cadd(t[2], t[3])));
+  dig_finish<N>(a, r, 0, e, i, 0, xs, zv);
 }
 
 // Batched FP64 residual r = b - D x of every pass with an unfinished column (coef: {-1, +1}).
@@ -563,17 +810,53 @@ __global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, kDigCols)) kb_resi
   dig_site<N, kDigCols>(a, d, site, p.cols, p.ldx, p.ldy, p.ldx);
 }
 
-template <int N, int C>
-int launch_dig_nc(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, cudaStream_t s) {
-  constexpr size_t smem = (size_t)kDW * C * dig_slab<N>();
-  if (smem > 32 * 1024) {  // with the static tables beyond the default 48 KB
-    static bool attr = false;
-    if (!attr) {
-      COARSE_CUDA(cudaFuncSetAttribute(k_apply_digits<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      attr = true;
-    }
+template <class K>
+int dig_attr(K kernel, size_t bytes) {
+  COARSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  return COARSE_OK;
+}
+
+// Two columns: one CTA per site (they share the block operand's loads and byte permutations; 8^4, n = 48:
+// 404 us for two against 2 x 240 us).
+template <int N>
+int launch_dig_2(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, cudaStream_t s) {
+  constexpr size_t smem = (size_t)kDW * 2 * dig_slab<N>();
+  static bool attr = false;
+  if (!attr) {
+    const int rc = dig_attr(k_site_digits<N, 2>, smem);
+    if (rc != COARSE_OK) return rc;
+    attr = true;
   }
-  k_apply_digits<N, C><<<a.V, 32 * kDW, smem, s>>>(a, d, ncol, ldc);
+  k_site_digits<N, 2><<<a.V, 32 * kDW, smem, s>>>(a, d, ncol, ldc);
+  note_launch();
+  COARSE_CUDA(cudaGetLastError());
+  return COARSE_OK;
+}
+
+// One column.  From kPushSites sites on every block once (push kernel and its finish); below, where the lattice
+// does not fill the chip, one launch of the pull kernel.  Both sides, us: 4^4 n = 16 15 / 19, n = 48 26 / 29;
+// 6^4 n = 16 28 / 27, n = 32 51 / 48, n = 48 74 / 74; 8^4 n = 32 132 / 95, n = 48 218 / 167; 16^4 n = 48
+// 3330 / 2240 (1800 at the copy bandwidth).
+constexpr int kPushSites = 1024;
+template <int N>
+int launch_dig_1(const ApplyArgs& a, const DigArgs& d, cudaStream_t s) {
+  static bool attr = false;
+  constexpr size_t ss = (size_t)kDW * dig_slab<N>(), su = (size_t)(kPW + 1) * dig_slab<N>() + (size_t)kPW * 2 * 4096;
+  if (!attr) {
+    int rc = dig_attr(k_push_digits<N>, su);
+    if (rc == COARSE_OK) rc = dig_attr(k_site_digits<N, 1>, ss);
+    if (rc != COARSE_OK) return rc;
+    attr = true;
+  }
+  if (a.V >= kPushSites) {
+    k_push_digits<N><<<a.V, 32 * kPW, su, s>>>(a, d);
+    note_launch();
+    COARSE_CUDA(cudaGetLastError());
+    const size_t total = (size_t)a.V * N;
+    k_push_finish<N><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(a);
+  } else {
+    k_site_digits<N, 1><<<a.V, 32 * kDW, ss, s>>>(a, d, 1, 0);
+  }
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   return COARSE_OK;
@@ -591,10 +874,7 @@ int launch_dig_n(const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {
   k_dig_x<N><<<dim3((a.V + 3) / 4, ncol), 128, 0, s>>>(static_cast<const double2*>(a.x), ldc, a.V, x.xd, x.xc, x.xs, a.stop);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
-  // two columns share the block operand's loads and byte permutations (8^4, n = 48: 427 us for two
-  // columns against 2 x 240 us); four would need 168 registers and spill (1008 us)
-  if (ncol == 1) return launch_dig_nc<N, 1>(a, d, ncol, ldc, s);
-  return launch_dig_nc<N, 2>(a, d, ncol, ldc, s);
+  return ncol == 1 ? launch_dig_1<N>(a, d, s) : launch_dig_2<N>(a, d, ncol, ldc, s);
 }
 
 template <int N>

@@ -62,7 +62,9 @@ def columns(cols, N, seed):
 
 
 @pytest.mark.parametrize("dims,nv,cols", [((2, 2, 2, 2), 8, 1), ((3, 2, 5, 2), 8, 4), ((2, 3, 2, 4), 16, 1),
-                                          ((5, 2, 2, 3), 16, 3), ((2, 2, 3, 2), 24, 1), ((3, 3, 2, 2), 24, 5)])
+                                          ((5, 2, 2, 3), 16, 3), ((2, 2, 3, 2), 24, 1), ((3, 3, 2, 2), 24, 5),
+                                          # from 1024 sites on one column takes the kernel that reads a block once
+                                          ((4, 4, 8, 8), 8, 1), ((7, 5, 6, 5), 16, 1), ((3, 7, 7, 7), 24, 1)])
 @pytest.mark.parametrize("adjoint", [False, True])
 def test_digit_products_match_oracle(dims, nv, cols, adjoint):
     s, f = blocks(dims, nv, 11)
@@ -100,15 +102,38 @@ def test_digit_products_hard_values(nv, what):
     check(s, f, dims, nv, 0.0, X, False, f"{what} nv={nv}")
 
 
-def test_digit_products_non_finite():
-    dims, nv = (4, 2, 4, 2), 8
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_digit_products_hard_values_push(adjoint):
+    """The hard values above on a lattice of the push kernel."""
+    dims, nv = (5, 6, 7, 5), 8
+    s, f = blocks(dims, nv, 25)
+    V, n = s.shape[0], 2 * nv
+    X = columns(1, V * n, 26)
+    x = X[0].reshape(V, n)
+    f[7, 2] = 0.0
+    x[3] = 0.0
+    x[5, nv:] = 0.0
+    x[20, :nv] *= 2.0 ** -40
+    f[40, 1, 3] *= 2.0 ** -30
+    f[60, 3, :, 5] *= 2.0 ** -30
+    x[100] *= 2.0 ** -980
+    f[200, 0] *= 2.0 ** 930
+    check(s, f, dims, nv, 0.02, X, adjoint, "push, hard values")
+
+
+@pytest.mark.parametrize("dims", [(4, 2, 4, 2), (5, 6, 7, 5)])
+def test_digit_products_non_finite(dims):
+    nv = 8
     s, f = blocks(dims, nv, 31)
     V, n = s.shape[0], 2 * nv
     X = columns(3, V * n, 32)
     X[0].reshape(V, n)[5, 3] = np.inf
     X[1].reshape(V, n)[0, 9] = np.nan
     dev = device_op(s, f, dims, nv, 0.0, 3)
-    y = dev.apply(torch.from_numpy(X).cuda(), precision=0).cpu().numpy().reshape(3, V, n)
+    if V < 1024:
+        y = dev.apply(torch.from_numpy(X).cuda(), precision=0).cpu().numpy().reshape(3, V, n)
+    else:
+        y = np.stack([dev.apply(torch.from_numpy(x).cuda(), precision=0).cpu().numpy().reshape(V, n) for x in X])
     nb = neighbours(dims)
     for c, site in ((0, 5), (1, 0)):
         hit = np.zeros(V, dtype=bool)
