@@ -22,6 +22,7 @@
 #include "batch.cuh"
 #include "mcol.cuh"
 #include "oddeven.cuh"
+#include "site8.cuh"
 
 namespace coarse {
 namespace {
@@ -93,6 +94,8 @@ template <int N> struct Piece<N, cbf16> {
 template <int N, class BT, bool ADD>
 __device__ __forceinline__ void mul_rows(const Piece<N, BT>& p, const float2* tab, float* out, int r0, int c0, int cs,
                                          int R, bool flip, int lane) {
+  // sigma3 of the operand: the second chirality's columns come first, then the sums change sign once
+  constexpr bool kFlips = sizeof(BT) == 8;  // columns of entry q >= N/2 for every lane or for none
   constexpr int Q = N / 4;
   const int g = lane >> 2, t = lane & 3;
   float2 e[2][Q];
@@ -109,7 +112,14 @@ __device__ __forceinline__ void mul_rows(const Piece<N, BT>& p, const float2* ta
 #pragma unroll
     for (int h = 0; h < 2; ++h) F1[h] = F2[h] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int q = 0; q < Q; q += 2) {  // entries q, q + 1 are neighbours
+    for (int i = 0; i < Q; i += 2) {
+      const int q = kFlips ? (i + Q / 2) % Q : i;  // entries q, q + 1 are neighbours
+      if (kFlips && i == Q / 2 && flip)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          F1[h] = make_float2(-F1[h].x, -F1[h].y);
+          F2[h] = make_float2(-F2[h].x, -F2[h].y);
+        }
       const float4 ww = *reinterpret_cast<const float4*>(w + Piece<N, BT>::col(q, t));
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -155,7 +165,14 @@ __device__ __forceinline__ void mul_cols(const Piece<N, BT>& p, const float2* ta
 #pragma unroll
     for (int j = 0; j < 2; ++j) B1[j] = B2[j] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < Q; k += 2) {
+    for (int i = 0; i < Q; i += 2) {
+      const int k = (i + Q / 2) % Q;  // rows of the second chirality first (sigma3 of the operand)
+      if (i == Q / 2 && flip)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          B1[j] = make_float2(-B1[j].x, -B1[j].y);
+          B2[j] = make_float2(-B2[j].x, -B2[j].y);
+        }
       const float4 ww = *reinterpret_cast<const float4*>(w + 4 * k);
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
@@ -191,15 +208,18 @@ struct McSite {
   int adj;          // D^H = sigma3 D sigma3 on the forward hops' side
 };
 
+// The R columns' entries at `off` into tab[column][N], by asynchronous copies (a loop of loads and stores would
+// expose one memory latency per round).
 template <int N>
-__device__ __forceinline__ void fill_table(float2* tab, const float2* const* vp, size_t off, int R, bool flip,
-                                           int lane) {
+__device__ __forceinline__ void fill_table(float2* tab, const float2* const* vp, size_t off, int R, int lane) {
   for (int i = lane; i < R * (N / 2); i += 32) {
     const int c = i / (N / 2), e = 2 * (i % (N / 2));
-    float4 v = *reinterpret_cast<const float4*>(vp[c] + off + e);
-    if (flip && e >= N / 2) v = make_float4(-v.x, -v.y, -v.z, -v.w);
-    *reinterpret_cast<float4*>(tab + c * N + e) = v;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(tab + c * N + e)),
+                 "l"(vp[c] + off + e)
+                 : "memory");
   }
+  asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
 // The two hops of the warp's direction into hp[c][row] of the warp; `tail` receives the warp's piece of the
@@ -215,8 +235,9 @@ __device__ __forceinline__ void mc_hops(const McSite& s, int mu, const int4 rec,
   Piece<N, BT> p, nx;
   p.load_rows(fb, 0, lane);
   float2* tab2 = tab + (size_t)kMW * s.R * N;
-  fill_table<N>(tab, vp, (size_t)rec.x * N, s.R, s.adj, lane);
-  fill_table<N>(tab2, vp, (size_t)rec.z * N, s.R, !s.adj, lane);
+  fill_table<N>(tab, vp, (size_t)rec.x * N, s.R, lane);
+  fill_table<N>(tab2, vp, (size_t)rec.z * N, s.R, lane);
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < NP; ++k) {
@@ -225,6 +246,7 @@ __device__ __forceinline__ void mc_hops(const McSite& s, int mu, const int4 rec,
     mul_rows<N, BT, false>(p, tab, hp, 16 * k, 0, 1, s.R, s.adj, lane);
     p = nx;
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncwarp();
 #pragma unroll
   for (int k = 0; k < NP; ++k) {
@@ -321,6 +343,33 @@ __device__ __forceinline__ McItem load_item(const McItem* p) {
   return it;
 }
 
+// The epilogue's operands of this thread's entries (thread + k * threads of [column][N]), loaded together.
+template <int N>
+struct McTail {
+  static constexpr int IT = (kMcCols * N + 32 * kMW - 1) / (32 * kMW);
+  float2 xs[IT], ac[IT];
+  __device__ __forceinline__ void load(const McPtrs& P, const McPhase& b, size_t off, int R) {
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int i = threadIdx.x + 32 * kMW * k, c = i / N;
+      xs[k] = ac[k] = make_float2(0.f, 0.f);
+      if (i < R * N && b.bsel != BS_NONE) xs[k] = P.base[c][off + i % N];
+      if (i < R * N && b.mode == APPLY_POLY) ac[k] = P.acc[c][off + i % N];
+    }
+  }
+  // u[column][N]: the inverse block's product
+  __device__ __forceinline__ void finish(const McPtrs& P, const McPhase& b, size_t off, int R, const float2* u) const {
+#pragma unroll
+    for (int k = 0; k < IT; ++k) {
+      const int i = threadIdx.x + 32 * kMW * k, c = i / N;
+      if (i >= R * N) break;
+      const size_t idx = off + i % N;
+      const float2 r = b.bsel != BS_NONE ? csub(xs[k], u[i]) : u[i];
+      s8_finish(b.mode, r, xs[k], ac[k], P.coef[c], P.y[c] + idx, P.acc[c] + idx);
+    }
+  }
+};
+
 // Batched half apply: CTA -> (operator's column chunk, output site); columns whose gate is closed drop out.
 template <int N, class BT>
 __global__ void __launch_bounds__(32 * kMW) kb_eo_mc(const __grid_constant__ McPhase b) {
@@ -360,19 +409,12 @@ __global__ void __launch_bounds__(32 * kMW) kb_eo_mc(const __grid_constant__ McP
     if (b.zsel != BS_NONE) g = csub(P.z[c][off + e], g);
     tabs[i] = g;
   }
+  McTail<N> ends;
+  ends.load(P, b, off, R);
   __syncthreads();
   mc_block<N, BT, false>(tail, tabs, hp, R, false, warp, lane);
   __syncthreads();
-  for (int i = threadIdx.x; i < R * N; i += blockDim.x) {
-    const int c = i / N;
-    const size_t idx = off + i % N;
-    float2 r = reinterpret_cast<const float2*>(hp)[i], xs = make_float2(0.f, 0.f);
-    if (b.bsel != BS_NONE) {
-      xs = P.base[c][idx];
-      r = csub(xs, r);
-    }
-    mc_finish(b.mode, r, xs, P.coef[c], P.y[c] + idx, P.acc[c] + idx);
-  }
+  ends.finish(P, b, off, R, reinterpret_cast<const float2*>(hp));
 }
 
 // ------------------------------------------------------------- BF16 blocks on the tensor cores
@@ -431,15 +473,28 @@ __device__ __forceinline__ void put_split(unsigned char* tab, int c, int j, cons
 template <int N>
 __device__ __forceinline__ void fill_split(unsigned char* tab, const float2* const* vp, size_t off, int R, bool flip,
                                            int lane) {
-  for (int i = lane; i < R * (N / 4); i += 32) {
-    const int c = i / (N / 4), j = 4 * (i % (N / 4));
-    const float4* p = reinterpret_cast<const float4*>(vp[c] + off + j);
-    const float4 u = p[0], w = p[1];
-    float2 v[4] = {make_float2(u.x, u.y), make_float2(u.z, u.w), make_float2(w.x, w.y), make_float2(w.z, w.w)};
-    if (flip && j >= N / 2)
+  constexpr int IT = (kMcCols * (N / 4) + 31) / 32;
+  float4 u[IT], w[IT];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = make_float2(-v[k].x, -v[k].y);
-    put_split<N>(tab, c, j, v);
+  for (int k = 0; k < IT; ++k) {  // every load on its way before the first is used
+    const int i = lane + 32 * k, c = i / (N / 4), j = 4 * (i % (N / 4));
+    if (i < R * (N / 4)) {
+      const float4* p = reinterpret_cast<const float4*>(vp[c] + off + j);
+      u[k] = p[0];
+      w[k] = p[1];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < IT; ++k) {
+    const int i = lane + 32 * k, c = i / (N / 4), j = 4 * (i % (N / 4));
+    if (i < R * (N / 4)) {
+      float2 v[4] = {make_float2(u[k].x, u[k].y), make_float2(u[k].z, u[k].w), make_float2(w[k].x, w[k].y),
+                     make_float2(w[k].z, w[k].w)};
+      if (flip && j >= N / 2)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = make_float2(-v[q].x, -v[q].y);
+      put_split<N>(tab, c, j, v);
+    }
   }
 }
 
@@ -636,6 +691,8 @@ __global__ void __launch_bounds__(32 * kMW, N == 48 ? 4 : 6) kb_eo_mma(const __g
     }
     put_split<N>(mc_sm, c, j, v);
   }
+  McTail<N> ends;
+  ends.load(P, b, off, R);
   __syncthreads();
   if (warp < NT) {
     const uint32_t lrow = lane_row((uint32_t)__cvta_generic_to_shared(mc_sm), split_row<N>(), lane);
@@ -646,16 +703,7 @@ __global__ void __launch_bounds__(32 * kMW, N == 48 ? 4 : 6) kb_eo_mma(const __g
     put_sums<N, false, false>(d, hp, warp, R, 1.f, lane);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < R * N; i += blockDim.x) {
-    const int c = i / N;
-    const size_t idx = off + i % N;
-    float2 r = hp[i], xs = make_float2(0.f, 0.f);
-    if (b.bsel != BS_NONE) {
-      xs = P.base[c][idx];
-      r = csub(xs, r);
-    }
-    mc_finish(b.mode, r, xs, P.coef[c], P.y[c] + idx, P.acc[c] + idx);
-  }
+  ends.finish(P, b, off, R, hp);
 }
 
 // Full stencil of one site for the columns in vp (shared memory); returns with the sums in hp.
@@ -668,7 +716,8 @@ __device__ __forceinline__ void mc_full_site(const McSite& s, const int* nb, con
   float* h = hp + (size_t)warp * s.R * 2 * N;
   Piece<N, BT> tail;
   mc_hops<N, BT>(s, warp, rec, vp, tab, h, static_cast<const BT*>(s.blocks) + (size_t)s.x * 5 * N * N, tail, lane);
-  fill_table<N>(tab, vp, (size_t)s.x * N, s.R, s.adj, lane);
+  fill_table<N>(tab, vp, (size_t)s.x * N, s.R, lane);
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncwarp();
   mc_block<N, BT, true>(tail, tab, h, s.R, s.adj, warp, lane);
   __syncthreads();
