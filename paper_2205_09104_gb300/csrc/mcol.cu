@@ -435,7 +435,8 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 
 constexpr int kMmaTiles = kMcCols / 4;  // column tiles of one pass
 // Split table of one hop: [column tile][split][8 rows (column, part)][N], rows padded to an odd number of
-// 16-byte units (conflict-free ldmatrix).
+// 16-byte units (conflict-free ldmatrix).  A row holds the entries 4i, 4i + 1 of all i, then 4i + 2, 4i + 3, so
+// that the lanes of a fill, four entries each, write neighbouring words.
 template <int N> constexpr int split_row() { return 2 * N + 16; }
 template <int N> constexpr int split_tile() { return 3 * 8 * split_row<N>(); }
 template <int N> constexpr size_t mma_smem(int R) {
@@ -456,7 +457,7 @@ __device__ __forceinline__ void split3(float v0, float v1, uint32_t (&o)[3]) {
 // entries j .. j + 3 (j a multiple of 4) of column c
 template <int N>
 __device__ __forceinline__ void put_split(unsigned char* tab, int c, int j, const float2 (&v)[4]) {
-  unsigned char* o = tab + (c >> 2) * split_tile<N>() + 2 * (c & 3) * split_row<N>() + (j & ~15) * 2 + (j & 15);
+  unsigned char* o = tab + (c >> 2) * split_tile<N>() + 2 * (c & 3) * split_row<N>() + j;
   uint32_t a[3], b[3];
 #pragma unroll
   for (int part = 0; part < 2; ++part) {
@@ -465,7 +466,7 @@ __device__ __forceinline__ void put_split(unsigned char* tab, int c, int j, cons
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       *reinterpret_cast<uint32_t*>(o + (k * 8 + part) * split_row<N>()) = a[k];
-      *reinterpret_cast<uint32_t*>(o + (k * 8 + part) * split_row<N>() + 16) = b[k];
+      *reinterpret_cast<uint32_t*>(o + (k * 8 + part) * split_row<N>() + N) = b[k];
     }
   }
 }
@@ -523,8 +524,9 @@ __device__ __forceinline__ void load_tile(uint32_t (&u)[8], const cbf16* blk, in
   }
 }
 
-__device__ __forceinline__ uint32_t lane_row(uint32_t tab, int rs, int lane) {
-  return tab + (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * rs + ((lane >> 3) & 1) * 16);
+template <int N>
+__device__ __forceinline__ uint32_t lane_row(uint32_t tab, int lane) {
+  return tab + (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * split_row<N>() + ((lane >> 3) & 1) * N);
 }
 
 // d[ct][plane] += tile times the columns' splits; the six sums of a step are independent, and each takes
@@ -536,7 +538,7 @@ __device__ __forceinline__ void mul_tile(const uint32_t (&u)[8], uint32_t lrow, 
 #pragma unroll
   for (int ct = 0; ct < kMmaTiles; ++ct)
     if (ct < T) {
-      const uint32_t addr = lrow + ct * split_tile<N>() + K * 32;
+      const uint32_t addr = lrow + ct * split_tile<N>() + K * 16;
       asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
                    : "=r"(c[ct][0]), "=r"(c[ct][1])
                    : "r"(addr + 16 * split_row<N>()));
@@ -611,7 +613,7 @@ template <int N, bool BWD>
 __device__ __forceinline__ void mul_block(uint32_t (&u)[3][8], const cbf16* blk, uint32_t tab, int T, float2* out, int R,
                                           int lane) {
   constexpr int NT = N / 16;
-  const uint32_t lrow = lane_row(tab, split_row<N>(), lane);
+  const uint32_t lrow = lane_row<N>(tab, lane);
   float d[kMmaTiles][2][4];
 #pragma unroll
   for (int i = 0; i < NT * NT; ++i) {
@@ -695,7 +697,7 @@ __global__ void __launch_bounds__(32 * kMW, N == 48 ? 4 : 6) kb_eo_mma(const __g
   ends.load(P, b, off, R);
   __syncthreads();
   if (warp < NT) {
-    const uint32_t lrow = lane_row((uint32_t)__cvta_generic_to_shared(mc_sm), split_row<N>(), lane);
+    const uint32_t lrow = lane_row<N>((uint32_t)__cvta_generic_to_shared(mc_sm), lane);
     float d[kMmaTiles][2][4];
     zero_sums(d);
 #pragma unroll
