@@ -1033,7 +1033,7 @@ int launch_eo_variant(int variant, int n, const EoArgs& a, cudaStream_t s) {
     }
     variant = 4;  // FP64 blocks, no hop input (the right-hand side pass) or unaligned vectors
   }
-  if (variant >= 4 && (al & 15)) variant -= 2;
+  if ((variant == 4 || variant == 5) && (al & 15)) variant -= 2;
   if (variant == 7) {
     if constexpr (sizeof(decltype(AC{}.x)) == 4) {
       switch (n) {
