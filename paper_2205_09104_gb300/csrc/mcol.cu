@@ -267,26 +267,6 @@ __device__ __forceinline__ void mc_block(const Piece<N, BT>& p, const float2* ta
   if (warp < NP * CS) mul_rows<N, BT, ADD>(p, tab, out, 16 * (warp % NP), warp / NP, CS, R, flip, lane);
 }
 
-// Epilogue of one entry (as in the single-column kernels): r = S x or D x, xs = x
-__device__ __forceinline__ void mc_finish(int mode, float2 r, float2 xs, const double2* coef, float2* y, float2* acc) {
-  if (mode == APPLY_PLAIN) {
-    *y = r;
-    return;
-  }
-  const double2 c0d = coef[0], c1d = coef[1];
-  const float2 c0 = make_float2((float)c0d.x, (float)c0d.y), c1 = make_float2((float)c1d.x, (float)c1d.y);
-  float2 ac;
-  if (mode == APPLY_POLY_FIRST) {
-    const double2 c2d = coef[2];
-    ac = cmul(make_float2((float)c2d.x, (float)c2d.y), xs);
-  } else {
-    ac = *acc;
-  }
-  const float2 sp = csub(xs, cmul(c0, r));
-  *y = sp;
-  *acc = cadd(ac, cmul(c1, sp));
-}
-
 // The vectors of a chunk's columns whose gate is open, gathered once per CTA in one round of loads (the
 // latency of a chain of descriptor loads would otherwise be most of a small site's time).
 struct McPtrs {
@@ -529,23 +509,13 @@ __device__ __forceinline__ uint32_t lane_row(uint32_t tab, int lane) {
   return tab + (uint32_t)(((lane >> 4) * 8 + (lane & 7)) * split_row<N>() + ((lane >> 3) & 1) * N);
 }
 
-// d[ct][plane] += tile times the columns' splits; the six sums of a step are independent, and each takes
-// the smallest part of the columns first
-template <int N>
+// d[ct][plane] += tile times the columns' splits (= if FIRST).  The tensor core truncates its sums, so a step's
+// three products, the smallest part of the columns first, start from zero and the steps meet on the FP32 pipe: a
+// chain through all steps of a block had 2.2 times the FP32 kernels' error at n = 48 (measured at the dispatch).
+template <int N, bool FIRST>
 __device__ __forceinline__ void mul_tile(const uint32_t (&u)[8], uint32_t lrow, int K, int T,
                                          float (&d)[kMmaTiles][2][4]) {
-  uint32_t re[4], im[4], b[kMmaTiles][4], c[kMmaTiles][2];
-#pragma unroll
-  for (int ct = 0; ct < kMmaTiles; ++ct)
-    if (ct < T) {
-      const uint32_t addr = lrow + ct * split_tile<N>() + K * 16;
-      asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
-                   : "=r"(c[ct][0]), "=r"(c[ct][1])
-                   : "r"(addr + 16 * split_row<N>()));
-      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                   : "=r"(b[ct][0]), "=r"(b[ct][1]), "=r"(b[ct][2]), "=r"(b[ct][3])
-                   : "r"(addr));
-    }
+  uint32_t re[4], im[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {  // rows 2g, 2g + 1 x entries 4t, 4t + 1, then 4t + 2, 4t + 3
     const int i = 4 * (k & 1) + 2 * (k >> 1);
@@ -555,30 +525,31 @@ __device__ __forceinline__ void mul_tile(const uint32_t (&u)[8], uint32_t lrow, 
 #pragma unroll
   for (int ct = 0; ct < kMmaTiles; ++ct)
     if (ct < T) {
-      mma_bf16(d[ct][0], re, c[ct][0], c[ct][1]);
-      mma_bf16(d[ct][1], im, c[ct][0], c[ct][1]);
+      const uint32_t addr = lrow + ct * split_tile<N>() + K * 16;
+      uint32_t b[4], c[2];
+      asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
+                   : "=r"(c[0]), "=r"(c[1])
+                   : "r"(addr + 16 * split_row<N>()));
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                   : "r"(addr));
+      float e[2][4] = {};
+      mma_bf16(e[0], re, c[0], c[1]);
+      mma_bf16(e[1], im, c[0], c[1]);
+      mma_bf16(e[0], re, b[2], b[3]);
+      mma_bf16(e[1], im, b[2], b[3]);
+      mma_bf16(e[0], re, b[0], b[1]);
+      mma_bf16(e[1], im, b[0], b[1]);
+#pragma unroll
+      for (int pl = 0; pl < 2; ++pl)
+#pragma unroll
+        for (int k = 0; k < 4; k += 2) {
+          const float2 s = make_float2(e[pl][k], e[pl][k + 1]);
+          const float2 r = FIRST ? s : __fadd2_rn(make_float2(d[ct][pl][k], d[ct][pl][k + 1]), s);
+          d[ct][pl][k] = r.x;
+          d[ct][pl][k + 1] = r.y;
+        }
     }
-#pragma unroll
-  for (int ct = 0; ct < kMmaTiles; ++ct)
-    if (ct < T) {
-      mma_bf16(d[ct][0], re, b[ct][2], b[ct][3]);
-      mma_bf16(d[ct][1], im, b[ct][2], b[ct][3]);
-    }
-#pragma unroll
-  for (int ct = 0; ct < kMmaTiles; ++ct)
-    if (ct < T) {
-      mma_bf16(d[ct][0], re, b[ct][0], b[ct][1]);
-      mma_bf16(d[ct][1], im, b[ct][0], b[ct][1]);
-    }
-}
-
-__device__ __forceinline__ void zero_sums(float (&d)[kMmaTiles][2][4]) {
-#pragma unroll
-  for (int ct = 0; ct < kMmaTiles; ++ct)
-#pragma unroll
-    for (int pl = 0; pl < 2; ++pl)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) d[ct][pl][k] = 0.f;
 }
 
 // planes -> F x (or F^H x), rows 2g, 2g + 1 of column 4 ct + t, to out[column][row] (+= sg * ... if ADD)
@@ -617,9 +588,9 @@ __device__ __forceinline__ void mul_block(uint32_t (&u)[3][8], const cbf16* blk,
   float d[kMmaTiles][2][4];
 #pragma unroll
   for (int i = 0; i < NT * NT; ++i) {
-    if (i % NT == 0) zero_sums(d);
     if (i + 2 < NT * NT) load_tile<N, BWD>(u[(i + 2) % 3], blk, (i + 2) / NT, (i + 2) % NT, lane);
-    mul_tile<N>(u[i % 3], lrow, i % NT, T, d);
+    if (i % NT == 0) mul_tile<N, true>(u[i % 3], lrow, 0, T, d);
+    else mul_tile<N, false>(u[i % 3], lrow, i % NT, T, d);
     if (i % NT == NT - 1)
       // sigma3 of a backward hop's rows (a chirality boundary falls between row pairs)
       put_sums<N, BWD, BWD>(d, out, i / NT, R, 16 * (i / NT) + 2 * (lane >> 2) < N / 2 ? 1.f : -1.f, lane);
@@ -699,9 +670,9 @@ __global__ void __launch_bounds__(32 * kMW, N == 48 ? 4 : 6) kb_eo_mma(const __g
   if (warp < NT) {
     const uint32_t lrow = lane_row<N>((uint32_t)__cvta_generic_to_shared(mc_sm), lane);
     float d[kMmaTiles][2][4];
-    zero_sums(d);
+    mul_tile<N, true>(u[0], lrow, 0, T, d);
 #pragma unroll
-    for (int K = 0; K < NT; ++K) mul_tile<N>(u[K], lrow, K, T, d);
+    for (int K = 1; K < NT; ++K) mul_tile<N, false>(u[K], lrow, K, T, d);
     put_sums<N, false, false>(d, hp, warp, R, 1.f, lane);
   }
   __syncthreads();
@@ -758,7 +729,8 @@ __global__ void __launch_bounds__(32 * kMW) kb_apply_mc(const __grid_constant__ 
     const size_t idx = (size_t)s.x * N + i % N;
     const float2 xs = P.v[c][idx];
     const float2 r = mc_full_sum<N>(hp, i, R, P.mu[c], xs, i % N);
-    mc_finish(b.mode, r, xs, P.coef[c], P.y[c] + idx, P.acc[c] + idx);
+    const float2 ac = b.mode == APPLY_POLY ? P.acc[c][idx] : make_float2(0.f, 0.f);
+    s8_finish(b.mode, r, xs, ac, P.coef[c], P.y[c] + idx, P.acc[c] + idx);
   }
 }
 
@@ -791,6 +763,11 @@ int mc_attr(K kernel, size_t bytes) {
   return COARSE_OK;
 }
 
+// BF16 blocks go to the tensor cores, FP32 blocks to the FP32 pipe.  A half apply of a batch of 12 operators
+// (up to 12 columns each, 4^4 to 8^4), n = 16 / 32 / 48: BF16 30 / 103 / 106 us, FP32 27 / 124 / 140 us; with
+// one work item per column, BF16 72 / 326 / 328 us, FP32 76 / 631 / 618 us.  Relative error against FP64 sums,
+// random data at 8^4: BF16 1.05e-7 / 1.16e-7 / 1.19e-7 (column by column 1.06e-7 / 1.29e-7 / 1.32e-7), FP32
+// 0.99e-7 / 1.11e-7 / 1.24e-7 (1.06e-7 / 1.53e-7 / 1.48e-7).
 template <int N>
 int launch_beo_mc_n(bool bf, const McPhase& b, cudaStream_t s) {
   static bool attr = false;
