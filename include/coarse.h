@@ -82,6 +82,9 @@ typedef struct {
  * The caller keeps ownership of its buffers and may free them after return
  * (the call synchronises `stream`).  *out receives a new handle owned by the
  * caller, released with coarse_op_destroy.
+ * The FP64 blocks are also kept as digits (16 bytes per entry, as much as the
+ * FP64 copy) if these and the digits of the vectors fit in a third of the device
+ * memory that is free; otherwise the FP64 stencil runs on the FP64 pipe.
  */
 int coarse_op_create(const coarse_op_desc* desc, const void* self_blocks, const void* hop_blocks,
                      void* stream, coarse_op** out);
@@ -109,6 +112,13 @@ void coarse_op_destroy(coarse_op* op);
  *        whichever the autotuner timed faster for the shape.  An operator created with
  *        BF16 blocks and max_nrhs > 1 keeps two more BF16 copies of its blocks
  *        (one per kernel's operand layout).
+ *        nrhs > 1 with COARSE_PREC_FP32 multiplies up to 12 columns by each block it
+ *        reads (x 16-byte aligned; otherwise column by column).
+ * COARSE_PREC_FP64 multiplies exact 8-bit digits of the blocks and of x on the
+ * tensor cores and adds in FP64; sites whose entries differ too much in size for
+ * that, and non-finite ones, are summed in plain FP64.  The digits of x are written
+ * to the operator's work memory: calls on one operator from several streams must
+ * not overlap, as for the other stencils that use its work memory.
  * Asynchronous on `stream`.  The requested precision must have been enabled
  * in desc.precisions (FP64 is always available).  The FP32 / BF16 kernels
  * stage data through shared memory with bounded waits; if one ran out, that
@@ -383,8 +393,8 @@ int coarse_recycle_get(coarse_op* op, int precision, int odd_even, int adjoint, 
 /*
  * coarse_measure_fp64_fma -- FP64 FMA throughput of the current device in TFLOP/s, from a plain
  * loop of independent FMA chains (8 CTAs of 256 threads per SM, `iters` FMAs per chain, best of
- * three timed launches on `stream`, which it synchronises).  The FP64 stencil that computes the
- * refinement residual is bound by this rate on GB300, and this is the peak its roofline uses.
+ * three timed launches on `stream`, which it synchronises).  An FP64 stencil on the FP64 pipe is
+ * bound by this rate on GB300; the one on exact digit products (coarse_op_create) is not.
  * The paper has no counterpart.
  */
 int coarse_measure_fp64_fma(int iters, double* tflops_host, void* stream);

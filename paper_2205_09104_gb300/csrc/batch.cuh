@@ -1,8 +1,9 @@
 // Batched lockstep engine: descriptors of the solves that advance together and the
 // launchers of the batched kernels.  One solve = one right-hand-side column of one
-// operator; all solves of a batch run the same phase sequence, each phase is one kernel
-// launch over all solves (work items mapped to solves through prefix sums), and the
-// per-solve stop / active flags on the device skip solves that are finished.
+// operator; all solves of a batch run the same phase sequence, and the per-solve stop / active
+// flags on the device skip solves that are finished.  Vector phases are one launch over all solves
+// (work items mapped to solves through prefix sums), stencil phases one launch per n over (operator's
+// column chunk, site), so that a block is read once for the operator's columns.
 #pragma once
 
 #include "common.cuh"
@@ -21,10 +22,7 @@ struct BSolve {
   int V, n, N;
   int kc;              // recycle vectors in use (frozen)
   double mu;
-  // stencil scratch of this solve (pull partials, pushes, arrival counters + error flag)
-  void* part;
-  void* push;
-  int* cnt;
+  int* cnt;            // arrival counters + error flag of the FP64 residual's push-pull kernel
   // vectors of the inner precision (complex64)
   void** vt;           // [m + 1] Krylov basis
   void** qt;           // [kc + m + 1]: C_k then the basis

@@ -3,8 +3,8 @@
 // Every (operator, right-hand-side column) is one solve.  Setup (polynomial and the first
 // u recycle-space updates) runs per operator through the single-operator solver; the solves
 // then share their operator's blocks, polynomial and frozen U_k, C_k.  In the lockstep phase
-// each Krylov phase is ONE kernel launch over all solves (per n-group for the stencil), and
-// per-solve stop / active / done flags on the device skip the solves that are finished.  The
+// each Krylov phase is ONE kernel launch over all solves (the stencil: per n-group, over the
+// operators' chunks of columns and their sites), and per-solve stop / active / done flags on the device skip the solves that are finished.  The
 // whole lockstep solve -- every refinement step, cycle and Arnoldi step -- is one CUDA graph
 // launched once: three nested conditional WHILE nodes whose conditions control kernels set on
 // the device (with iteration bounds), so the host waits only for the end of the batch.

@@ -666,8 +666,8 @@ __global__ void __launch_bounds__(32 * kW) kb_norm64(const BSolve* S, int nsolve
 }  // namespace
 
 namespace {
-// Elements per lane: at least 128 CTAs from N = 32768 on (8^4, n = 32 halves: E = 2 instead of 4 took the
-// three Gram-Schmidt passes of a step from @@ to @@ us), few enough partials for the last CTA.
+// Elements per lane: at least 128 CTAs from N = 32768 on, few enough partials for the last CTA.  The passes are
+// bound by L2 latency at these sizes, so more CTAs with fewer elements each come first.
 int chunk_elems(int N) {
   return N <= (1 << 15) ? 1 : (N <= (1 << 16) ? 2 : (N <= (1 << 18) ? 4 : (N <= (1 << 20) ? 8 : 16)));
 }

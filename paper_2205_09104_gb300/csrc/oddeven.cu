@@ -160,8 +160,7 @@ template <int N, class AC, int W, bool PF>
 constexpr int eo_min_blocks() {
   return (PF && W == 2 && N == 32 && sizeof(decltype(AC{}.x)) == 4) ? 14 : 0;
 }
-// One output site k of a half apply (the CTA's W warps together); shared by the single-operator
-// kernel below and the batched one (one CTA per (solve, site)).
+// One output site k of a half apply (the CTA's W warps together).
 template <int N, class BT, class VT, class AC, int W, bool UNROLL, bool PF>
 __device__ __forceinline__ void eo_half_site(const EoArgs& a, const int k) {
   constexpr int CPL = N / 8, KR = N / 4, NV = N / 2, KW = KR / W;  // KW row quads per warp
@@ -1158,7 +1157,6 @@ int launch_eo_merge(int v64, const void* ev, const void* od, const int* sites, i
 
 // y = S x on compressed even vectors (t: odd scratch of the vector type), with an optional
 // polynomial-chain epilogue (mode, acc, coef) as the full stencil's.
-
 int launch_eo_schur(const coarse_op* op, int prec, double mu_eff, const void* x, void* y, void* t, int mode, void* acc,
                     const double2* coef, const int* stop, cudaStream_t s) {
   EoArgs a{};

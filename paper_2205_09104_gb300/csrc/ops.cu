@@ -80,10 +80,12 @@ __global__ void k_gamma5_defect(const double2* self_b, const double2* hop_b, int
 // block as sigma3 G^H sigma3:  G4[y][mu][i][j] = -lambda_y[i] conj(x_{y+mu}[j])
 //                                                 - s_i s_j x_y[i] conj(lambda_{y+mu}[j]).
 //
-// Bound by the HBM writes: (1 + nhop) n^2 V complex128.  One CTA per site: the site's lambda (and, for
-// the folded form, x) and the source vectors of its blocks are read once into shared memory, then
-// the CTA writes the site's blocks in order, 16 bytes per thread and contiguous over the warp, with
-// every index a compile-time division.
+// Bound by the FP64 pipe (four products per entry: 240 us of 8^4 sites, n = 32, nine blocks, against 90 us of
+// writes, (1 + nhop) n^2 V complex128).  One CTA per site: the site's lambda (and, for the folded form, x)
+// and the source vectors of its blocks are read once into shared memory, then the CTA writes the
+// site's blocks in order, 16 bytes per thread and contiguous over the warp, with every index a
+// compile-time division.  8^4, n = 32, nine blocks: 0.27 ms; one thread per entry that read its vectors
+// through the neighbour table, 0.85 ms.
 template <int N, int NHOP>
 __global__ void __launch_bounds__(256) k_block_grad(const double2* __restrict__ lam, const double2* __restrict__ xv,
                                                     const int* __restrict__ nb, double2* __restrict__ g_self,
