@@ -1,7 +1,6 @@
-// FP64 FMA throughput of the device, measured with a plain dependent-FMA loop.  The FP64
-// stencil (the refinement residual r = b - D_c x) is bound by this rate rather than by HBM on
-// GB300, whose FP64 rate is far below its bandwidth-to-flop balance; the measured peak is the
-// denominator of that kernel's roofline.
+// FP64 FMA throughput of the device, measured with a plain dependent-FMA loop.  A stencil on the FP64
+// pipe is bound by this rate rather than by HBM on GB300, whose FP64 rate is far below its
+// bandwidth-to-flop balance: the reason for the digit products of digits.cu.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
