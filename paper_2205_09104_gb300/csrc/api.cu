@@ -171,11 +171,11 @@ int apply_impl(const coarse_op* op, const void* x, void* y, int nrhs, int precis
   if (nrhs > 1 && precision == COARSE_PREC_BF16) return launch_apply_mrhs_bf16(op, x, y, nrhs, adjoint, s);
   const size_t esz = precision == COARSE_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t col = esz * (size_t)op->V * op->n;
-  // several columns share each block: FP64 digit products two at a time, FP32 up to kMcCols in passes of
+  // several columns share each block: FP64 digit products (dig_columns), FP32 up to kMcCols in passes of
   // nearly equal size (16-byte reads of the columns)
   const bool mc = precision == COARSE_PREC_FP32 && nrhs > 1 && ((uintptr_t)x & 15) == 0;
   const int passes = (nrhs + kMcCols - 1) / kMcCols;
-  const int pass = precision == COARSE_PREC_FP64 && op->dig ? kDigCols : (mc ? (nrhs + passes - 1) / passes : 1);
+  const int pass = precision == COARSE_PREC_FP64 && op->dig ? dig_columns(op->n, op->V) : (mc ? (nrhs + passes - 1) / passes : 1);
   for (int c = 0; c < nrhs; c += pass) {
     ApplyArgs a = make_apply_args(op, precision, (const char*)x + c * col, (char*)y + c * col);
     a.mu = adjoint ? -op->mu : op->mu;

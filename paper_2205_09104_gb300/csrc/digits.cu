@@ -816,8 +816,8 @@ int dig_attr(K kernel, size_t bytes) {
   return COARSE_OK;
 }
 
-// Two columns: one CTA per site (they share the block operand's loads and byte permutations; 8^4, n = 48:
-// 404 us for two against 2 x 240 us).
+// Two columns: one CTA per site (they share the block operand's loads and byte permutations; dig_columns says
+// when).
 template <int N>
 int launch_dig_2(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, cudaStream_t s) {
   constexpr size_t smem = (size_t)kDW * 2 * dig_slab<N>();
@@ -915,6 +915,12 @@ int launch_bresidual_digits(int n, const DigPass* passes, const int* map, int si
   set_error("batched residual: unsupported n = %d", n);
   return COARSE_ERR_INVALID_ARG;
 }
+
+// The pair kernel reads a hop block twice, the second time from L2 while the lattice is small; the push kernel
+// reads it once per column.  Two columns, us, pair / column by column: 6^4 n = 32 82 / 101, n = 48 152 / 165;
+// 8^4 n = 16 92 / 114, n = 32 (336 MB of digits) 205 / 198, n = 48 452 / 354; 12^4 n = 16 406 / 415, n = 32 954 /
+// 759, n = 48 2191 / 1565.
+int dig_columns(int n, int V) { return n > 16 && dig_block_bytes(n, V) > (size_t(320) << 20) ? 1 : kDigCols; }
 
 int launch_apply_digits(int n, const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {
   if (ncol < 1 || ncol > kDigCols) {

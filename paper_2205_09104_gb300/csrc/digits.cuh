@@ -22,6 +22,8 @@ inline size_t dig_block_bytes(int n, int V) { return (size_t)V * 5 * n * n * 16;
 inline size_t dig_scale_bytes(int V) { return (size_t)V * 5 * sizeof(double); }
 int launch_dig_blocks(const double2* blocks, int V, int n, void* dig, double* scale, cudaStream_t s);
 
+// Columns that one pass of a multi-column FP64 stencil should take (1 or kDigCols).
+int dig_columns(int n, int V);
 // y = D x (with a's epilogue) for ncol <= kDigCols columns x + c * ldc, y + c * ldc, through the digit
 // operands a.dig (must be set); a.digx holds room for ncol columns.
 int launch_apply_digits(int n, const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s);
