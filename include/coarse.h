@@ -115,8 +115,10 @@ void coarse_op_destroy(coarse_op* op);
  *        nrhs > 1 with COARSE_PREC_FP32 multiplies up to 12 columns by each block it
  *        reads (x 16-byte aligned; otherwise column by column).
  * COARSE_PREC_FP64 multiplies exact 8-bit digits of the blocks and of x on the
- * tensor cores and adds in FP64; sites whose entries differ too much in size for
- * that, and non-finite ones, are summed in plain FP64.  The digits of x are written
+ * tensor cores and adds in FP64.  Every entry is within 6.4 n + 20 units of 2^-53
+ * of sum_j |D_ij| |x_j|: rows whose products are too small for that against the
+ * largest entries of their blocks and sites, and non-finite ones, are summed in
+ * plain FP64.  The digits of x are written
  * to the operator's work memory: calls on one operator from several streams must
  * not overlap, as for the other stencils that use its work memory.
  * Asynchronous on `stream`.  The requested precision must have been enabled

@@ -368,7 +368,7 @@ int coarse_op_create(const coarse_op_desc* d, const void* self_blocks, const voi
   {
     // digit copy of the FP64 blocks, where it leaves most of the free memory to the solvers
     const size_t db = dig_block_bytes(op->n, op->V);
-    const size_t xb = dig_x_bytes(op->n, op->V, op->max_nrhs < kDigCols ? op->max_nrhs : kDigCols);
+    const size_t xb = dig_work_bytes(op->n, op->V, op->max_nrhs < kDigCols ? op->max_nrhs : kDigCols);
     size_t mfree = 0, mtotal = 0;
     cudaMemGetInfo(&mfree, &mtotal);
     if (db + xb <= mfree / 3 &&

@@ -138,7 +138,7 @@ struct ApplyArgs {
   int* err;             // raised (1) if a bounded wait of the TMA-staged kernel expired
   const void* dig;      // FP64: the blocks as digits (digits.cuh), or null: the FP64 pipe
   const double* digscale;  // their scales
-  void* digx;           // room for the column operands (dig_x_bytes)
+  void* digx;           // room for the column operands and row magnitudes (dig_work_bytes)
 };
 
 int launch_apply(int prec, int n, const ApplyArgs& a, cudaStream_t s);

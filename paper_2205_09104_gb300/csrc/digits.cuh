@@ -7,14 +7,22 @@ namespace coarse {
 
 constexpr int kDigCols = 2;  // columns of one pass
 
-// Halves of the packed digits of one (column, site): [part][digit][n]; bytes of one record of row
+// Halves of the packed digits of one (column, site): [part][digit][n], then the magnitudes of the leading digits
+// |re| + |im|, [n]; bytes of one record of row
 // corrections: [sigma3 variant][part][level] floats.
-__host__ __device__ constexpr size_t dig_x_halves(int n) { return 16 * (size_t)n; }
+__host__ __device__ constexpr size_t dig_x_halves(int n) { return 17 * (size_t)n; }
 constexpr size_t kDigCorr = 32;
 
-// Bytes of the column operands of `cols` columns on V sites: digits, corrections, scales.
+// Bytes of the column operands of `cols` columns on V sites: digits, corrections, scales, the rows' demands.
 __host__ __device__ inline size_t dig_x_bytes(int n, int V, int cols) {
-  return (size_t)cols * V * (dig_x_halves(n) * 2 + kDigCorr * sizeof(float) + sizeof(double));
+  return (size_t)cols * V * (dig_x_halves(n) * 2 + kDigCorr * sizeof(float) + sizeof(double) + sizeof(float));
+}
+// Bytes of the work memory of a stencil of up to `cols` columns per pass (ApplyArgs::digx): the column operands, behind
+// those of one column the push kernel's row magnitudes and exponents.
+inline size_t dig_work_bytes(int n, int V, int cols) {
+  const size_t push = dig_x_bytes(n, V, 1) + (size_t)5 * V * (n * sizeof(float) + sizeof(int));
+  const size_t pass = dig_x_bytes(n, V, cols);
+  return push > pass ? push : pass;
 }
 
 // Blocks of one operator as digits and their scales (sizes: dig_block_bytes, dig_scale_bytes).
