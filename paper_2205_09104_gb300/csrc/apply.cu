@@ -363,11 +363,8 @@ int launch_8(int n, const ApplyArgs& a, cudaStream_t s) {
 template <int N, class BT>
 int launch_tma_n(const ApplyArgs& a, cudaStream_t s) {
   using Cfg = TmaCfg<N, BT>;
-  static bool attr = false;
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(k_apply_tma<N, BT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_apply_tma<N, BT>, Cfg::kSmem));
   int ctas = sm_count();
   const int need = (a.V + Cfg::kWarps - 1) / Cfg::kWarps;
   if (need < ctas) ctas = need;

@@ -121,11 +121,8 @@ constexpr int kBMaxSmem = 200 * 1024;
 template <int N, int P>
 int launch_bm(int S, const BMApply& a, cudaStream_t s) {
   constexpr int THREADS = (P * (N / 16) + 1) * 32;
-  static bool attr = false;
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(kb_apply_mrhs<N, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBMaxSmem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)kb_apply_mrhs<N, P>, kBMaxSmem));
   const uint32_t SB = mrhs_stage_bytes(N, P, kMrhsMaxT);
   S = S < 2 ? 2 : (S > 8 ? 8 : S);
   while (S > 2 && (size_t)S * SB + 16 * S > (size_t)kBMaxSmem) --S;

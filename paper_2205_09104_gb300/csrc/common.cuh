@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/coarse.h"
+#include "smem_limit.cuh"
 
 namespace coarse {
 

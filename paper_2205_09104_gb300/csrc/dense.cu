@@ -443,12 +443,9 @@ int launch_step_finalize(CycleState* st, const double2* h1, const double2* h2, c
 }
 
 int launch_cycle_solve(const CycleState* st, const Dense& d, cudaStream_t s) {
-  static bool attr = false;
   const size_t smem = sizeof(double2) * (size_t)kMaxDense * d.ldh;
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(k_cycle_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_cycle_solve, smem));
   k_cycle_solve<<<1, 32, smem, s>>>(st, d);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
@@ -468,12 +465,9 @@ size_t poly_smem() {
 }
 
 int launch_recycle(CycleState* st, const Dense& d, const double2* SW, int ldsw, int knew, cudaStream_t s) {
-  static bool attr = false;
   const size_t smem = recycle_smem();
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(k_recycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_recycle, smem));
   k_recycle<<<1, 32, smem, s>>>(st, d, SW, ldsw, knew);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
@@ -481,12 +475,9 @@ int launch_recycle(CycleState* st, const Dense& d, const double2* SW, int ldsw, 
 }
 
 int launch_poly_roots(CycleState* st, const Dense& d, int dmax, cudaStream_t s) {
-  static bool attr = false;
   const size_t smem = poly_smem();
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(k_poly_roots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_poly_roots, smem));
   k_poly_roots<<<1, 32, smem, s>>>(st, d, dmax);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
@@ -515,12 +506,9 @@ int launch_bfinalize(const BSolve* S, int nsolves, cudaStream_t s) {
 
 int launch_bcycle_solve(const BSolve* S, int nsolves, cudaStream_t s) {
   if (nsolves <= 0) return COARSE_OK;
-  static bool attr = false;
   const size_t smem = sizeof(double2) * (size_t)kMaxDense * (kMaxDense + 1);
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(kb_cycle_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)kb_cycle_solve, smem));
   kb_cycle_solve<<<nsolves, 32, smem, s>>>(S);
   note_launch();
   COARSE_CUDA(cudaGetLastError());

@@ -949,23 +949,13 @@ __global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, kDigCols)) kb_resi
   dig_site<N, kDigCols>(a, d, site, p.cols, p.ldx, p.ldy, p.ldx);
 }
 
-template <class K>
-int dig_attr(K kernel, size_t bytes) {
-  COARSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return COARSE_OK;
-}
-
 // Two columns: one CTA per site (they share the block operand's loads and byte permutations; dig_columns says
 // when).
 template <int N>
 int launch_dig_2(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, cudaStream_t s) {
   constexpr size_t smem = (size_t)kDW * 2 * dig_slab<N>();
-  static bool attr = false;
-  if (!attr) {
-    const int rc = dig_attr(k_site_digits<N, 2>, smem);
-    if (rc != COARSE_OK) return rc;
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_site_digits<N, 2>, smem));
   k_site_digits<N, 2><<<a.V, 32 * kDW, smem, s>>>(a, d, ncol, ldc);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
@@ -979,21 +969,17 @@ int launch_dig_2(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, 
 constexpr int kPushSites = 1024;
 template <int N>
 int launch_dig_1(const ApplyArgs& a, const DigArgs& d, cudaStream_t s) {
-  static bool attr = false;
+  static SmemLimit push, site;
   constexpr size_t ss = (size_t)kDW * dig_slab<N>(), su = (size_t)(kPW + 1) * dig_slab<N>() + (size_t)kPW * 2 * 4096;
-  if (!attr) {
-    int rc = dig_attr(k_push_digits<N>, su);
-    if (rc == COARSE_OK) rc = dig_attr(k_site_digits<N, 1>, ss);
-    if (rc != COARSE_OK) return rc;
-    attr = true;
-  }
   if (a.V >= kPushSites) {
+    COARSE_CUDA(raise_smem_limit(push, (const void*)k_push_digits<N>, su));
     k_push_digits<N><<<a.V, 32 * kPW, su, s>>>(a, d);
     note_launch();
     COARSE_CUDA(cudaGetLastError());
     const size_t total = (size_t)a.V * N;
     k_push_finish<N><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(a);
   } else {
+    COARSE_CUDA(raise_smem_limit(site, (const void*)k_site_digits<N, 1>, ss));
     k_site_digits<N, 1><<<a.V, 32 * kDW, ss, s>>>(a, d, 1, 0);
   }
   note_launch();
@@ -1022,11 +1008,8 @@ template <int N>
 int launch_bresidual_n(const DigPass* passes, const int* map, int sites, const int* flags, const double2* coef,
                        cudaStream_t s) {
   constexpr size_t smem = (size_t)kDW * kDigCols * dig_slab<N>();
-  static bool attr = false;
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(kb_residual_digits<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)kb_residual_digits<N>, smem));
   kb_dig_x<N><<<sites / 4, 128, 0, s>>>(passes, map, flags);
   note_launch();
   COARSE_CUDA(cudaGetLastError());

@@ -757,12 +757,6 @@ __global__ void __launch_bounds__(32 * kMW) k_apply_mc(const __grid_constant__ A
   }
 }
 
-template <class K>
-int mc_attr(K kernel, size_t bytes) {
-  COARSE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return COARSE_OK;
-}
-
 // BF16 blocks go to the tensor cores, FP32 blocks to the FP32 pipe.  A half apply of a batch of 12 operators
 // (up to 12 columns each, 4^4 to 8^4), n = 16 / 32 / 48: BF16 30 / 103 / 106 us, FP32 27 / 124 / 140 us; with
 // one work item per column, BF16 72 / 326 / 328 us, FP32 76 / 631 / 618 us.  Relative error against FP64 sums,
@@ -770,15 +764,14 @@ int mc_attr(K kernel, size_t bytes) {
 // 0.99e-7 / 1.11e-7 / 1.24e-7 (1.06e-7 / 1.53e-7 / 1.48e-7).
 template <int N>
 int launch_beo_mc_n(bool bf, const McPhase& b, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    int rc = mc_attr(kb_eo_mc<N, float2>, mc_smem<N>(kMcCols));
-    if (rc == COARSE_OK) rc = mc_attr(kb_eo_mma<N>, mma_smem<N>(kMcCols));
-    if (rc != COARSE_OK) return rc;
-    attr = true;
+  static SmemLimit mma, mc;
+  if (bf) {
+    COARSE_CUDA(raise_smem_limit(mma, (const void*)kb_eo_mma<N>, mma_smem<N>(kMcCols)));
+    kb_eo_mma<N><<<b.count, 32 * kMW, mma_smem<N>(b.rmax), s>>>(b);
+  } else {
+    COARSE_CUDA(raise_smem_limit(mc, (const void*)kb_eo_mc<N, float2>, mc_smem<N>(kMcCols)));
+    kb_eo_mc<N, float2><<<b.count, 32 * kMW, mc_smem<N>(b.rmax), s>>>(b);
   }
-  if (bf) kb_eo_mma<N><<<b.count, 32 * kMW, mma_smem<N>(b.rmax), s>>>(b);
-  else kb_eo_mc<N, float2><<<b.count, 32 * kMW, mc_smem<N>(b.rmax), s>>>(b);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
   return COARSE_OK;
@@ -786,12 +779,8 @@ int launch_beo_mc_n(bool bf, const McPhase& b, cudaStream_t s) {
 
 template <int N, class BT>
 int launch_bapply_mc_n(const McPhase& b, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    const int rc = mc_attr(kb_apply_mc<N, BT>, mc_smem<N>(kMcCols));
-    if (rc != COARSE_OK) return rc;
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)kb_apply_mc<N, BT>, mc_smem<N>(kMcCols)));
   kb_apply_mc<N, BT><<<b.count, 32 * kMW, mc_smem<N>(b.rmax), s>>>(b);
   note_launch();
   COARSE_CUDA(cudaGetLastError());
@@ -800,12 +789,8 @@ int launch_bapply_mc_n(const McPhase& b, cudaStream_t s) {
 
 template <int N>
 int launch_apply_mc_n(const ApplyArgs& a, int R, long long ldc, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    const int rc = mc_attr(k_apply_mc<N, float2>, mc_smem<N>(kMcCols));
-    if (rc != COARSE_OK) return rc;
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_apply_mc<N, float2>, mc_smem<N>(kMcCols)));
   k_apply_mc<N, float2><<<a.V, 32 * kMW, mc_smem<N>(R), s>>>(a, R, ldc);
   note_launch();
   COARSE_CUDA(cudaGetLastError());

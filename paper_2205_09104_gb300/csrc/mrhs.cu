@@ -149,11 +149,8 @@ constexpr int kMrhsMaxSmem = 200 * 1024;
 template <int N, int T, int P>
 int launch_mrhs_cfg(MrhsArgs a, int S, cudaStream_t s) {
   using Sh = MrhsShape<N, P>;
-  static bool attr = false;
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(k_apply_mrhs<N, T, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMrhsMaxSmem));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_apply_mrhs<N, T, P>, kMrhsMaxSmem));
   a.SB = mrhs_stage_bytes(N, P, T);
   if (S <= 0) S = (int)((64u * 1024u) / a.SB);
   S = S < 2 ? 2 : (S > 8 ? 8 : S);

@@ -379,11 +379,8 @@ int launch_tc_nt(TcArgs a, int ctas_per_sm, int S, cudaStream_t s) {
     set_error("tcgen05 multi-RHS apply: %zu bytes of shared memory for %d CTAs per SM", smem, ctas_per_sm);
     return COARSE_ERR_INVALID_ARG;
   }
-  static bool attr = false;
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(k_apply_mrhs_tc<N, T, MASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_apply_mrhs_tc<N, T, MASS>, 210 * 1024));
   int grid = ctas_per_sm * sm_count();
   if (grid > a.V) grid = a.V;
   k_apply_mrhs_tc<N, T, MASS><<<grid, kTcThreads, smem, s>>>(a);

@@ -949,11 +949,8 @@ int eo_prepare(coarse_op* op, double mu_eff, cudaStream_t s) {
     }
   }
   const size_t smem = sizeof(double2) * (size_t)n * 2 * n;
-  static bool attr = false;
-  if (!attr) {
-    COARSE_CUDA(cudaFuncSetAttribute(k_block_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-    attr = true;
-  }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_block_inverse, 96 * 1024));
   COARSE_CUDA(cudaMemsetAsync(op->apply_cnt + op->V + 1, 0, sizeof(int), s));
   k_block_inverse<<<op->V, 256, smem, s>>>((const double2*)op->blk[0].ptr, n, mu_eff, (double2*)op->inv[sg][0].ptr,
                                            op->apply_cnt + op->V + 1);
@@ -995,15 +992,14 @@ int launch_eo_ring_n(const EoArgs& a, cudaStream_t s) {
       dyn = (size_t)sv * SB + 16 * (size_t)sv;
       if (dyn + fa.sharedSizeBytes + 128 <= (size_t)optin) break;
     }
-    if (sv >= 1)
-      COARSE_CUDA(cudaFuncSetAttribute(k_eo_ring<N, BT, VT, AC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)dyn));
     S = std::max(sv, 0);
   }
   if (S < 1) {
     set_error("odd-even: the streamed layout does not fit in shared memory for n = %d", N);
     return COARSE_ERR_INVALID_ARG;
   }
+  static SmemLimit limit;
+  COARSE_CUDA(raise_smem_limit(limit, (const void*)k_eo_ring<N, BT, VT, AC>, dyn));
   const int grid = std::min(a.V / 2, sm_count());
   k_eo_ring<N, BT, VT, AC><<<grid, kEoRingThreads, dyn, s>>>(a, S);
   return COARSE_OK;
