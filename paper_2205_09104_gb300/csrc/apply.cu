@@ -430,8 +430,9 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
     set_error("coarse_apply: unsupported n = %d (nv must be 8, 16 or 24)", n);
     return COARSE_ERR_INVALID_ARG;
   }
-  // the staged kernel copies site vectors in bulk: 16-byte aligned x only
-  if ((uintptr_t)a.x & 15) return launch_t<BT, float2, float2>(n, a, s);
+  // the staged kernel copies site vectors in bulk: 16-byte aligned x only; for other x the register kernel
+  // takes its place, and nothing is timed
+  const bool staged = ((uintptr_t)a.x & 15) == 0;
   int choice = tune_fast_get(0, prec, ni, vb);
   if (choice < 0) {
     char key[64];
@@ -455,15 +456,18 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
     TuneChoice c;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(s, &cap);
-    const int rc = tune_pick(key, {TuneChoice{0, 0, 0}, TuneChoice{1, 0, 0}, TuneChoice{2, 0, 0}}, run, s, &c);
+    std::vector<TuneChoice> cands{TuneChoice{1, 0, 0}};
+    if (staged) cands = {TuneChoice{0, 0, 0}, TuneChoice{1, 0, 0}, TuneChoice{2, 0, 0}};
+    const int rc = tune_pick(key, cands, run, s, &c);
     if (scratch) {
       cudaStreamSynchronize(s);
       cudaFree(scratch);
     }
     if (rc != COARSE_OK) return rc;
-    if (cap == cudaStreamCaptureStatusNone) tune_fast_put(0, prec, ni, vb, c.a);
+    if (cap == cudaStreamCaptureStatusNone && staged) tune_fast_put(0, prec, ni, vb, c.a);
     choice = c.a;
   }
+  if (choice == 0 && !staged) choice = 1;
   return choice == 2 ? launch_8<BT>(n, a, s) : choice == 1 ? launch_t<BT, float2, float2>(n, a, s) : launch_tma<BT>(n, a, s);
 }
 
