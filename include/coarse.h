@@ -52,12 +52,21 @@ typedef enum {
 } coarse_precision;
 
 #define COARSE_ASSUME_GAMMA5 0x1u /* hop_blocks holds only the 4 forward hops */
+#define COARSE_FP64_PIPE 0x2u     /* never keep a digit copy: FP64 stencils on the FP64 pipe */
+
+/* Which way the FP64 stencils of an operator go (coarse_op_fp64_path). */
+typedef enum {
+  COARSE_FP64_UNDECIDED = 0,   /* none has run yet */
+  COARSE_FP64_DIGITS = 1,      /* exact digit products: the copy is held */
+  COARSE_FP64_PIPE_ASKED = 2,  /* FP64 pipe: COARSE_FP64_PIPE was given */
+  COARSE_FP64_PIPE_MEMORY = 3  /* FP64 pipe: no room for the copy, or it was given back */
+} coarse_fp64_path;
 
 typedef struct {
   int32_t dims[4];      /* coarse lattice extents, each >= 2 */
   int32_t nv;           /* test vectors per chirality: n = 2*nv, nv in {8, 16, 24} */
   double mu;            /* twisted mass: D_c gets + i*mu*sigma3 on the diagonal (0 = Wilson-clover) */
-  uint32_t flags;       /* COARSE_ASSUME_GAMMA5 or 0 */
+  uint32_t flags;       /* COARSE_ASSUME_GAMMA5, COARSE_FP64_PIPE or 0 */
   int32_t max_nrhs;     /* largest nrhs later passed to coarse_apply / coarse_solve (>= 1) */
   uint32_t precisions;  /* bit mask of (1u << coarse_precision) block copies to keep; FP64 always kept */
 } coarse_op_desc;
@@ -82,9 +91,14 @@ typedef struct {
  * The caller keeps ownership of its buffers and may free them after return
  * (the call synchronises `stream`).  *out receives a new handle owned by the
  * caller, released with coarse_op_destroy.
- * The FP64 blocks are also kept as digits (16 bytes per entry, as much as the
- * FP64 copy) if these and the digits of the vectors fit in a third of the device
- * memory that is free; otherwise the FP64 stencil runs on the FP64 pipe.
+ * The first FP64 stencil on the operator that is not being captured (an apply, a
+ * residual, a solve's refinement) also makes a copy of the FP64 blocks as digits,
+ * 16 bytes per entry, as much as the FP64 blocks, and synchronises its stream once.
+ * The copies of all operators take at most a quarter of the device's memory; where
+ * there is no room, and with COARSE_FP64_PIPE, FP64 stencils run on the FP64 pipe,
+ * at up to four times the time and with other rounding.  An allocation of this
+ * library that fails takes back copies that no running call and no captured graph
+ * uses, and is tried again.  coarse_op_fp64_path tells which way an operator goes.
  */
 int coarse_op_create(const coarse_op_desc* desc, const void* self_blocks, const void* hop_blocks,
                      void* stream, coarse_op** out);
@@ -98,6 +112,9 @@ int coarse_op_update(coarse_op* op, const void* self_blocks, const void* hop_blo
 
 /* Releases the handle and all device memory it owns (synchronises the device). */
 void coarse_op_destroy(coarse_op* op);
+
+/* coarse_op_fp64_path -- *path receives a coarse_fp64_path; the paper has no counterpart. */
+int coarse_op_fp64_path(const coarse_op* op, int* path);
 
 /*
  * coarse_apply -- y = D_c x (Sec. 2.2, the coarse nearest-neighbour stencil):

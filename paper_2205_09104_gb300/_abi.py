@@ -9,6 +9,9 @@ lib_path = os.path.join(HERE, "_build", "libcoarse.so")
 
 PREC_FP64, PREC_FP32, PREC_BF16 = 0, 1, 2
 COARSE_ASSUME_GAMMA5 = 0x1
+COARSE_FP64_PIPE = 0x2
+# coarse_op_fp64_path: how an operator's FP64 stencils run
+FP64_UNDECIDED, FP64_DIGITS, FP64_PIPE_ASKED, FP64_PIPE_MEMORY = 0, 1, 2, 3
 COARSE_ZERO_GUESS = 0x1
 COARSE_REBUILD_POLY = 0x2
 COARSE_RESET_RECYCLE = 0x4
@@ -26,7 +29,8 @@ EXPORTS = ["coarse_op_create", "coarse_op_update", "coarse_op_destroy", "coarse_
            "coarse_residual", "coarse_solve", "coarse_solve_adjoint", "coarse_solve_batched", "coarse_block_grad",
            "coarse_op_poly", "coarse_last_error", "coarse_version", "coarse_residual_noalloc",
            "coarse_autotune_report", "coarse_schur_apply", "coarse_recycle_check",
-           "coarse_recycle_get", "coarse_autotune_set", "coarse_measure_fp64_fma", "coarse_recycle_set"]
+           "coarse_recycle_get", "coarse_autotune_set", "coarse_measure_fp64_fma", "coarse_recycle_set",
+           "coarse_op_fp64_path"]
 
 
 class CoarseError(RuntimeError):
@@ -97,6 +101,7 @@ def lib() -> ctypes.CDLL:
     L.coarse_recycle_set.argtypes = [vp, i32, i32, i32, vp, vp, i32, i32, vp]
     L.coarse_autotune_report.argtypes = [ctypes.c_char_p, ctypes.c_longlong]
     L.coarse_autotune_set.argtypes = [ctypes.c_char_p, i32, i32, i32]
+    L.coarse_op_fp64_path.argtypes = [vp, P(i32)]
     L.coarse_measure_fp64_fma.argtypes = [i32, P(dbl), vp]
     L.coarse_last_error.restype = ctypes.c_char_p
     L.coarse_version.restype = ctypes.c_char_p

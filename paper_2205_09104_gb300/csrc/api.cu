@@ -3,6 +3,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <string>
 #include <vector>
@@ -50,7 +51,7 @@ bool valid_nv(int nv) { return nv == 8 || nv == 16 || nv == 24; }
 
 template <class T>
 int dmalloc(T** p, size_t bytes) {
-  cudaError_t e = cudaMalloc((void**)p, bytes == 0 ? 1 : bytes);
+  cudaError_t e = device_malloc((void**)p, bytes == 0 ? 1 : bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     set_error("device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
@@ -85,9 +86,7 @@ void free_op(coarse_op* op) {
   if (op->red) cudaFree(op->red);
   if (op->apply_scratch) cudaFree(op->apply_scratch);
   if (op->apply_cnt) cudaFree(op->apply_cnt);
-  if (op->dig) cudaFree(op->dig);
-  if (op->digscale) cudaFree(op->digscale);
-  if (op->digx) cudaFree(op->digx);
+  dig_store_delete(op->digits);
   delete op;
 }
 
@@ -118,7 +117,7 @@ int ingest(coarse_op* op, const void* self_b, const void* hop_b, uint32_t flags,
   TRY(launch_ingest((const double2*)self_b, (const double2*)hop_b, gamma5_only, op->V, op->n, op->nb,
                     op->blk[0].ptr, op->blk[1].ptr, op->blk[2].ptr, s));
   TRY(launch_pack_mrhs(op, s));
-  if (op->dig) TRY(launch_dig_blocks((const double2*)op->blk[0].ptr, op->V, op->n, op->dig, op->digscale, s));
+  TRY(dig_store_refill(op->digits, dig_plan(op), s));
   COARSE_CUDA(cudaStreamSynchronize(s));
   return COARSE_OK;
 }
@@ -154,6 +153,22 @@ int validate_solve(const coarse_op* op, const void* b, const void* x, int nrhs, 
   return COARSE_OK;
 }
 
+// Several columns in FP64: as many as dig_columns says share the digits of each block.
+int apply64_columns(const coarse_op* op, const void* x, void* y, int nrhs, int adjoint, cudaStream_t s) {
+  const DigUse d(op->digits, dig_plan(op), s);
+  TRY(d.rc());
+  const size_t N = (size_t)op->V * op->n;
+  const int pass = d.dig() ? dig_columns(op->n, op->V) : 1;
+  for (int c = 0; c < nrhs; c += pass) {
+    ApplyArgs a = make_apply_args(op, COARSE_PREC_FP64, (const double2*)x + c * N, (double2*)y + c * N);
+    a.mu = adjoint ? -op->mu : op->mu;
+    a.adjoint = adjoint;
+    if (d.dig()) TRY(launch_apply_digits(op->n, a, d, std::min(pass, nrhs - c), (long long)N, s));
+    else TRY(launch_apply(COARSE_PREC_FP64, op->n, a, s));
+  }
+  return COARSE_OK;
+}
+
 int apply_impl(const coarse_op* op, const void* x, void* y, int nrhs, int precision, void* stream, int adjoint) {
   if (!op) { set_error("op is NULL"); return COARSE_ERR_INVALID_ARG; }
   TRY(check_ptr(x, "x"));
@@ -171,18 +186,18 @@ int apply_impl(const coarse_op* op, const void* x, void* y, int nrhs, int precis
   if (nrhs > 1 && precision == COARSE_PREC_BF16) return launch_apply_mrhs_bf16(op, x, y, nrhs, adjoint, s);
   const size_t esz = precision == COARSE_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t col = esz * (size_t)op->V * op->n;
-  // several columns share each block: FP64 digit products (dig_columns), FP32 up to kMcCols in passes of
-  // nearly equal size (16-byte reads of the columns)
+  // several FP32 columns share each block: up to kMcCols in passes of nearly equal size (16-byte reads of the columns)
   const bool mc = precision == COARSE_PREC_FP32 && nrhs > 1 && ((uintptr_t)x & 15) == 0;
   const int passes = (nrhs + kMcCols - 1) / kMcCols;
-  const int pass = precision == COARSE_PREC_FP64 && op->dig ? dig_columns(op->n, op->V) : (mc ? (nrhs + passes - 1) / passes : 1);
+  if (precision == COARSE_PREC_FP64 && nrhs > 1) return apply64_columns(op, x, y, nrhs, adjoint, s);
+  const int pass = mc ? (nrhs + passes - 1) / passes : 1;
   for (int c = 0; c < nrhs; c += pass) {
     ApplyArgs a = make_apply_args(op, precision, (const char*)x + c * col, (char*)y + c * col);
     a.mu = adjoint ? -op->mu : op->mu;
     a.adjoint = adjoint;
     const int nc = nrhs - c < pass ? nrhs - c : pass;
     if (mc) TRY(launch_apply_mc(op->n, a, nc, (long long)op->V * op->n, s));
-    else if (nc > 1) TRY(launch_apply_digits(op->n, a, nc, (long long)op->V * op->n, s));
+    else if (precision == COARSE_PREC_FP64) TRY(launch_apply64(op, a, s));
     else TRY(launch_apply(precision, op->n, a, s));
   }
   return COARSE_OK;
@@ -290,6 +305,7 @@ int coarse_op_create(const coarse_op_desc* d, const void* self_blocks, const voi
   op->mu = d->mu;
   op->max_nrhs = d->max_nrhs;
   op->precisions = d->precisions | 1u;
+  op->digits = dig_store_new(op->device, (d->flags & COARSE_FP64_PIPE) != 0);
   const size_t N = (size_t)op->V * op->n;
   // neighbour table
   std::vector<int> nb((size_t)op->V * 8);
@@ -365,23 +381,6 @@ int coarse_op_create(const coarse_op_desc* d, const void* self_blocks, const voi
   op->norms = op->red + 2 * 304;
   op->coef = (double2*)(op->norms + 8);
   op->counter = (unsigned*)(op->coef + 2);
-  {
-    // digit copy of the FP64 blocks, where it leaves most of the free memory to the solvers
-    const size_t db = dig_block_bytes(op->n, op->V);
-    const size_t xb = dig_work_bytes(op->n, op->V, op->max_nrhs < kDigCols ? op->max_nrhs : kDigCols);
-    size_t mfree = 0, mtotal = 0;
-    cudaMemGetInfo(&mfree, &mtotal);
-    if (db + xb <= mfree / 3 &&
-        (cudaMalloc(&op->dig, db) != cudaSuccess || cudaMalloc((void**)&op->digscale, dig_scale_bytes(op->V)) != cudaSuccess ||
-         cudaMalloc(&op->digx, xb) != cudaSuccess)) {
-      cudaGetLastError();
-      cudaFree(op->dig);
-      cudaFree(op->digscale);
-      op->dig = nullptr;
-      op->digscale = nullptr;
-      op->digx = nullptr;
-    }
-  }
   const double2 cst[2] = {make_double2(-1.0, 0.0), make_double2(1.0, 0.0)};
   if ((op->eo_sites &&
        (cudaMemcpyAsync(op->eo_sites, eo_sites.data(), eo_sites.size() * sizeof(int), cudaMemcpyHostToDevice, s) !=
@@ -408,6 +407,7 @@ int coarse_op_update(coarse_op* op, const void* self_blocks, const void* hop_blo
   if (!op) { set_error("op is NULL"); return COARSE_ERR_INVALID_ARG; }
   TRY(check_ptr(self_blocks, "self_blocks"));
   TRY(check_ptr(hop_blocks, "hop_blocks"));
+  dig_store_retry(op->digits);
   TRY(ingest(op, self_blocks, hop_blocks, 0, (cudaStream_t)stream));
   op->inv_ok[0] = op->inv_ok[1] = 0;
   for (int p = 0; p < 3; ++p) {
@@ -420,6 +420,13 @@ int coarse_op_update(coarse_op* op, const void* self_blocks, const void* hop_blo
 }
 
 void coarse_op_destroy(coarse_op* op) { free_op(op); }
+
+int coarse_op_fp64_path(const coarse_op* op, int* path) {
+  if (!op) { set_error("op is NULL"); return COARSE_ERR_INVALID_ARG; }
+  TRY(check_ptr(path, "path"));
+  *path = dig_store_path(op->digits);
+  return COARSE_OK;
+}
 
 int coarse_apply(const coarse_op* op, const void* x, void* y, int nrhs, int precision, void* stream) {
   return apply_impl(op, x, y, nrhs, precision, stream, 0);
@@ -458,7 +465,7 @@ int coarse_residual(const coarse_op* op, const void* b, const void* x, void* r, 
   a.z = b;
   a.coef = op->coef;
   a.mode = APPLY_AXPBY;
-  TRY(launch_apply(COARSE_PREC_FP64, op->n, a, s));
+  TRY(launch_apply64(op, a, s));
   TRY(launch_norm2(1, r, N, op->norms + 4, op->red, op->counter, s));
   TRY(launch_norm2(1, b, N, op->norms + 5, op->red, op->counter, s));
   double h[2];

@@ -20,7 +20,6 @@
 #include "common.cuh"
 #include "apply_core.cuh"
 #include "batch.cuh"
-#include "digits.cuh"
 #include "pipe.cuh"
 #include "site8.cuh"
 #include "tune.cuh"
@@ -439,7 +438,7 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
     snprintf(key, sizeof(key), "apply/p%d/n%d/v%d", prec, n, vb);
     void* scratch = nullptr;
     auto run = [&](const TuneChoice& c) -> int {
-      if (!scratch && cudaMalloc(&scratch, sizeof(float2) * (size_t)a.V * n) != cudaSuccess) {
+      if (!scratch && device_malloc(&scratch, sizeof(float2) * (size_t)a.V * n) != cudaSuccess) {
         cudaGetLastError();
         set_error("coarse_apply: autotuner scratch allocation failed");
         return COARSE_ERR_OOM;
@@ -474,9 +473,7 @@ int launch_tuned(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
 int launch_apply(int prec, int n, const ApplyArgs& a, cudaStream_t s) {
   if (a.V <= 0) return COARSE_OK;
   switch (prec) {
-    case COARSE_PREC_FP64:
-      if (a.dig) return launch_apply_digits(n, a, 1, 0, s);
-      return launch_t<double2, double2, double2>(n, a, s);
+    case COARSE_PREC_FP64: return launch_t<double2, double2, double2>(n, a, s);
     case COARSE_PREC_FP32: return launch_tuned<float2>(prec, n, a, s);
     case COARSE_PREC_BF16: return launch_tuned<cbf16>(prec, n, a, s);
   }

@@ -13,6 +13,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <memory>
 #include <vector>
 
 #include "batch.cuh"
@@ -95,8 +96,8 @@ struct Batch {
   int* chunk_off_f = nullptr;
   int total_chunks_f = 0;
   std::vector<CGroup> cgroups;  // stencil phases (half-site counts with the odd-even reduction)
-  std::vector<Group> groups;    // FP64 residual on the FP64 pipe, n-groups with an operator without digits
-  std::vector<DGroup> dgroups;  // ... through the digit operands
+  std::vector<Group> groups;    // FP64 residual on the FP64 pipe, the operators without digits
+  std::vector<DGroup> dgroups;  // ... through the digit operands, the others
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   long long launches = 0;
@@ -469,7 +470,7 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
     size_t maxN = 0;
     for (int i = 0; i < nops; ++i) maxN = std::max(maxN, (size_t)ops[i]->V * ops[i]->n);
     double2* tmp = nullptr;
-    if (cudaMalloc((void**)&tmp, 2 * maxN * sizeof(double2)) != cudaSuccess) {
+    if (device_malloc((void**)&tmp, 2 * maxN * sizeof(double2)) != cudaSuccess) {
       cudaGetLastError();
       set_error("coarse_solve_batched: setup allocation failed");
       return COARSE_ERR_OOM;
@@ -601,7 +602,7 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
   }
   B.total_chunks = chunk_off[ns];
   B.total_chunks_f = chunk_off_f[ns];
-  if (cudaMalloc((void**)&B.mem, bytes) != cudaSuccess) {
+  if (device_malloc((void**)&B.mem, bytes) != cudaSuccess) {
     cudaGetLastError();
     set_error("coarse_solve_batched: allocation of %zu bytes failed", bytes);
     return COARSE_ERR_OOM;
@@ -807,51 +808,52 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
     COARSE_CUDA(cudaMemcpyAsync(B.mem + o_mgrp, mgroup_tab.data(), sizeof(int) * mgroup_tab.size(),
                                 cudaMemcpyHostToDevice, s));
   }
-  // n-groups of the FP64 residual
+  // n-groups of the FP64 residual; the operators' digits are held until the batch has ended
+  std::vector<std::unique_ptr<DigUse>> uses;
+  for (int i = 0; i < nops; ++i) {
+    uses.push_back(std::make_unique<DigUse>(ops[i]->digits, dig_plan(ops[i]), s));
+    TRY(uses.back()->rc());
+  }
   std::vector<DigPass> dpasses[3];
   std::vector<int> dmaps[3];
   size_t dpass_at = 0, dmap_at = 0;
   {
     int* g0 = reinterpret_cast<int*>(B.mem + o_groups);
     for (int n : {16, 32, 48}) {
-      std::vector<int> idx, off(1, 0);
-      for (int q = 0; q < ns; ++q)
-        if (hs[q].n == n) {
-          idx.push_back(q);
-          off.push_back(off.back() + hs[q].V);
+      std::vector<int> idx, off(1, 0);  // solves on the FP64 pipe
+      std::vector<DigPass>& dp = dpasses[n / 16 - 1];
+      std::vector<int>& map = dmaps[n / 16 - 1];
+      int s0 = 0;
+      for (int i = 0; i < nops; s0 += nrhs[i], ++i) {
+        if (ops[i]->n != n) continue;
+        const size_t N = (size_t)ops[i]->V * n;
+        for (int c = 0; !uses[i]->dig() && c < nrhs[i]; ++c) {
+          idx.push_back(s0 + c);
+          off.push_back(off.back() + ops[i]->V);
         }
-      if (idx.empty()) continue;
-      bool digits = true;
-      for (int i = 0; i < nops; ++i) digits = digits && (ops[i]->n != n || ops[i]->dig);
-      if (digits) {
-        std::vector<DigPass>& dp = dpasses[n / 16 - 1];
-        std::vector<int>& map = dmaps[n / 16 - 1];
-        int s0 = 0;
-        for (int i = 0; i < nops; ++i) {
-          const size_t N = (size_t)ops[i]->V * n;
-          for (int c = 0; ops[i]->n == n && c < nrhs[i]; c += kDigCols) {
-            const BSolve& S = hs[s0 + c];
-            DigPass d{};
-            d.x = S.x64;
-            d.z = S.b64;
-            d.y = S.r64;
-            d.ldx = N;
-            d.cols = std::min(kDigCols, nrhs[i] - c);
-            d.ldy = d.cols > 1 ? (size_t)(hs[s0 + c + 1].r64 - S.r64) : 0;  // equal records of one operator's solves
-            d.dig = ops[i]->dig;
-            d.digscale = ops[i]->digscale;
-            d.digx = S.part64;
-            d.blocks = S.blk64;
-            d.nb = S.nb;
-            d.mu = S.mu;
-            d.V = S.V;
-            d.start = (int)map.size() * kDigMapSites;
-            d.q0 = s0 + c;
-            map.insert(map.end(), (S.V + kDigMapSites - 1) / kDigMapSites, (int)dp.size());
-            dp.push_back(d);
-          }
-          s0 += nrhs[i];
+        for (int c = 0; uses[i]->dig() && c < nrhs[i]; c += kDigCols) {
+          const BSolve& S = hs[s0 + c];
+          DigPass d{};
+          d.x = S.x64;
+          d.z = S.b64;
+          d.y = S.r64;
+          d.ldx = N;
+          d.cols = std::min(kDigCols, nrhs[i] - c);
+          d.ldy = d.cols > 1 ? (size_t)(hs[s0 + c + 1].r64 - S.r64) : 0;  // equal records of one operator's solves
+          d.dig = uses[i]->dig();
+          d.digscale = uses[i]->scale();
+          d.digx = S.part64;
+          d.blocks = S.blk64;
+          d.nb = S.nb;
+          d.mu = S.mu;
+          d.V = S.V;
+          d.start = (int)map.size() * kDigMapSites;
+          d.q0 = s0 + c;
+          map.insert(map.end(), (S.V + kDigMapSites - 1) / kDigMapSites, (int)dp.size());
+          dp.push_back(d);
         }
+      }
+      if (!dp.empty()) {
         DGroup g;
         g.n = n;
         g.sites = (int)map.size() * kDigMapSites;
@@ -864,8 +866,8 @@ extern "C" int coarse_solve_batched(coarse_op* const* ops, int nops, const void*
         dpass_at += dp.size();
         dmap_at += map.size();
         B.dgroups.push_back(g);
-        continue;
       }
+      if (idx.empty()) continue;
       Group g;
       g.n = n;
       g.count = (int)idx.size();

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/coarse.h"
+#include "dig_store.cuh"
 #include "smem_limit.cuh"
 
 namespace coarse {
@@ -102,9 +103,7 @@ struct coarse_op {
   double2* coef = nullptr;          // device constants: {-1, 1} for r = b - D x
   unsigned* counter = nullptr;      // last-block counter of the op-level reductions
   void* apply_scratch = nullptr;    // 5 * V * n complex128: pull partials and pushes of the stencil
-  void* dig = nullptr;              // FP64 blocks as digits (null: memory too short for a second copy)
-  double* digscale = nullptr;       // their scales
-  void* digx = nullptr;             // column operands of the digit stencil
+  coarse::DigStore* digits = nullptr;  // FP64 blocks as digits, where they are held
   int* apply_cnt = nullptr;         // V arrival counters of the stencil (zero between launches), then an error flag
   int device = 0;
 };
@@ -137,11 +136,9 @@ struct ApplyArgs {
   void* push;           // scratch [4][V][n] pushes to the forward neighbours
   int* cnt;             // [V] arrival counters, zero between launches
   int* err;             // raised (1) if a bounded wait of the TMA-staged kernel expired
-  const void* dig;      // FP64: the blocks as digits (digits.cuh), or null: the FP64 pipe
-  const double* digscale;  // their scales
-  void* digx;           // room for the column operands and row magnitudes (dig_work_bytes)
 };
 
+// The FP64 pipe for COARSE_PREC_FP64; launch_apply64 (digits.cuh) goes through the operator's digits.
 int launch_apply(int prec, int n, const ApplyArgs& a, cudaStream_t s);
 
 // Arguments of a plain y = D x launch on operator `op` with the blocks of precision `prec`.
@@ -163,9 +160,6 @@ inline ApplyArgs make_apply_args(const coarse_op* op, int prec, const void* x, v
   a.push = (char*)op->apply_scratch + (size_t)op->V * op->n * (prec == COARSE_PREC_FP64 ? 16 : 8);
   a.cnt = op->apply_cnt;
   a.err = op->apply_cnt + op->V;
-  a.dig = prec == COARSE_PREC_FP64 ? op->dig : nullptr;
-  a.digscale = op->digscale;
-  a.digx = op->digx;
   return a;
 }
 int launch_apply_mrhs_bf16(const coarse_op* op, const void* x, void* y, int nrhs, int adjoint, cudaStream_t s);

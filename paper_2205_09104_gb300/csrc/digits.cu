@@ -292,6 +292,7 @@ struct DigArgs {
   const float* xc;
   const double* xs;
   const float* xn;
+  void* work;  // push kernel: dig_rows_at
 };
 
 // One output tile's level sums [plane of the block][part of the column] -> this lane's (row, part) of the
@@ -670,9 +671,9 @@ struct DigRows {
   int* exp;
 };
 template <int N>
-__host__ __device__ __forceinline__ DigRows dig_rows_at(void* digx, int V) {
+__device__ __forceinline__ DigRows dig_rows_at(void* work, int V) {
   DigRows r;
-  r.have = reinterpret_cast<float*>(static_cast<char*>(digx) + dig_x_bytes(N, V, 1));
+  r.have = reinterpret_cast<float*>(static_cast<char*>(work) + dig_x_bytes(N, V, 1));
   r.exp = reinterpret_cast<int*>(r.have + (size_t)5 * V * N);
   return r;
 }
@@ -844,7 +845,7 @@ __global__ void __launch_bounds__(32 * kPW, N == 16 ? 5 : 4) k_push_digits(const
   }
 #pragma unroll
   for (int U = 0; U < NT; ++U) part[mu][2 * (16 * U + g + 8 * (t & 1)) + (t >> 1)] = pull[U];
-  const DigRows rows = dig_rows_at<N>(a.digx, V);
+  const DigRows rows = dig_rows_at<N>(dgt.work, V);
   const float need = needs[0], needn = needs[1 + mu];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -873,13 +874,13 @@ __global__ void __launch_bounds__(32 * kPW, N == 16 ? 5 : 4) k_push_digits(const
 // y_z = P_z + T_0[z-0] + .. + T_3[z-3] + i mu sigma3 x_z, then the epilogue; one thread per entry.  Rows whose
 // magnitudes do not meet their demand are summed on the FP64 pipe, four of a warp's at a time.
 template <int N>
-__global__ void __launch_bounds__(256, 3) k_push_finish(const __grid_constant__ ApplyArgs a) {
+__global__ void __launch_bounds__(256, 3) k_push_finish(const __grid_constant__ ApplyArgs a, void* work) {
   if (a.stop != nullptr && *a.stop) return;
   const size_t i = blockIdx.x * (size_t)256 + threadIdx.x;
   const bool in = i < (size_t)a.V * N;
   const int z = in ? (int)(i / N) : 0, e = (int)(i % N), lane = threadIdx.x & 31;
   const double2* T = static_cast<const double2*>(a.push);
-  const DigRows rows = dig_rows_at<N>(a.digx, a.V);
+  const DigRows rows = dig_rows_at<N>(work, a.V);
   double2 r = make_double2(0.0, 0.0), xs = r, zv = r;
   bool bad = false;
   if (in) {
@@ -936,6 +937,7 @@ __global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, kDigCols)) kb_resi
   d.xc = dx.xc;
   d.xs = dx.xs;
   d.xn = dx.xn;
+  d.work = nullptr;
   ApplyArgs a{};
   a.blocks = p.blocks;
   a.nb = p.nb;
@@ -977,7 +979,7 @@ int launch_dig_1(const ApplyArgs& a, const DigArgs& d, cudaStream_t s) {
     note_launch();
     COARSE_CUDA(cudaGetLastError());
     const size_t total = (size_t)a.V * N;
-    k_push_finish<N><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(a);
+    k_push_finish<N><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(a, d.work);
   } else {
     COARSE_CUDA(raise_smem_limit(site, (const void*)k_site_digits<N, 1>, ss));
     k_site_digits<N, 1><<<a.V, 32 * kDW, ss, s>>>(a, d, 1, 0);
@@ -988,11 +990,12 @@ int launch_dig_1(const ApplyArgs& a, const DigArgs& d, cudaStream_t s) {
 }
 
 template <int N>
-int launch_dig_n(const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {
+int launch_dig_n(const ApplyArgs& a, const DigUse& use, int ncol, long long ldc, cudaStream_t s) {
   DigArgs d;
-  d.dig = static_cast<const uint4*>(a.dig);
-  d.bscale = a.digscale;
-  const DigX x = dig_x_at<N>(a.digx, a.V, ncol);
+  d.dig = static_cast<const uint4*>(use.dig());
+  d.bscale = use.scale();
+  d.work = use.work();
+  const DigX x = dig_x_at<N>(d.work, a.V, ncol);
   d.xd = x.xd;
   d.xc = x.xc;
   d.xs = x.xs;
@@ -1028,6 +1031,25 @@ int launch_dig_blocks(const double2* blocks, int V, int n, void* dig, double* sc
   return COARSE_OK;
 }
 
+DigPlan dig_plan(const coarse_op* op) {
+  DigPlan p;
+  p.dig = dig_block_bytes(op->n, op->V);
+  p.scale = dig_scale_bytes(op->V);
+  p.work = dig_work_bytes(op->n, op->V, op->max_nrhs < kDigCols ? op->max_nrhs : kDigCols);
+  p.ctx = op;
+  p.pack = [](const void* ctx, void* dig, double* scale, cudaStream_t s) {
+    const coarse_op* o = static_cast<const coarse_op*>(ctx);
+    return launch_dig_blocks(static_cast<const double2*>(o->blk[COARSE_PREC_FP64].ptr), o->V, o->n, dig, scale, s);
+  };
+  return p;
+}
+
+int launch_apply64(const coarse_op* op, const ApplyArgs& a, cudaStream_t s) {
+  const DigUse d(op->digits, dig_plan(op), s);
+  if (d.rc() != COARSE_OK) return d.rc();
+  return d.dig() ? launch_apply_digits(op->n, a, d, 1, 0, s) : launch_apply(COARSE_PREC_FP64, op->n, a, s);
+}
+
 int launch_bresidual_digits(int n, const DigPass* passes, const int* map, int sites, const int* flags,
                             const double2* coef, cudaStream_t s) {
   if (sites <= 0) return COARSE_OK;
@@ -1046,15 +1068,15 @@ int launch_bresidual_digits(int n, const DigPass* passes, const int* map, int si
 // 759, n = 48 2191 / 1565.
 int dig_columns(int n, int V) { return n > 16 && dig_block_bytes(n, V) > (size_t(320) << 20) ? 1 : kDigCols; }
 
-int launch_apply_digits(int n, const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s) {
+int launch_apply_digits(int n, const ApplyArgs& a, const DigUse& d, int ncol, long long ldc, cudaStream_t s) {
   if (ncol < 1 || ncol > kDigCols) {
     set_error("digit stencil: %d columns in one pass", ncol);
     return COARSE_ERR_INVALID_ARG;
   }
   switch (n) {
-    case 16: return launch_dig_n<16>(a, ncol, ldc, s);
-    case 32: return launch_dig_n<32>(a, ncol, ldc, s);
-    case 48: return launch_dig_n<48>(a, ncol, ldc, s);
+    case 16: return launch_dig_n<16>(a, d, ncol, ldc, s);
+    case 32: return launch_dig_n<32>(a, d, ncol, ldc, s);
+    case 48: return launch_dig_n<48>(a, d, ncol, ldc, s);
   }
   set_error("coarse_apply: unsupported n = %d (nv must be 8, 16 or 24)", n);
   return COARSE_ERR_INVALID_ARG;

@@ -17,7 +17,7 @@ constexpr size_t kDigCorr = 32;
 __host__ __device__ inline size_t dig_x_bytes(int n, int V, int cols) {
   return (size_t)cols * V * (dig_x_halves(n) * 2 + kDigCorr * sizeof(float) + sizeof(double) + sizeof(float));
 }
-// Bytes of the work memory of a stencil of up to `cols` columns per pass (ApplyArgs::digx): the column operands, behind
+// Bytes of the work memory of a stencil of up to `cols` columns per pass: the column operands, behind
 // those of one column the push kernel's row magnitudes and exponents.
 inline size_t dig_work_bytes(int n, int V, int cols) {
   const size_t push = dig_x_bytes(n, V, 1) + (size_t)5 * V * (n * sizeof(float) + sizeof(int));
@@ -32,9 +32,13 @@ int launch_dig_blocks(const double2* blocks, int V, int n, void* dig, double* sc
 
 // Columns that one pass of a multi-column FP64 stencil should take (1 or kDigCols).
 int dig_columns(int n, int V);
-// y = D x (with a's epilogue) for ncol <= kDigCols columns x + c * ldc, y + c * ldc, through the digit
-// operands a.dig (must be set); a.digx holds room for ncol columns.
-int launch_apply_digits(int n, const ApplyArgs& a, int ncol, long long ldc, cudaStream_t s);
+// How the copy of `op` is built (up to `op->max_nrhs` columns a call).
+DigPlan dig_plan(const coarse_op* op);
+// y = D x (with a's epilogue) for ncol <= kDigCols columns x + c * ldc, y + c * ldc, through the operator's digits
+// (d.dig() must be set).
+int launch_apply_digits(int n, const ApplyArgs& a, const DigUse& d, int ncol, long long ldc, cudaStream_t s);
+// y = D x (with a's epilogue), one column, in FP64: through the operator's digits, or on the FP64 pipe.
+int launch_apply64(const coarse_op* op, const ApplyArgs& a, cudaStream_t s);
 
 // Batched FP64 residual: one pass = up to kDigCols columns of one operator.  Launches cover the passes' sites
 // padded to kDigMapSites each; map[i] is the pass of sites i * kDigMapSites ..

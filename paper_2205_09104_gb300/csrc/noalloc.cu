@@ -102,8 +102,7 @@ extern "C" int coarse_residual_noalloc(const coarse_op* op, const void* b, const
   a.push = p + N * sizeof(double2);
   a.cnt = cnt;
   a.err = cnt + op->V;
-  // the digit kernels need the operator's work memory for x; this call uses none but its own
-  a.dig = nullptr;
+  // the FP64 pipe: the digit kernels need the operator's work memory for x, this call uses none but its own
   rc = launch_apply(COARSE_PREC_FP64, op->n, a, s);
   if (rc != COARSE_OK) return rc;
   rc = launch_norm2(1, r, (int)N, norms, partial, counter, s);

@@ -941,7 +941,7 @@ int eo_prepare(coarse_op* op, double mu_eff, cudaStream_t s) {
   for (int p = 0; p < 3; ++p) {
     if (!op->blk[p].ptr || op->inv[sg][p].ptr) continue;
     op->inv[sg][p].bytes = nn * esz[p];
-    if (cudaMalloc(&op->inv[sg][p].ptr, op->inv[sg][p].bytes) != cudaSuccess) {
+    if (device_malloc(&op->inv[sg][p].ptr, op->inv[sg][p].bytes) != cudaSuccess) {
       cudaGetLastError();
       op->inv[sg][p].ptr = nullptr;
       set_error("odd-even: allocation of the block inverses failed");
@@ -1084,7 +1084,7 @@ int launch_eo_tuned(int prec, int n, const EoArgs& a, cudaStream_t s) {
     const size_t hv = (size_t)(a.V / 2) * n;
     auto run = [&](const TuneChoice& c) -> int {
       if (!scratch) {
-        if (cudaMalloc(&scratch, 2 * sizeof(VT) * hv) != cudaSuccess) {
+        if (device_malloc(&scratch, 2 * sizeof(VT) * hv) != cudaSuccess) {
           cudaGetLastError();
           scratch = nullptr;
           set_error("odd-even: autotuner scratch allocation failed");

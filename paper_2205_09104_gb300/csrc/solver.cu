@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "digits.cuh"
 #include "oddeven.cuh"
 #include "solver.cuh"
 #include "solver_state.cuh"
@@ -23,7 +24,7 @@ size_t csize(int v64) { return v64 ? sizeof(double2) : sizeof(float2); }
 template <class T>
 int dalloc(T** p, size_t count) {
   if (count == 0) count = 1;
-  cudaError_t e = cudaMalloc((void**)p, sizeof(T) * count);
+  cudaError_t e = device_malloc((void**)p, sizeof(T) * count);
   if (e != cudaSuccess) {
     cudaGetLastError();
     set_error("device allocation of %zu bytes failed: %s", sizeof(T) * count, cudaGetErrorString(e));
@@ -256,7 +257,7 @@ int Solver::apply(const void* x, void* y, int mode, void* accp, const double2* c
     a.mu = mu_eff;
     a.mode = mode;
     a.stop = stop;
-    return launch_apply(bprec, op->n, a, stream);
+    return bprec == COARSE_PREC_FP64 ? launch_apply64(op, a, stream) : launch_apply(bprec, op->n, a, stream);
   };
   ++matvecs;
   if (!time_apply) return launch();
@@ -659,7 +660,7 @@ int solve_column(coarse_op* op, Solver* s, const double2* b64, double2* x64, con
     a.coef = op->coef;  // {-1, +1}: r = -D x + b
     a.mu = mu_eff;
     a.mode = APPLY_AXPBY;
-    TRY(launch_apply(COARSE_PREC_FP64, op->n, a, stream));
+    TRY(launch_apply64(op, a, stream));
     return launch_norm2(1, r64, N, op->norms, op->red, op->counter, stream);
   };
 
@@ -697,7 +698,7 @@ int solve_column(coarse_op* op, Solver* s, const double2* b64, double2* x64, con
   float2 *eo_re = nullptr, *eo_ro = nullptr, *eo_to = nullptr, *eo_eo = nullptr;
   if (s->eo) {
     TRY(eo_prepare(op, mu_eff, stream));
-    if (!op->eo_scratch && cudaMalloc(&op->eo_scratch, sizeof(float2) * 3 * (size_t)N) != cudaSuccess) {
+    if (!op->eo_scratch && device_malloc(&op->eo_scratch, sizeof(float2) * 3 * (size_t)N) != cudaSuccess) {
       cudaGetLastError();
       op->eo_scratch = nullptr;
       set_error("odd-even: scratch allocation failed");

@@ -38,11 +38,12 @@ class CoarseOp:
 
     self_blocks: complex128 [V, n, n]; hop_blocks: complex128 [V, 8, n, n] (or [V, 4, n, n]
     with ``assume_gamma5``), both CUDA tensors in the canonical layout of include/coarse.h.
+    fp64_pipe: keep no digit copy of the blocks; FP64 stencils run on the FP64 pipe (half the memory, slower).
     """
 
     def __init__(self, self_blocks: torch.Tensor, hop_blocks: torch.Tensor, dims, nv: int, mu: float = 0.0,
                  precisions=(_abi.PREC_FP32, _abi.PREC_BF16), max_nrhs: int = 1, assume_gamma5: bool = False,
-                 stream=None):
+                 stream=None, fp64_pipe: bool = False):
         for t in (self_blocks, hop_blocks):
             if not (t.is_cuda and t.dtype == torch.complex128 and t.is_contiguous()):
                 raise ValueError("blocks must be contiguous complex128 CUDA tensors")
@@ -55,7 +56,7 @@ class CoarseOp:
         d = OpDesc()
         d.dims[:] = self.dims
         d.nv, d.mu, d.max_nrhs = self.nv, self.mu, max_nrhs
-        d.flags = _abi.COARSE_ASSUME_GAMMA5 if assume_gamma5 else 0
+        d.flags = (_abi.COARSE_ASSUME_GAMMA5 if assume_gamma5 else 0) | (_abi.COARSE_FP64_PIPE if fp64_pipe else 0)
         d.precisions = sum(1 << p for p in precisions) | 1
         h = ctypes.c_void_p()
         check(lib().coarse_op_create(ctypes.byref(d), _ptr(self_blocks), _ptr(hop_blocks), _stream(stream),
@@ -83,6 +84,13 @@ class CoarseOp:
             self.close()
         except Exception:
             pass
+
+    def fp64_path(self) -> int:
+        """How FP64 stencils of this operator run: FP64_UNDECIDED (none has), FP64_DIGITS, FP64_PIPE_ASKED
+        (``fp64_pipe=True``) or FP64_PIPE_MEMORY (no room for the digit copy of the blocks)."""
+        path = ctypes.c_int()
+        check(lib().coarse_op_fp64_path(self.handle, ctypes.byref(path)))
+        return path.value
 
     def update(self, self_blocks, hop_blocks, stream=None):
         check(lib().coarse_op_update(self.handle, _ptr(self_blocks), _ptr(hop_blocks), _stream(stream)))
