@@ -1068,7 +1068,9 @@ int launch_eo_variant(int variant, int n, const EoArgs& a, cudaStream_t s) {
 // site (candidate 0), one warp per site (candidate 1) and one CTA of 2 warps per site with the
 // direction loop rolled (candidates 2, 4) or unrolled (3, 5), the last two with the inverse block
 // and the epilogue vectors prefetched into shared memory, and (FP32 / BF16 blocks) the streamed
-// persistent layout (6) and the CTA of 8 warps (7); candidates run in plain mode into a scratch output.
+// persistent layout (6) and the CTA of 8 warps (7).  What is timed is a whole S apply on scratch vectors, both halves:
+// on 8^4 sites with n = 32 (FP32) the layouts 0, 1, 4 and 6 lie within a few per cent of each other in one half
+// alone, in varying order, while the S apply takes 57.7 / 61.5 / 57.9 / 58.2 us.
 template <class BT, class VT, class AC>
 int launch_eo_tuned(int prec, int n, const EoArgs& a, cudaStream_t s) {
   const int ni = n / 16 - 1, vb = std::min(tune_bucket(a.V), 31);
@@ -1084,22 +1086,32 @@ int launch_eo_tuned(int prec, int n, const EoArgs& a, cudaStream_t s) {
     const size_t hv = (size_t)(a.V / 2) * n;
     auto run = [&](const TuneChoice& c) -> int {
       if (!scratch) {
-        if (device_malloc(&scratch, 2 * sizeof(VT) * hv) != cudaSuccess) {
+        if (device_malloc(&scratch, 3 * sizeof(VT) * hv) != cudaSuccess) {
           cudaGetLastError();
           scratch = nullptr;
           set_error("odd-even: autotuner scratch allocation failed");
           return COARSE_ERR_OOM;
         }
-        COARSE_CUDA(cudaMemsetAsync(scratch, 0, 2 * sizeof(VT) * hv, s));
+        COARSE_CUDA(cudaMemsetAsync(scratch, 0, 3 * sizeof(VT) * hv, s));
       }
+      // an S apply: the odd half, then the even half on its result (launch_eo_schur)
+      VT* v = static_cast<VT*>(scratch);
       EoArgs t = a;
-      // candidates are always timed with the hops (a pass without them is not representative)
-      if (!t.v) t.v = static_cast<VT*>(scratch) + hv;
       t.mode = APPLY_PLAIN;
-      t.y = scratch;
+      t.z = nullptr;
       t.acc = nullptr;
       t.coef = nullptr;
       t.stop = nullptr;
+      t.out_par = 1;
+      t.v = v;
+      t.base = nullptr;
+      t.y = v + hv;
+      const int rc = launch_eo_variant<BT, VT, AC>(c.a, n, t, s);
+      if (rc != COARSE_OK) return rc;
+      t.out_par = 0;
+      t.v = v + hv;
+      t.base = v;
+      t.y = v + 2 * hv;
       return launch_eo_variant<BT, VT, AC>(c.a, n, t, s);
     };
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
