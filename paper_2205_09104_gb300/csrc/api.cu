@@ -186,7 +186,10 @@ int apply_impl(const coarse_op* op, const void* x, void* y, int nrhs, int precis
   if (nrhs > 1 && precision == COARSE_PREC_BF16) return launch_apply_mrhs_bf16(op, x, y, nrhs, adjoint, s);
   const size_t esz = precision == COARSE_PREC_FP64 ? sizeof(double2) : sizeof(float2);
   const size_t col = esz * (size_t)op->V * op->n;
-  // several FP32 columns share each block: up to kMcCols in passes of nearly equal size (16-byte reads of the columns)
+  // several FP32 columns share each block: up to kMcCols in passes of nearly equal size (16-byte reads of the columns).
+  // Also two columns on large lattices, where nine blocks per site are read instead of five per column (us, together /
+  // one by one, two and three columns): 16^4 n = 48 1110 / 1915, 1209 / 2872; n = 16 185 / 302, 213 / 451; 8^4 n = 32
+  // 39 / 82, 46 / 122
   const bool mc = precision == COARSE_PREC_FP32 && nrhs > 1 && ((uintptr_t)x & 15) == 0;
   const int passes = (nrhs + kMcCols - 1) / kMcCols;
   if (precision == COARSE_PREC_FP64 && nrhs > 1) return apply64_columns(op, x, y, nrhs, adjoint, s);

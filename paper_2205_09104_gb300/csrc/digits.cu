@@ -281,9 +281,9 @@ template <int N> constexpr int dig_row() { return 2 * N + 16; }
 template <int N> constexpr int dig_part() { return 15 * dig_row<N>(); }
 template <int N> constexpr int dig_slab() { return 2 * dig_part<N>() + 2 * N; }
 
-// CTAs per SM to keep registers for: as many as measured faster (two columns, 8^4: n = 16 89 us with three
-// against 135 us with one, n = 32 174 us with two against 226 us, n = 48 404 us with one against 437 us)
-__host__ __device__ constexpr int dig_min_blocks(int N, int C) { return N == 16 ? 3 : (N == 48 && C > 1 ? 1 : 2); }
+// CTAs per SM to keep registers for, as many as measured faster with two columns: n = 16 three (8^4: 93 us against 95
+// with two), n = 32 and 48 two (n = 48, 8^4: 357 us, in 96 registers with spills, against 449 with one CTA).
+__host__ __device__ constexpr int dig_min_blocks(int N) { return N == 16 ? 3 : 2; }
 
 struct DigArgs {
   const uint4* dig;
@@ -648,16 +648,17 @@ __device__ __forceinline__ void dig_site(const ApplyArgs& a, const DigArgs& dgt,
 
 // One CTA per site: two columns, and small lattices.
 template <int N, int C>
-__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, C)) k_site_digits(
+__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N)) k_site_digits(
     const __grid_constant__ ApplyArgs a, const __grid_constant__ DigArgs dgt, int ncol, long long ldc) {
   if (a.stop != nullptr && *a.stop) return;
   dig_site<N, C>(a, dgt, blockIdx.x, ncol, ldc, ldc, ldc);
 }
 
 // ------------------------------------------------------------------ one column: every block once
-// The pull kernel reads a hop block twice, as a forward hop and transposed for the site in front: nine blocks per
-// site through L2, of which about a quarter hit (16^4, n = 48: 3.3 ms at 4.9 TB/s of DRAM).  Here the four warps of site x multiply each tile of F_{x,mu} both ways while it is in registers: forward with
-// the digits of x + mu into the site's own sum, transposed with the site's digits into the push for x + mu,
+// The pull kernel reads a hop block twice, as a forward hop and transposed for the site in front: nine blocks per site
+// through L2, of which about a quarter hit (16^4, n = 48: 3.4 ms).  Here the four warps of site x multiply each tile of
+// F_{x,mu} both ways while it is in registers: forward with the digits of x + mu into the site's own sum, transposed
+// with the site's digits into the push for x + mu,
 //   P_x = A_x v_x + sum_mu F_{x,mu} v_{x+mu},   T_mu[x] = sigma3 F_{x,mu}^H sigma3 v_x,
 // and k_push_finish adds y_z = P_z + sum_mu T_mu[z - mu], the mass term and the epilogue.  The self block's tile
 // rows are dealt to the warps.  The rows' magnitudes less their demands travel with P and T, and the finish
@@ -921,7 +922,7 @@ __global__ void __launch_bounds__(256, 3) k_push_finish(const __grid_constant__ 
 
 // Batched FP64 residual r = b - D x of every pass with an unfinished column (coef: {-1, +1}).
 template <int N>
-__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N, kDigCols)) kb_residual_digits(const DigPass* __restrict__ passes,
+__global__ void __launch_bounds__(32 * kDW, dig_min_blocks(N)) kb_residual_digits(const DigPass* __restrict__ passes,
                                                                   const int* __restrict__ map,
                                                                   const int* __restrict__ flags,
                                                                   const double2* coef) {
@@ -965,9 +966,9 @@ int launch_dig_2(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, 
 }
 
 // One column.  From kPushSites sites on every block once (push kernel and its finish); below, where the lattice
-// does not fill the chip, one launch of the pull kernel.  Both sides, us: 4^4 n = 16 15 / 19, n = 48 26 / 29;
-// 6^4 n = 16 28 / 27, n = 32 51 / 48, n = 48 74 / 74; 8^4 n = 32 132 / 95, n = 48 218 / 167; 16^4 n = 48
-// 3330 / 2240 (1800 at the copy bandwidth).
+// does not fill the chip, one launch of the pull kernel.  Both sides, us, pull / push: 6^4 n = 16 23 / 25, n = 32 49 / 43,
+// n = 48 77 / 72; 8^4 n = 16 56 / 52, n = 32 123 / 97, n = 48 215 / 178; 16^4 n = 16 797 / 598, n = 32 1753 / 1237,
+// n = 48 3351 / 2485 (1800 at the copy bandwidth).
 constexpr int kPushSites = 1024;
 template <int N>
 int launch_dig_1(const ApplyArgs& a, const DigArgs& d, cudaStream_t s) {
@@ -1062,11 +1063,15 @@ int launch_bresidual_digits(int n, const DigPass* passes, const int* map, int si
   return COARSE_ERR_INVALID_ARG;
 }
 
-// The pair kernel reads a hop block twice, the second time from L2 while the lattice is small; the push kernel
-// reads it once per column.  Two columns, us, pair / column by column: 6^4 n = 32 82 / 101, n = 48 152 / 165;
-// 8^4 n = 16 92 / 114, n = 32 (336 MB of digits) 205 / 198, n = 48 452 / 354; 12^4 n = 16 406 / 415, n = 32 954 /
-// 759, n = 48 2191 / 1565.
-int dig_columns(int n, int V) { return n > 16 && dig_block_bytes(n, V) > (size_t(320) << 20) ? 1 : kDigCols; }
+// The pair kernel reads a hop block twice, the second time from L2 while the lattice is small, and pays the block
+// operand's byte permutations once for two columns; the push kernel reads a block once per column.  Two columns, us,
+// pair / column by column, by sites:
+//           1296        2304        4096        6144        9216        20736
+//   n = 16  33 / 50     53 / 66     93 / 105    136 / 142   198 / 197   437 / 412
+//   n = 32  64 / 85     103 / 123   172 / 193   249 / 271   378 / 389   862 / 815
+//   n = 48  118 / 143   198 / 215   357 / 357   533 / 514   798 / 747   1803 / 1624
+// (The batched residual takes pairs at every size: its passes share one launch.)
+int dig_columns(int n, int V) { return V >= (n == 16 ? 8192 : n == 32 ? 12288 : 4096) ? 1 : kDigCols; }
 
 int launch_apply_digits(int n, const ApplyArgs& a, const DigUse& d, int ncol, long long ldc, cudaStream_t s) {
   if (ncol < 1 || ncol > kDigCols) {
