@@ -72,6 +72,13 @@ bool capturing(cudaStream_t s) {
   return true;
 }
 
+// Allocations of this thread do not disturb a capture of another stream (they are not part of it).
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Gives the copies of the current device back that nothing uses; false if there was none.
 bool reclaim() {
   int dev = 0;
@@ -144,6 +151,7 @@ DigUse::DigUse(DigStore* st, const DigPlan& plan, cudaStream_t s) {
   const bool cap = capturing(s);
   if (!st->dig) {
     if (cap) return;  // nothing can be allocated
+    const RelaxedCapture relaxed;
     st->bytes = plan.dig + plan.scale + plan.work;
     if (!reserve(st->device, st->bytes)) {
       st->refused = true;

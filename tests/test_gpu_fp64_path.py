@@ -130,3 +130,29 @@ def test_batch_of_both_kinds(pipes):
             r = B[q] - ocoarse.apply(s, h, dims, x[q].cpu().numpy(), 0.01)
             assert np.linalg.norm(r) <= 1.001e-10 * np.linalg.norm(B[q])
         op.close()
+
+
+def test_first_use_while_another_stream_is_captured():
+    """The copy is built on one stream in the middle of the capture of another."""
+    dims, nv = (2, 3, 2, 2), 8
+    s, f = blocks(dims, nv, 131)
+    x = columns(1, s.shape[0] * 2 * nv, 132)[0]
+    xd = torch.from_numpy(x).cuda()
+    dev = operator(s, f, dims, nv, 0.0, 1, False)
+    side = torch.cuda.Stream()
+    y, a = torch.empty_like(xd), torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        a += 1
+        dev.apply(xd, precision=0, stream=side, out=y)
+        a += 1
+    side.synchronize()
+    assert dev.fp64_path() == DIGITS
+    g.replay()
+    torch.cuda.synchronize()
+    assert (a == 2).all()
+    h = canonical(f, dims)
+    assert_entrywise(y.cpu().numpy(), ocoarse.apply(s, h, dims, x, 0.0), stencil_factor(0, 2 * nv) * abs_apply(s, h, dims, x),
+                     "built beside a capture")
+    dev.close()
