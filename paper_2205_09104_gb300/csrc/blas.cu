@@ -666,8 +666,9 @@ __global__ void __launch_bounds__(32 * kW) kb_norm64(const BSolve* S, int nsolve
 }  // namespace
 
 namespace {
-// Elements per lane: at least 128 CTAs from N = 32768 on, few enough partials for the last CTA.  The passes are
-// bound by L2 latency at these sizes, so more CTAs with fewer elements each come first.
+// Elements per lane (a CTA covers 256 of each): up to 128 CTAs for N <= 2^15, 65 to 128 for N <= 2^16, 65 to 256 for
+// N <= 2^18, 129 to 512 for N <= 2^20, more above; few enough partials for the last CTA.  The passes are bound by L2
+// latency at these sizes, so more CTAs with fewer elements each come first.
 int chunk_elems(int N) {
   return N <= (1 << 15) ? 1 : (N <= (1 << 16) ? 2 : (N <= (1 << 18) ? 4 : (N <= (1 << 20) ? 8 : 16)));
 }

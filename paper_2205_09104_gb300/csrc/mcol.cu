@@ -1,5 +1,6 @@
-// Multi-column stencil and half apply on the FP32 pipe: the columns that share an operator are
-// multiplied together, so that a block is read once for all of them instead of once per column.
+// Multi-column stencil and half apply: the columns that share an operator are multiplied together, so that a block is
+// read once for all of them instead of once per column.  The FP32 blocks' kernels and the full BF16 stencil run on the
+// FP32 pipe (below), the half apply with BF16 blocks on the tensor cores (kb_eo_mma).
 //
 // With R columns the block traffic per column falls by R and the FP32 rate bounds the product from about
 // four columns on (72 n^2 flops per site and column against 40 n^2 bytes of FP32 or 20 n^2 bytes of BF16
@@ -94,7 +95,8 @@ template <int N> struct Piece<N, cbf16> {
 template <int N, class BT, bool ADD>
 __device__ __forceinline__ void mul_rows(const Piece<N, BT>& p, const float2* tab, float* out, int r0, int c0, int cs,
                                          int R, bool flip, int lane) {
-  // sigma3 of the operand: the second chirality's columns come first, then the sums change sign once
+  // sigma3 of the operand: the second chirality's columns come first, then the sums change sign once; where a lane's
+  // columns do not divide so, the entries change sign
   constexpr bool kFlips = sizeof(BT) == 8;  // columns of entry q >= N/2 for every lane or for none
   constexpr int Q = N / 4;
   const int g = lane >> 2, t = lane & 3;
@@ -120,7 +122,8 @@ __device__ __forceinline__ void mul_rows(const Piece<N, BT>& p, const float2* ta
           F1[h] = make_float2(-F1[h].x, -F1[h].y);
           F2[h] = make_float2(-F2[h].x, -F2[h].y);
         }
-      const float4 ww = *reinterpret_cast<const float4*>(w + Piece<N, BT>::col(q, t));
+      float4 ww = *reinterpret_cast<const float4*>(w + Piece<N, BT>::col(q, t));
+      if (!kFlips && flip && Piece<N, BT>::col(q, t) >= N / 2) ww = make_float4(-ww.x, -ww.y, -ww.z, -ww.w);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         F1[h] = __ffma2_rn(e[h][q], make_float2(ww.x, ww.x), F1[h]);
@@ -423,7 +426,8 @@ template <int N> constexpr size_t mma_smem(int R) {
   return (size_t)kMW * (((R + 3) / 4) * split_tile<N>() + (size_t)R * N * sizeof(float2));
 }
 
-// (v0, v1) = h + m + l exactly, each part a BF16 pair
+// (v0, v1) = h + m + l exactly, each part a BF16 pair.  From the largest BF16 number on (3.39e38) h overflows and the
+// other parts are NaN, as for infinities: the cycle reports either as non-finite.
 __device__ __forceinline__ void split3(float v0, float v1, uint32_t (&o)[3]) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) {

@@ -1,4 +1,4 @@
-// Multi-column stencil and half apply on the FP32 pipe (mcol.cu).
+// Multi-column stencil and half apply (mcol.cu).
 #pragma once
 
 #include "batch.cuh"

@@ -60,25 +60,18 @@ void Solver::clear_graphs() {
   cycles_done = 0;
 }
 
-// Steps j0 .. j0+cnt-1 of the current cycle: eager launches for the solver's first cycle and
+// Step j of the current cycle: eager launches for the solver's first cycle and
 // for solves that time their stencil launches (COARSE_TIME_APPLY: per-launch events), otherwise a
-// CUDA graph per (j0, cnt, kc, recycle parity, chain precision, degree) captured once, replayed.
-int Solver::run_chunk(int j0, int cnt, int kc, void* const* tab) {
+// CUDA graph per (j, kc, recycle parity, chain precision, degree) captured once, replayed.
+int Solver::run_step(int j, int kc, void* const* tab) {
   auto issue = [&]() -> int {
-    for (int j = j0; j < j0 + cnt; ++j) {
-      cur_tag = j;
-      if (p1_active) {
-        TRY(p1_step(j, kc, tab));
-      } else {
-        TRY(opA(V[j], V[j + 1], &st->stop));
-        TRY(arnoldi_step(j, kc, tab));
-      }
-    }
-    return COARSE_OK;
+    cur_tag = j;
+    if (p1_active) return p1_step(j, kc, tab);
+    TRY(opA(V[j], V[j + 1], &st->stop));
+    return arnoldi_step(j, kc, tab);
   };
   if (cycles_done < 1 || time_apply) return issue();
-  const unsigned long long key = (unsigned long long)j0 | ((unsigned long long)cnt << 8) |
-                                 ((unsigned long long)kc << 16) | ((unsigned long long)par << 24) |
+  const unsigned long long key = (unsigned long long)j | ((unsigned long long)kc << 16) | ((unsigned long long)par << 24) |
                                  ((unsigned long long)poly_prec << 26) | ((unsigned long long)d << 28) |
                                  ((unsigned long long)(p1_active ? 1 : 0) << 36);
   auto it = graphs.find(key);
@@ -508,7 +501,7 @@ int Solver::inner(double target_abs, int max_cycles, int m, int kdef, int ulimit
     int launched = 0;
     for (int j = 0; j < steps; ++j) {
       stop_host[j] = 0;
-      TRY(run_chunk(j, 1, kc, tab));
+      TRY(run_step(j, kc, tab));
       ++launched;
       COARSE_CUDA(cudaEventRecord(chunk_ev[j & 1], stream));
       if (j > 0) {

@@ -102,7 +102,7 @@ struct Solver {
   // (N = V n / 2); eo_t is the odd-site scratch of its half applies
   int eo = 0;
   void* eo_t = nullptr;
-  // Arnoldi-step chunks captured as CUDA graphs (after the solver's first eager cycle, so that
+  // Arnoldi steps captured as CUDA graphs (after the solver's first eager cycle, so that
   // every autotuner decision is made), replayed for every later cycle with the same shape
   struct ChunkGraph {
     cudaGraphExec_t exec = nullptr;
@@ -114,7 +114,7 @@ struct Solver {
   int cycles_done = 0;
   cudaStream_t cap_stream = nullptr;
   void clear_graphs();
-  int run_chunk(int j0, int cnt, int kc, void* const* tab);
+  int run_step(int j, int kc, void* const* tab);
   void harvest(int steps_done);     // after a stream sync: add the elapsed time of the applies that ran
 
   ~Solver();
