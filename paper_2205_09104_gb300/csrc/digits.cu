@@ -745,7 +745,14 @@ __global__ void __launch_bounds__(32 * kPW, N == 16 ? 5 : 4) k_push_digits(const
   dig_table<N>(nbr, dgt.xd + (size_t)src * dig_x_halves(N), lane);
   if (mu == 0) dig_zero_rows<N, 1>(own, lane);
   dig_zero_rows<N, 1>(nbr, lane);
-  // the warp's product scales (forward hop, push, self block) and demands wait in shared memory: registers are short
+  float cf[4], cb[4];
+  dig_corr(dgt.xc + (size_t)src * kDigCorr, adj, cf, lane);
+  dig_corr(dgt.xc + (size_t)site * kDigCorr, !adj, cb, lane);
+  asm volatile("cp.async.commit_group;" ::: "memory");  // the tables, then the first two tiles
+  fetch(0);
+  fetch(1);
+  // the warp's product scales (forward hop, push, self block) and demands wait in shared memory: registers are short.
+  // Behind the fetches, which would otherwise start one latency later (16^4, n = 48: 2484 against 2464 us)
   if (lane == 0) {
     const double bh = __ldg(dgt.bscale + (size_t)site * 5 + 1 + mu), b0 = __ldg(dgt.bscale + (size_t)site * 5);
     const double x0 = __ldg(dgt.xs + site), xn = __ldg(dgt.xs + src);
@@ -755,12 +762,6 @@ __global__ void __launch_bounds__(32 * kPW, N == 16 ? 5 : 4) k_push_digits(const
     needs[1 + mu] = __ldg(dgt.xn + src);
     if (mu == 0) needs[0] = __ldg(dgt.xn + site);
   }
-  float cf[4], cb[4];
-  dig_corr(dgt.xc + (size_t)src * kDigCorr, adj, cf, lane);
-  dig_corr(dgt.xc + (size_t)site * kDigCorr, !adj, cb, lane);
-  asm volatile("cp.async.commit_group;" ::: "memory");  // the tables, then the first two tiles
-  fetch(0);
-  fetch(1);
   asm volatile("cp.async.wait_group 2;" ::: "memory");
   __syncthreads();
   double2* P = static_cast<double2*>(a.part) + (size_t)site * N;
@@ -968,7 +969,7 @@ int launch_dig_2(const ApplyArgs& a, const DigArgs& d, int ncol, long long ldc, 
 // One column.  From kPushSites sites on every block once (push kernel and its finish); below, where the lattice
 // does not fill the chip, one launch of the pull kernel.  Both sides, us, pull / push: 6^4 n = 16 23 / 25, n = 32 49 / 43,
 // n = 48 77 / 72; 8^4 n = 16 56 / 52, n = 32 123 / 97, n = 48 215 / 178; 16^4 n = 16 797 / 598, n = 32 1753 / 1237,
-// n = 48 3351 / 2485 (1800 at the copy bandwidth).
+// n = 48 3351 / 2465 (1800 at the copy bandwidth).
 constexpr int kPushSites = 1024;
 template <int N>
 int launch_dig_1(const ApplyArgs& a, const DigArgs& d, cudaStream_t s) {
